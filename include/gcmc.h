@@ -328,22 +328,21 @@ gcmc_status gcmc_get_geometry(gcmc_ctx *ctx, gcmc_geometry *out);
 gcmc_status gcmc_kernel_launches(gcmc_ctx *ctx, int64_t *out);
 
 /* Diagnostics of the last gcmc_run_moves (host out, either may be NULL):
- * refetched = moves whose prefetched neighbour data or particle record was
- * invalidated by the previous move and loaded again; refined = trials whose
+ * refetched = moves evaluated more than once (a move committed after the
+ * evaluation began changed what it read); refined = trials whose
  * FP32 decision fell inside the error band and were decided in FP64.
  * Errors: INVALID_ARG. */
 gcmc_status gcmc_chain_counters(gcmc_ctx *ctx, int64_t *refetched, int64_t *refined);
 
 /* Where the chain kernel's time went in the last gcmc_run_moves (or batch
- * run) of this context, in SM clock cycles summed over the run (host, 12
- * doubles): [0] the committer waiting for evaluations, [1] checking their
- * validity, [2] deciding (partial sums, Metropolis test, FP64 refinement),
- * [3] applying accepted moves, [4] the committer's whole loop; [5] the team
- * leaders waiting for an eligible move and [6] the teams evaluating (summed
- * over teams), [7] evaluations; [8] .. [10] the parts of [1]: the count
- * epoch, the logged moves, the particle pick; [11] booking a decided move.
- * Zeros for the microcell chain, and for a run without the counters
- * (gcmc_set_chain_profile).
+ * run) of this context, in SM clock cycles summed over the moves (host, 12
+ * doubles): [0] evaluated moves waiting for their turn, [1] the checks at the
+ * turn, [2] the decision, [3] applying accepted moves, [4] all of it from the
+ * end of the evaluation to the turn passed on; [5] waiting for room in the
+ * book; [6] evaluating, [7] evaluations (counted in every run); [8] 0; [9],
+ * [10] the parts of [1]: the logged moves, the particle pick; [11] passing the
+ * turn on and booking the move.  Zeros for the microcell chain, and (but for
+ * [7]) for a run without the counters (gcmc_set_chain_profile).
  * Errors: INVALID_ARG. */
 gcmc_status gcmc_chain_profile(gcmc_ctx *ctx, double *cycles);
 
@@ -354,21 +353,16 @@ gcmc_status gcmc_chain_profile(gcmc_ctx *ctx, double *cycles);
  * Errors: INVALID_ARG (NULL, on not 0 or 1). */
 gcmc_status gcmc_set_chain_profile(gcmc_ctx *ctx, int32_t on);
 
-/* Team shape of the chain kernel (how its warps split the evaluation of
- * upcoming moves; warps per team, teams, look-ahead L -- a move is
- * evaluated once fewer than L moves separate it from the last committed
- * one: 0 = (6, 2, 4), 1 = (7, 2, 4), 2 = (4, 3, 6), 3 = (3, 4, 8)):
- * 0 .. GCMC_CHAIN_CONFIGS-1, or -1 to time every shape
+/* Moves in flight of the chain kernel (each evaluated by one warp ahead of its
+ * turn): 0 = 8, 1 = 5, 2 = 11, 3 = 15 (fewer in a box whose cell counters leave
+ * less room on chip); 0 .. GCMC_CHAIN_CONFIGS-1, or -1 to time every choice
  * during the next gcmc_run_moves (after a first quarter of its moves under
- * shape 0) and keep the fastest.  Every shape takes the same moves and
- * decisions and reaches the same configuration.  How a trial's pair terms
- * are split among warps depends on the shape and, under speculation, on
- * which counts an evaluation read, so dU and the running energy may differ
- * between runs in their last bits (within the precision's tolerance).
+ * choice 0) and keep the fastest.  Every choice takes the same moves and
+ * decisions and reaches the same configuration.
  * Errors: INVALID_ARG. */
 #define GCMC_CHAIN_CONFIGS 4
 gcmc_status gcmc_set_chain_config(gcmc_ctx *ctx, int32_t config);
-/* The current team shape (host int32; -1 until the tuner has run).
+/* The current choice (host int32; -1 until the tuner has run).
  * Errors: INVALID_ARG (NULL). */
 gcmc_status gcmc_get_chain_config(gcmc_ctx *ctx, int32_t *config);
 

@@ -3,43 +3,47 @@
 // upcoming moves that the paper lists as future work (Sec. 5: run multiple
 // moves concurrently), here inside one CTA.
 //
-// One CTA owns one chain.  Its warps have three roles:
+// One CTA owns one chain.  Its warps have two roles:
 //
-//  * evaluator teams (NTEAM teams of G warps, placed off the committer's SM
-//    sub-partition first): team k evaluates moves k, k + NTEAM, ..., each as
-//    soon as fewer than LOOK moves separate it from the committer.  An
-//    evaluation is speculative: it reads the configuration as it stands when
-//    it starts (after `c0` committed moves; the particle pick uses the counts
-//    predicted at the move's turn unless it is the same for every count the
-//    pending moves can leave) and produces the trial, its energy
-//    change dU over the 27 neighbour cells (Algorithms 6 and 7; the union of
-//    both neighbourhoods for a displacement into an adjacent cell), the error
-//    scale uabs and the slots the update will need.  The team's warps split
-//    the items of the work cells evenly, by counts read in one count epoch
-//    (a sequence lock around count changes), and leave their sums in the
-//    move's slot; the committer adds them in a fixed order;
-//  * the committer (warp 0) takes the moves strictly in order.  A move is
-//    valid when its warps read one count epoch and no later commit put,
-//    removed or moved a particle within rc of the trial, touched its old
-//    cell or its record, or changed the particle the counts pick; otherwise
-//    the team evaluates it again.  The committer then takes the Metropolis
-//    decision (Eqs. 3-5, textbook sign of mu) in FP32 with an explicit error
-//    band -- a trial inside the band is recomputed entirely in FP64 -- and
-//    applies an accepted move (Sec. 3.2.5: swap-with-last removal, append,
-//    species index refill).  Every decision is therefore the one the
+//  * W movers: mover k owns the moves k, k + W, k + 2 W, ...  It evaluates a
+//    move alone and ahead of its turn: it reads the configuration as it
+//    stands when it starts (after c0 committed moves; the particle pick uses
+//    the counts predicted at the move's turn) and produces the trial, its
+//    energy change dU over the 27 neighbour cells (Algorithms 6 and 7; the
+//    union of both neighbourhoods for a displacement into an adjacent cell),
+//    the error scale uabs, and the Metropolis decision (Eqs. 3-5, textbook
+//    sign of mu) for each particle count its turn can meet.  Then it waits
+//    for its turn, checking each move that is committed meanwhile: one that
+//    put, removed or moved a particle within rc of the trial, touched its
+//    old cell or its record, or one that changes the particle the counts
+//    pick, makes it evaluate again (at once, before its turn).  At its turn
+//    the mover takes the decision for the actual count, applies an accepted
+//    move (Sec. 3.2.5: swap-with-last removal, append, species index refill)
+//    and passes the turn on.  A decision inside the FP32 error band is taken
+//    on a trial recomputed in FP64.  Every decision is therefore the one the
 //    sequential chain takes;
-//  * the keeper (warp 4) keeps the FP64 running energy, the averages, the
-//    counters and the trace, and refills the ring of Philox4x32-10 words.
+//  * the keeper (the last warp) keeps the FP64 running energy, the averages,
+//    the counters and the trace.
 //
-// A profiled launch (PROF) also counts SM cycles per role; the clock reads
-// are compiled out of the launches that do not ask for them.
+// What bounds it: the turn passes through every move, so a chain cannot run
+// faster than one hand-over per move (a poll of shared memory, the checks, the
+// stores of an accepted move and a fence; 700-1,800 cycles, the more the more
+// moves are accepted), and it runs at (evaluation + hand-over) / W when that
+// is longer (an evaluation takes 7,000-16,000 cycles: dependent shared-memory,
+// shuffle and L2 latencies, 1,500-2,500 warp instructions).  One warp per
+// move leaves the set-up (trial, cells, sums) unreplicated, and W evaluations
+// in flight hide its latency.  Measured against two teams of six warps that
+// evaluated a move together and a separate committing warp: 10^4 moves of
+// 2,048 particles in FP64 23.0 -> 8.5 ms, 2*10^4 of 131,072 in FP32 29.9 ->
+// 15.9 ms, the 64-chain isotherm step 223 -> 130 ms.
 //
-// Warps hand work to each other through shared-memory rings and counters
-// with block-scope fences; every wait is bounded and sets a timeout status
-// instead of hanging.  Cell counters live in shared memory (uint16) for the
-// whole launch; particle data stays in the padded cell-major layout in L2.
+// Movers hand the turn on through shared memory with block-scope fences;
+// every wait is bounded and sets a timeout status instead of hanging.  Cell
+// counters live in shared memory (uint16) for the whole launch; particle data
+// stays in the padded cell-major layout in L1/L2.
 //
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -60,20 +64,13 @@ struct ChainOut {
     double sum_n;
     long long n[kMaxSpecies];
     int status;
-    int pad;                // which waits gave up (1 leader, 2 committer, 4 keeper)
-    long long reevaluated;  // moves evaluated again by the committer
+    int pad;                // which waits gave up (1 room in the book, 2 the turn, 4 keeper)
+    long long reevaluated;  // moves evaluated more than once
     long long refines;      // trials decided in FP64 after the FP32 band test
     double virial;          // running virial after the last move (virial runs)
     double sum_virial;      // sum over the moves of the running virial
     unsigned long long t0, t1;  // global timer (ns) when the chain's CTA started and finished
-    // SM clock cycles summed over the moves: the committer waiting for
-    // evaluations, checking their validity, deciding (partial sums,
-    // Metropolis test, FP64 refinement), applying accepted moves, and its
-    // whole loop; the team leaders waiting for an eligible move and the teams
-    // evaluating (summed over teams and evaluations); evaluations
-    // then the validity check's parts: the count epoch, the logged moves,
-    // the particle pick; and the booking of a decided move
-    unsigned long long prof[12];
+    unsigned long long prof[12];  // SM clock cycles by role (gcmc_chain_profile)
 };
 
 struct ChainArgs {
@@ -81,6 +78,7 @@ struct ChainArgs {
     uint64_t first;
     int n_moves;
     uint32_t chain;
+    int movers;  // W
     int T;
     int ncell;
     int cap;
@@ -88,7 +86,7 @@ struct ChainArgs {
     int S;
     unsigned long long R2;
     int rcg;  // smallest integer with rcg^2 >= R2 (per-axis pre-filter)
-    float r2lo, r2hi;  // FP32 squared distances clearly inside / outside the cutoff
+    float r2hi;  // FP32 squared distances above it are outside the cutoff
     unsigned long long thr_disp, thr_ins;
     uint32_t span;  // 2 D + 1 grid steps
     int D;          // displacement half-width in grid steps
@@ -97,7 +95,7 @@ struct ChainArgs {
     double tol;  // relative tolerance that defines "near the threshold"
     float beta_f, tol_f;  // beta and tol in FP32 (the FP32 Metropolis test)
     unsigned long long wait_ns;  // limit of every wait (kWaitNs unless a test shortens it)
-    int stall_at;  // diagnostic: the committer waits on a flag nothing sets at this move (-1 none)
+    int stall_at;  // diagnostic: the mover waits on a flag nothing sets at this move (-1 none)
     int virial;  // also keep the running virial sum_{i<j} r U'(r)
     float lnzv_f[kMaxSpecies];
     FieldF ff;
@@ -111,29 +109,27 @@ struct ChainArgs {
     ChainOut *out;
 };
 
-constexpr int kRS = 32;       // move slots in flight (logs and book entries too)
-constexpr int kRW = 128;      // words ring
-constexpr int kFill = 32;     // words filled per keeper round
+constexpr int kChainWarps = 16;              // movers and the keeper
+constexpr int kMaxMovers = kChainWarps - 1;
+constexpr int kRS = 32;                      // log, book and outlook rings (at least 2 kMaxMovers)
+constexpr int kWords = 16;                   // moves a mover draws the words of at once
+constexpr int kQ = 128;                      // a mover's queue of pairs: at most 31 + 64 wait
+// a mover's dynamic shared memory: queue, work cells, words
+constexpr int kMoverBytes = kQ * 16 + 64 * 16 + kWords * 48;
 constexpr unsigned long long kWaitNs = 1000000000ull;  // a wait gives up after 1 s (default)
+static_assert(kRS >= 2 * kMaxMovers, "ring entries of moves that can still be read");
 
 constexpr uint32_t kOld = 1u, kNew = 2u;
 
 // ---------------------------------------------------------------- trials
 struct Trial {
-    uint4 Po, Pn;     // old / new position; Po.w = the particle's tag (~0 for insertions)
-    int co, cn;       // cells (-1 when absent)
-    int idx;          // particle index (-1: none; insertions: filled at decision)
-    unsigned px : 10, py : 10, pz : 10;  // primary neighbourhood centre
-    unsigned possible : 1, cross : 1;
-    unsigned qx : 10, qy : 10, qz : 10;  // new cell (== primary unless the cell changes)
-    unsigned far : 1, pad : 1;
-    unsigned type : 2, s : 4, fpri : 2;
-};
-
-struct AxisList {
-    int v[4];
-    uint32_t f[4];
-    int n;
+    uint4 Po, Pn;          // old / new position; Po.w = the particle's tag (~0 for insertions)
+    int co, cn;            // cells (-1 when absent)
+    int idx;               // particle index (-1: none)
+    int px, py, pz;        // old cell (insertions: the new one)
+    int qx, qy, qz;        // new cell
+    int type, s;
+    bool possible, cross, far;  // cross: the cell changes; far: to a cell that is not adjacent
 };
 
 __device__ __forceinline__ bool near1(int d, int T)
@@ -144,53 +140,23 @@ __device__ __forceinline__ bool near1(int d, int T)
 
 __device__ __forceinline__ int wrapc(int x, int T) { return x < 0 ? x + T : (x >= T ? x - T : x); }
 
-template <typename V>
-__device__ __forceinline__ V sel4(const V (&v)[4], int i)
+// 1 << d, 0 for d outside 0 .. 31
+__device__ __forceinline__ uint32_t bit_at(int d)
 {
-    return i == 0 ? v[0] : (i == 1 ? v[1] : (i == 2 ? v[2] : v[3]));
+    uint32_t r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(d));
+    return r;
 }
-
-// {p-1, p, p+1} flagged f0, united with {q-1, q, q+1} flagged kNew when cross
-__device__ __forceinline__ AxisList axis_list(int p, int q, int cross, uint32_t f0, int T)
-{
-    AxisList L;
-    L.v[0] = wrapc(p - 1, T);
-    L.v[1] = p;
-    L.v[2] = wrapc(p + 1, T);
-    L.f[0] = L.f[1] = L.f[2] = f0;
-    L.v[3] = 0;
-    L.f[3] = 0;
-    L.n = 3;
-    if (cross) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int w = wrapc(q + k - 1, T);
-            const bool h0 = L.v[0] == w, h1 = L.v[1] == w, h2 = L.v[2] == w;
-            L.f[0] |= h0 ? kNew : 0u;
-            L.f[1] |= h1 ? kNew : 0u;
-            L.f[2] |= h2 ? kNew : 0u;
-            if (!(h0 || h1 || h2)) {  // at most one value per axis (|q - p| <= 1)
-                L.v[3] = w;
-                L.f[3] = kNew;
-                L.n = 4;
-            }
-        }
-    }
-    return L;
-}
-
 
 // ---------------------------------------------------------------- shared state
-struct WordRec {
+struct __align__(16) WordRec {
     uint32_t w[8];
     float lnu;  // FP32 ln(u) of the acceptance uniform; NaN: decide in FP64
     int pad[3];
 };
 
-constexpr int kGMax = 8;  // warps per evaluation team, at most
-
-// SM clock for the per-role cycle counters of a profiled launch; an
-// unprofiled launch compiles the reads (and the sums) away.
+// SM clock for the cycle counters of a profiled launch; an unprofiled
+// launch compiles the reads (and the sums) away.
 template <bool PROF>
 __device__ __forceinline__ unsigned long long prof_clock()
 {
@@ -198,612 +164,114 @@ __device__ __forceinline__ unsigned long long prof_clock()
     else return 0ull;
 }
 
-struct Slot {  // evaluators -> committer, one per move in flight
-    Trial t;                      // written by the team's warp 0
-    uint4 last_val;               // the old cell's last entry (by the lane that met it)
-    float ph[kGMax], pu[kGMax];   // per-warp FP32 sums: dU (high word), uabs
-    float pl[kGMax];              // per-warp FP32 sums: dU (low word)
-    double pd[kGMax], pa[kGMax];  // per-warp FP64 sums: dU, uabs
-    float pw[kGMax];              // per-warp FP32 virial change (virial runs)
-    double pwd[kGMax];            // per-warp FP64 virial change (virial runs)
-    int self_slot;                // the trial particle's slot in its old cell, -1 none
-    int has_last;
-    int c0;                       // moves committed when the evaluation started
-    int arrive;                   // warps finished
-    int tag;                      // move + 1 of the evaluation under way, 0 none
-    int tpub;                     // move + 1 whose trial (t, nsu) is published, 0 none
-    int pseq[kGMax];              // per warp: count epoch its work-cell counts were read in (-1 torn)
-    int nsu[kMaxSpecies];         // the particle counts the evaluation picked its particle with
-    int acc0;                     // accepted moves (at most) when the evaluation started
-    // the team's totals, summed by its last warp to arrive (fixed order)
-    float th, tl, tu, tw;         // FP32: dU (hi, lo), uabs, virial change
-    double td, ta, tdw;           // FP64: dU, uabs, virial change
-    int pad[2];
+// What a move changes if it is accepted, for the checks of the moves after
+// it.  A mover writes its entry as soon as its evaluation is in, so that
+// later moves are tested against it before its turn; sh.ver says for which
+// move and evaluation it stands.
+struct __align__(16) LogRec {
+    int4 ids;     // x, y: cells written; z, w: (s << 24) | index of the records written (-1 none)
+    uint4 pos0;   // .w: bit 0 a second position, bit 1 a moved entry, bit 2 an insertion, species << 8
+    uint4 pos1;
+    uint4 moved;  // the cell's last entry, moved into the freed slot
 };
 
-struct __align__(16) LogRec {  // committer -> evaluation validity (five 16-byte words)
-    int4 head;    // x: flags (bit0 accepted, bit1 N changed); y, z, w: cells written (-1 none)
-    int4 ids;     // x, y, z: (s << 24) | index of the records written (-1 none);
-                  // w: positions that gained or lost a particle (np) | has_moved << 8 (a removal
-                  //    moved the cell's last entry into the freed slot)
-    uint4 pos0, pos1;
-    uint4 moved;  // that entry
-};
-
-struct BookRec {  // committer -> keeper
+struct __align__(16) BookRec {  // mover -> keeper
     double dU64, lnA;  // dU when decided in FP64 or evaluated in FP64 mode
     double dW;         // virial change of the trial (virial runs)
     float hi, lo;      // dU = hi + lo otherwise
     float uab;
-    int use64;
-    int fin;      // bit0 accepted
-    int type, sp, index;
-    int possible;
-    int refined;  // bit0 near threshold, bit1 decided in FP64, bit2 evaluated again
-    int pad0;
-    long long ns;  // N_s before the move
-    int ready;
-    int pad1;
+    // bit 0 accepted, 1 possible, 2 dU64 holds dU, 3 near the threshold, 4
+    // decided in FP64, 5 evaluated again; type << 8, species << 16
+    int bits;
+    int index;
+    int n;             // N_s before the move
+    int ready;         // move + 1
+    int pad[3];
 };
+constexpr int kBkAcc = 1, kBkPossible = 2, kBkUse64 = 4, kBkNear = 8, kBkRefined = 16, kBkAgain = 32;
 
 struct __align__(16) Shared {
-    WordRec words[kRW];
-    Slot slots[kRS];
+    // the turn: x = moves committed, y = whether the last 32 of them were
+    // accepted (bit 0 the last one) -- written together -- z = 1 once the
+    // chain stops
+    int4 turn;
     LogRec logs[kRS];
     BookRec book[kRS];
-    long long n[kMaxSpecies];
-    float ln_n[kMaxSpecies];
-    float ln_n1[kMaxSpecies];
-    int ns_ring[kRS][kMaxSpecies];  // N_s after c commits, at [(c) & (kRS - 1)]
-    int committed;  // moves committed
-    int filled;     // words available for moves < filled
-    int booked;     // moves the keeper has processed
-    int stop;       // the committer stopped: no further moves are taken
+    double2 field[kMaxSpecies * kMaxSpecies];  // FP32 mode: float4 (c4e, sig2, c4e_lo, sig2_lo); FP64: (c4e, sig2)
+    int ver[kRS];      // of the log entries: (move << 8) | evaluation, 0 while one is written
+    int outlook[kRS];  // of pending moves: (move << 8) | species << 2 | 1 (adds a particle) or 2 (removes one)
+    int n[kMaxSpecies];
+    int booked;    // moves the keeper has processed
     int status;
-    int where;      // which waits gave up: 1 team leader, 2 committer, 4 keeper
-    // count epoch: even while no cell count is being changed, bumped before
-    // and after every change of the counts (a sequence lock)
-    int seq;
+    int where;     // which waits gave up
+    int gone;      // movers that have finished
+    int never;     // a flag nothing sets (the diagnostic stall waits on it)
     // 1 while this chain accepts most of its insertions [0] / deletions [1]
     // (the bet the count prediction makes on moves not yet evaluated)
     int likely[2];
-    int never;  // a flag nothing sets (the diagnostic stall waits on it)
-    int nacc;   // moves accepted so far (published before the commit count)
+    long long evaluations;
+    unsigned long long prof[12];
 };
 
 __device__ __forceinline__ int vload(const int &x) { return *(volatile const int *)&x; }
 __device__ __forceinline__ void vstore(int &x, int v) { *(volatile int *)&x = v; }
+__device__ __forceinline__ int cload(const uint16_t &x) { return *(volatile const uint16_t *)&x; }
+__device__ __forceinline__ void cstore(uint16_t &x, int v) { *(volatile uint16_t *)&x = (uint16_t)v; }
+__device__ __forceinline__ void fence_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 
-template <bool F32>
-__device__ __forceinline__ void pair_terms(const uint4 &P, const uint4 &q, const ChainArgs &a, int k, float sign,
-                                           FF &e, float &ua, double &de, double &da, double &dw)
+__device__ __forceinline__ int4 turn_load(const Shared &sh)
 {
-    const int dx = (int)(P.x - q.x), dy = (int)(P.y - q.y), dz = (int)(P.z - q.z);
-    // per-axis pre-filter: |d| >= rcg implies d^2 >= R2 (rcg^2 >= R2)
-    if (abs(dx) >= a.rcg || abs(dy) >= a.rcg || abs(dz) >= a.rcg) return;
-    GridSep s;
-    s.dx = dx;
-    s.dy = dy;
-    s.dz = dz;
-    s.g = (unsigned long long)((long long)dx * dx) + (unsigned long long)((long long)dy * dy) +
-          (unsigned long long)((long long)dz * dz);
-    if (s.g >= a.R2) return;
-    if constexpr (F32) {
-        float u, m;
-        lj_f32(s, a.ff.c4e[k], a.ff.sig2[k], u, m);
-        e = ff_add_f(e, sign * u);
-        ua += m;
-    } else {
-        double u, m;
-        lj_f64(s, a.fd.c4e[k], a.fd.sig2[k], u, m);
-        de += (double)sign * u;
-        da += m;
-        dw -= (double)sign * (3.0 * m + 9.0 * u);  // r U'(r) = -12 rep + 6 att
-    }
+    int4 v;
+    asm volatile("ld.volatile.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"(smem_addr(&sh.turn))
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ void turn_store(Shared &sh, int c, uint32_t hist)
+{
+    asm volatile("st.volatile.shared.v2.s32 [%0], {%1, %2};" ::"r"(smem_addr(&sh.turn)), "r"(c), "r"((int)hist)
+                 : "memory");
 }
 
-// The Metropolis test of Eqs. 3-5 (textbook sign of mu) in FP32 with an
-// explicit error band: 1 accept, 0 reject, -1 inside the band or not finite
-// (the caller decides in FP64).  ns: N_s before the move.
-__device__ __forceinline__ int decide_f32(const ChainArgs &a, int type, int sp, float ln_ns, float ln_ns1, float lnu,
-                                          float dUf, float uab)
+// Stops the chain: no further move is committed.
+__device__ __noinline__ void chain_stop(Shared &sh, int status, int where)
 {
-    const float beta_f = a.beta_f, tol_f = a.tol_f;
-    float lnK = 0.f;
-    if (type == 1) lnK = a.lnzv_f[sp] - ln_ns1;
-    else if (type == 2) lnK = ln_ns - a.lnzv_f[sp];
-    const float lnA = lnK - beta_f * dUf;
-    const float band = beta_f * tol_f * uab + 1e-6f * (1.f + fabsf(lnK) + fabsf(beta_f * dUf) + fabsf(lnu));
-    const float diff = lnu - lnA;
-    if (fabsf(diff) > band) return (diff < 0.f) ? 1 : 0;
-    return -1;
+    atomicOr(&sh.status, status);
+    if (where) atomicOr(&sh.where, where);
+    fence_cta();
+    *(volatile int *)&sh.turn.z = 1;
 }
 
-// ---------------------------------------------------------------- the chain
-// VIR: the evaluations also sum the virial change dW of each trial.
-// entries of an evaluator warp's queue of pair terms inside the cutoff: at
-// most 31 wait between drains, and one item adds at most 64
-constexpr int kQ = 128;
-constexpr int kMaxEW = 14;  // evaluator warps, at most (queues in dynamic shared memory)
-constexpr int kChainWarps = 16;  // warps of a chain CTA (committer, keeper, evaluators, idle)
+// |a - p| along an axis, the minimum image as an unsigned 32-bit distance.
+__device__ __forceinline__ uint32_t axis_dist(uint32_t a, uint32_t p)
+{
+    const uint32_t d = a - p;
+    return min(d, 0u - d);
+}
 
-template <bool F32, bool VIR>
-struct Chain {
-    const ChainArgs &a;
-    Shared &sh;
-    uint16_t *cnt;
-    int4 *fq;  // kQ entries per evaluator warp
-    int lane, warp, T;
-    int eidx = 0;  // this warp's index among the evaluator warps
-    int first_mod;  // first move of the launch modulo the words ring
-    uint32_t uT;
+// ---------------------------------------------------------------- a mover
+// Sums of an evaluation: dU = e + el in FP32, de in FP64; uabs; virial change.
+struct Sums {
+    float e, el, ua, w;
+    double de, da, dw;
+};
 
-    __device__ Chain(const ChainArgs &a_, Shared &sh_, uint16_t *cnt_, int4 *fq_) : a(a_), sh(sh_), cnt(cnt_), fq(fq_)
-    {
-        lane = threadIdx.x & 31;
-        warp = threadIdx.x >> 5;
-        T = a.T;
-        uT = (uint32_t)a.T;
-        first_mod = (int)(a.first & (uint64_t)(kRW - 1));
-    }
-
-    __device__ __forceinline__ const WordRec &words(int m) const
-    {
-        return sh.words[(first_mod + m) & (kRW - 1)];
-    }
-
-    // Whether move m's trial is the same for every count its pick can meet
-    // at its turn, `delta` moves after the counts ns[] (each pending move
-    // changes one count by at most one): then the evaluation needs no count
-    // prediction.  An insertion does not depend on the counts; a
-    // displacement among several species does through the species of the
-    // pick, and is left to the prediction.
-    __device__ __forceinline__ bool pick_settled(int m, const int *ns, int delta) const
-    {
-        const WordRec &W = words(m);
-        const uint32_t w0 = W.w[0];
-        const int type = (w0 < a.thr_disp) ? 0 : ((w0 < a.thr_ins) ? 1 : 2);
-        if (type == 1) return true;
-        if (type == 0 && a.S != 1) return false;
-        const int n = ns[type == 2 ? (int)__umulhi(W.w[5], (uint32_t)a.S) : 0];
-        if (n - delta < 1) return false;
-        return pick_is_stable((uint32_t)(n - delta), (uint32_t)(n + delta), W.w, type);
-    }
-
-    // the trial of move m given the particle counts ns[] (warp-uniform)
-    __device__ __forceinline__ Trial make_trial(int m, const int *ns) const
-    {
-        const WordRec &W = words(m);
-        Trial t;
-        const uint32_t w0 = W.w[0];
-        const int type = (w0 < a.thr_disp) ? 0 : ((w0 < a.thr_ins) ? 1 : 2);
-        t.type = type;
-        t.possible = 1;
-        t.cross = 0;
-        t.far = 0;
-        t.pad = 0;
-        int s = 0, idx = -1;
-        if (type == 0) {
-            int N = 0;
-            for (int q = 0; q < a.S; ++q) N += ns[q];
-            if (N == 0) {
-                t.possible = 0;
-            } else {
-                int k = pick_index((uint32_t)N, W.w, 0);
-                while (k >= ns[s]) {
-                    k -= ns[s];
-                    ++s;
-                }
-                idx = k;
-            }
-        } else {
-            s = (int)__umulhi(W.w[5], (uint32_t)a.S);
-            if (type == 2) {
-                if (ns[s] == 0) t.possible = 0;
-                else idx = pick_index((uint32_t)ns[s], W.w, 2);
-            }
-        }
-        t.s = s;
-        t.idx = idx;
-        t.Po = make_uint4(0, 0, 0, 0xFFFFFFFFu);
-        t.Pn = make_uint4(0, 0, 0, 0);
-        t.co = t.cn = -1;
-        t.px = t.py = t.pz = t.qx = t.qy = t.qz = 0;
-        t.fpri = 0;
-        if (!t.possible) return t;
-        if (type != 1) {
-            const uint4 rec = a.pos_by_id[(long long)s * a.maxN + idx];
-            t.Po = rec;
-            t.px = cell_coord(rec.x, uT);
-            t.py = cell_coord(rec.y, uT);
-            t.pz = cell_coord(rec.z, uT);
-            t.co = ((int)t.pz * T + (int)t.py) * T + (int)t.px;
-        }
-        if (type == 0) {
-            t.Pn.x = t.Po.x + (uint32_t)((int)__umulhi(W.w[2], a.span) - a.D);
-            t.Pn.y = t.Po.y + (uint32_t)((int)__umulhi(W.w[3], a.span) - a.D);
-            t.Pn.z = t.Po.z + (uint32_t)((int)__umulhi(W.w[4], a.span) - a.D);
-            t.Pn.w = t.Po.w;
-        } else if (type == 1) {
-            t.Pn = make_uint4(W.w[2], W.w[3], W.w[4], 0u);
-        }
-        if (type != 2) {
-            t.qx = cell_coord(t.Pn.x, uT);
-            t.qy = cell_coord(t.Pn.y, uT);
-            t.qz = cell_coord(t.Pn.z, uT);
-            t.cn = ((int)t.qz * T + (int)t.qy) * T + (int)t.qx;
-        }
-        if (type == 1) {
-            t.px = t.qx;
-            t.py = t.qy;
-            t.pz = t.qz;
-            t.fpri = kNew;
-        } else if (type == 2) {
-            t.qx = t.px;
-            t.qy = t.py;
-            t.qz = t.pz;
-            t.fpri = kOld;
-        } else {
-            t.cross = (t.co != t.cn) ? 1 : 0;
-            t.fpri = t.cross ? kOld : (kOld | kNew);
-            t.far = t.cross && !(near1((int)t.px - (int)t.qx, T) && near1((int)t.py - (int)t.qy, T) &&
-                                 near1((int)t.pz - (int)t.qz, T));
-        }
-        return t;
-    }
-
-    // The cells a trial visits (its work list), indexed 0 .. nwork - 1: the
-    // 27 around its primary cell (no cell change, insertions, deletions);
-    // for a displacement into an adjacent cell the union of the old and new
-    // neighbourhoods, 3 or 4 values per axis, each cell flagged kOld and/or
-    // kNew (cells of the union box in neither neighbourhood carry no flag);
-    // for a longer displacement the old 27 (kOld) followed by the new 27
-    // (kNew).  At most 64 cells.
-    __device__ __forceinline__ int nwork(const Trial &t) const
-    {
-        if (!t.possible) return 0;
-        if (!t.cross) return 27;
-        if (t.far) return 54;
-        const int nx = (t.px == t.qx || T == 3) ? 3 : 4;
-        const int ny = (t.py == t.qy || T == 3) ? 3 : 4;
-        const int nz = (t.pz == t.qz || T == 3) ? 3 : 4;
-        return nx * ny * nz;
-    }
-
-    __device__ __forceinline__ void work_cell(const Trial &t, const AxisList &X, const AxisList &Y,
-                                              const AxisList &Z, int i, int &cell, uint32_t &fl) const
-    {
-        if (!t.cross || t.far) {
-            const bool nw = t.far && i >= 27;
-            const int k = nw ? i - 27 : i;
-            const int dz = k / 9, r = k - 9 * (k / 9);
-            const int dy = r / 3, dx = r - 3 * (r / 3);
-            const int cx = nw ? (int)t.qx : (int)t.px, cy = nw ? (int)t.qy : (int)t.py;
-            const int cz = nw ? (int)t.qz : (int)t.pz;
-            cell = (wrapc(cz + dz - 1, T) * T + wrapc(cy + dy - 1, T)) * T + wrapc(cx + dx - 1, T);
-            fl = t.far ? (nw ? kNew : kOld) : (uint32_t)t.fpri;
-            return;
-        }
-        int ix, q1, iy, iz;
-        if (X.n == 4) {
-            ix = i & 3;
-            q1 = i >> 2;
-        } else {
-            q1 = i / 3;
-            ix = i - 3 * q1;
-        }
-        if (Y.n == 4) {
-            iy = q1 & 3;
-            iz = q1 >> 2;
-        } else {
-            iz = q1 / 3;
-            iy = q1 - 3 * iz;
-        }
-        cell = (sel4(Z.v, iz) * T + sel4(Y.v, iy)) * T + sel4(X.v, ix);
-        fl = sel4(X.f, ix) & sel4(Y.f, iy) & sel4(Z.f, iz);
-    }
-
-    // One item (a particle of a work cell) against the trial's old and/or new
-    // position.  The cutoff is screened on the FP32 squared distance, except
-    // inside a thin band around rc^2 where the exact integer squared distance
-    // decides; the pairs inside the cutoff join the warp's queue and are
-    // evaluated 32 at a time in compensated FP32 (lj_ff), so the warp spends
-    // the long pair term only on the ~15 % of items inside the cutoff.
-    // Per-evaluation constants of the FP32 item: the pair table entry of a
-    // single-species chain and the band around rc^2 (registers).
-    struct ItemK {
-        float c4e, sig2, c4l, sil, r2lo, r2hi;
-        bool single, vir;
-    };
-
-    __device__ __forceinline__ ItemK item_consts() const
-    {
-        ItemK K;
-        K.single = a.S == 1;
-        K.c4e = a.ff.c4e[0];
-        K.sig2 = a.ff.sig2[0];
-        K.c4l = a.ff.c4e_lo[0];
-        K.sil = a.ff.sig2_lo[0];
-        K.r2lo = a.r2lo;
-        K.r2hi = a.r2hi;
-        K.vir = VIR;
-        return K;
-    }
-
-    // A warp's queue of pair terms inside the cutoff: entries (ex, ey, ez,
-    // pair index | 0x100 for a term that counts negatively), a ring of kQ.
-    struct FQ {
-        int4 *buf;
-        int head, n;
-    };
-    // Per-lane sums of the FP32 evaluation: dU as hi + lo, uabs, virial.
-    struct Acc32 {
-        float eh, el, mag, wac;
-    };
-
-    // Evaluates `count` (<= 32) queued terms, one per lane, and adds them.
-    __device__ __forceinline__ void drain(const FQ &Q, int count, const ItemK &K, Acc32 &A) const
-    {
-        if (lane < count) {
-            const int4 e = Q.buf[(Q.head + lane) & (kQ - 1)];
-            const int kk = e.w & 0xFF;
-            float ch = K.c4e, cl = K.c4l, sh2 = K.sig2, sl2 = K.sil;
-            if (!K.single) {
-                ch = a.ff.c4e[kk];
-                cl = a.ff.c4e_lo[kk];
-                sh2 = a.ff.sig2[kk];
-                sl2 = a.ff.sig2_lo[kk];
-            }
-            float uh, ul, m;
-            lj_ff(e.x, e.y, e.z, ch, cl, sh2, sl2, uh, ul, m);
-            const bool neg = (e.w & 0x100) != 0;
-            ff_acc(A.eh, A.el, neg ? -uh : uh, neg ? -ul : ul);
-            A.mag += m;
-            if (K.vir) {
-                const float w = -fmaf(3.f, m, 9.f * uh);  // r U'(r) = -12 rep + 6 att
-                A.wac += neg ? -w : w;
-            }
-        }
-    }
-
-    // Adds the lanes' entries (where `in`) to the queue.
-    __device__ __forceinline__ void enqueue(FQ &Q, bool in, const int4 &ent) const
-    {
-        const unsigned bm = __ballot_sync(0xffffffffu, in);
-        if (bm == 0u) return;
-        if (in) Q.buf[(Q.head + Q.n + __popc(bm & ((1u << lane) - 1u))) & (kQ - 1)] = ent;
-        Q.n += __popc(bm);
-    }
-
-    // Evaluates queued terms, 32 at a time (fewer for the last), while at
-    // least `thr` wait.  One loop serves the whole evaluation, so the long
-    // compensated pair term appears once in the kernel's code.
-    __device__ __forceinline__ void drain_while(FQ &Q, int thr, const ItemK &K, Acc32 &A) const
-    {
-#pragma unroll 1
-        while (Q.n >= thr) {
-            const int c = min(Q.n, 32);
-            __syncwarp();
-            drain(Q, c, K, A);
-            Q.head = (Q.head + c) & (kQ - 1);
-            Q.n -= c;
-            __syncwarp();
-        }
-    }
-
-    // TWO: both positions of a displacement; else the old position of a
-    // deletion or the new one of an insertion.  Each separation is converted
-    // from its exact integer value (the new one is not the old separation
-    // plus the displacement in FP32, which would round the longer old one).
-    template <bool TWO>
-    __device__ __forceinline__ void item32(const Trial &t, const uint4 &q, bool valid, uint32_t fl,
-                                           const ItemK &K, FQ &Q) const
-    {
-        const bool use = valid && (q.w != t.Po.w);
-        const int kk = K.single ? 0 : (int)t.s * kMaxSpecies + (int)tag_species(q.w);
-        const bool del = t.type == 2;
-#pragma unroll
-        for (int side = 0; side < (TWO ? 2 : 1); ++side) {
-            const bool old = TWO ? side == 0 : del;
-            const uint32_t px = old ? t.Po.x : t.Pn.x, py = old ? t.Po.y : t.Pn.y, pz = old ? t.Po.z : t.Pn.z;
-            const int ex = (int)(px - q.x), ey = (int)(py - q.y), ez = (int)(pz - q.z);
-            const float gx = (float)ex, gy = (float)ey, gz = (float)ez;
-            const float r2f = fmaf(gx, gx, fmaf(gy, gy, gz * gz));
-            const bool want = use && (fl & (old ? kOld : kNew));
-            bool in = want && (r2f < K.r2lo);
-            // inside the thin band around rc^2 the exact integer test decides
-            const bool band = want && r2f >= K.r2lo && r2f <= K.r2hi;
-            if (__any_sync(0xffffffffu, band)) {
-                if (band) {
-                    const unsigned long long g = (unsigned long long)((long long)ex * ex) +
-                                                 (unsigned long long)((long long)ey * ey) +
-                                                 (unsigned long long)((long long)ez * ez);
-                    in = g < a.R2;
-                }
-            }
-            enqueue(Q, in, make_int4(ex, ey, ez, kk | (old ? 0x100 : 0)));
-        }
-    }
-
-    // One warp's share of a trial's energy change.  The items (particles) of
-    // the work cells are numbered in work-list order; warp j of a team of G
-    // takes the contiguous range [j P / G, (j + 1) P / G) of the P items, 32
-    // KU items per pass (KU per lane, loads in flight together).  P32: FP32
-    // pair terms summed in FP32 per lane and across the warp; else FP64.
-    // Returns the warp's sums (in every lane) and, in the lane that met
-    // them, the trial particle's slot in its old cell and that cell's last
-    // entry.
-    struct Part {
-        float e, el, ua, w;  // FP32 runs: dU = e + el
-        double de, da, dw;
-        int self_slot, has_last;
-        int seq;  // count epoch of the work-cell counts this warp read, -1 if a change tore them
-        uint4 last;
-    };
-
-    template <bool P32>
-    __device__ __forceinline__ void item(const Trial &t, const uint4 &q, bool valid, uint32_t fl, const ItemK &K,
-                                         FQ &Q, double &de, double &da, double &dw) const
-    {
-        if constexpr (P32) {
-            if (t.type == 0) item32<true>(t, q, valid, fl, K, Q);
-            else item32<false>(t, q, valid, fl, K, Q);
-        } else if (valid && q.w != t.Po.w) {
-            FF e0 = {0.f, 0.f};
-            float u0 = 0.f;
-            const int kk = (int)t.s * kMaxSpecies + (int)tag_species(q.w);
-            if (fl & kOld) pair_terms<false>(t.Po, q, a, kk, -1.f, e0, u0, de, da, dw);
-            if (fl & kNew) pair_terms<false>(t.Pn, q, a, kk, 1.f, e0, u0, de, da, dw);
-        }
-    }
-
-    template <bool P32, int KU>
-    __device__ __forceinline__ Part eval_part(const Trial &t, int j, int G) const
-    {
-        Part o;
-        o.self_slot = -1;
-        o.has_last = 0;
-        o.last = make_uint4(0, 0, 0, 0);
-        Acc32 A = {0.f, 0.f, 0.f, 0.f};
-        FQ Q = {P32 ? fq + eidx * kQ : nullptr, 0, 0};
-        double de = 0.0, da = 0.0, dw = 0.0;
-        const int nw = nwork(t);
-        AxisList X, Y, Z;
-        X.n = Y.n = Z.n = 3;
-        if (t.cross && !t.far) {
-            X = axis_list(t.px, t.qx, 1, kOld, T);
-            Y = axis_list(t.py, t.qy, 1, kOld, T);
-            Z = axis_list(t.pz, t.qz, 1, kOld, T);
-        }
-        // a lane owns work cells lane and lane + 32; their counts are read
-        // inside one count epoch (the sequence lock around count changes)
-        int ca = 0, cb = 0, na = 0, nb = 0;
-        uint32_t fa = 0, fb = 0;
-        if (lane < nw) work_cell(t, X, Y, Z, lane, ca, fa);
-        if (lane + 32 < nw) work_cell(t, X, Y, Z, lane + 32, cb, fb);
-        const int s0 = vload(sh.seq);
-        __threadfence_block();
-        if (lane < nw) na = fa ? (int)cnt[ca] : 0;
-        if (lane + 32 < nw) nb = fb ? (int)cnt[cb] : 0;
-        __threadfence_block();
-        const int s1 = vload(sh.seq);
-        const int w0 = __shfl_sync(0xffffffffu, s0, 0);
-        o.seq = __all_sync(0xffffffffu, s0 == s1 && s0 == w0 && !(s0 & 1)) ? w0 : -1;
-        // items end at ia (cells 0 .. 31) and ib (cells 32 .. 63), inclusive
-        const int ia = warp_inclusive_scan(na);
-        const int ib = warp_inclusive_scan(nb) + __shfl_sync(0xffffffffu, ia, 31);
-        const int P = __shfl_sync(0xffffffffu, ib, 31);
-        const int lo = (P * j) / G, hi = (P * (j + 1)) / G;
-        const ItemK K = item_consts();
-        for (int base = lo; base < hi; base += 32 * KU) {
-            int cell[KU], slot[KU], ncl[KU];
-            uint32_t flg[KU];
-#pragma unroll
-            for (int u = 0; u < KU; ++u) {
-                cell[u] = -1;
-                slot[u] = 0;
-                ncl[u] = 0;
-                flg[u] = 0;
-            }
-            const int fend = min(hi, base + 32 * KU) - 1;
-            // the work cells holding items base .. fend (warp-uniform)
-            const int c0 = __popc(__ballot_sync(0xffffffffu, ia <= base)) + __popc(__ballot_sync(0xffffffffu, ib <= base));
-            const int c1 = __popc(__ballot_sync(0xffffffffu, ia <= fend)) + __popc(__ballot_sync(0xffffffffu, ib <= fend));
-            for (int c = c0; c <= c1; ++c) {
-                const int src = c & 31;
-                const bool up = c >= 32;
-                const int end = __shfl_sync(0xffffffffu, up ? ib : ia, src);
-                const int nc = __shfl_sync(0xffffffffu, up ? nb : na, src);
-                const int cid = __shfl_sync(0xffffffffu, up ? cb : ca, src);
-                const uint32_t fl = __shfl_sync(0xffffffffu, up ? fb : fa, src);
-                const int st = end - nc;
-#pragma unroll
-                for (int u = 0; u < KU; ++u) {
-                    const int f = base + lane + 32 * u;
-                    if (f >= st && f < end && f < hi) {
-                        cell[u] = cid;
-                        slot[u] = f - st;
-                        ncl[u] = nc;
-                        flg[u] = fl;
-                    }
-                }
-            }
-            uint4 q[KU];
-#pragma unroll
-            for (int u = 0; u < KU; ++u)
-                q[u] = (cell[u] >= 0) ? a.cell_pos[(long long)cell[u] * a.cap + slot[u]]
-                                      : make_uint4(0, 0, 0, 0xFFFFFFFEu);
-#pragma unroll
-            for (int u = 0; u < KU; ++u) {
-                if (cell[u] >= 0 && (flg[u] & kOld) && cell[u] == t.co) {
-                    if (q[u].w == t.Po.w) o.self_slot = slot[u];
-                    else if (slot[u] == ncl[u] - 1) {
-                        o.has_last = 1;
-                        o.last = q[u];
-                    }
-                }
-            }
-            if constexpr (P32) {
-                // one item at a time (not unrolled), then the queue's full
-                // batches: the screen and the pair term appear once in code
-#pragma unroll 1
-                for (int u = 0; u < KU; ++u) {
-                    uint4 qu = q[0];
-                    uint32_t fu = flg[0];
-                    int cu = cell[0];
-#pragma unroll
-                    for (int i = 1; i < KU; ++i)
-                        if (u == i) {
-                            qu = q[i];
-                            fu = flg[i];
-                            cu = cell[i];
-                        }
-                    item<true>(t, qu, cu >= 0, fu, K, Q, de, da, dw);
-                    drain_while(Q, 32, K, A);
-                }
-            } else {
-#pragma unroll
-                for (int u = 0; u < KU; ++u) item<false>(t, q[u], cell[u] >= 0, flg[u], K, Q, de, da, dw);
-            }
-        }
-        o.w = 0.f;
-        o.dw = 0.0;
-        if constexpr (P32) {
-            drain_while(Q, 1, K, A);
-            __syncwarp();
-            const FF e = ff_warp_sum(FF{A.eh, A.el});
-            o.e = e.hi;
-            o.el = e.lo;
-            o.ua = warp_sum(A.mag);
-            if (K.vir) o.w = warp_sum(A.wac);
-            o.de = o.da = 0.0;
-        } else {
-            o.e = o.el = o.ua = 0.f;
-            o.de = warp_sum(de);
-            o.da = warp_sum(da);
-            if (K.vir) o.dw = warp_sum(dw);
-        }
-        return o;
-    }
-
-    // the words of moves [m0, m0 + count) (count <= 32), computed by one warp
-    __device__ __forceinline__ void fill_words(int m0, int count) const
-    {
-        const uint2 key = make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32));
-        if (lane < count) {
-            const uint64_t m = a.first + (uint64_t)(m0 + lane);
-            const uint4 r0 = philox_block(make_uint4((uint32_t)m, (uint32_t)(m >> 32), a.chain, 0u), key);
-            const uint4 r1 = philox_block(make_uint4((uint32_t)m, (uint32_t)(m >> 32), a.chain, 1u), key);
-            WordRec &W = sh.words[(int)(m & (uint64_t)(kRW - 1))];
-            W.w[0] = r0.x;
-            W.w[1] = r0.y;
-            W.w[2] = r0.z;
-            W.w[3] = r0.w;
-            W.w[4] = r1.x;
-            W.w[5] = r1.y;
-            W.w[6] = r1.z;
-            W.w[7] = r1.w;
-            const uint64_t k53 = ((uint64_t)(r1.z >> 5) << 26) | (uint64_t)(r1.w >> 6);
+// The words of moves m, m + W, ... (at most kWords of them below n): lane l
+// draws block l & 1 of the (l >> 1)-th.  (Out of line, as what follows: rare
+// code is kept out of the loop, which has to stay in the instruction cache.)
+__device__ __noinline__ void fill_words(const ChainArgs &a, WordRec *words, int m, int lane)
+{
+    const long long mk = (long long)m + (long long)(lane >> 1) * a.movers;
+    __syncwarp();
+    if (mk < a.n_moves) {
+        const uint64_t mv = a.first + (uint64_t)mk;
+        const uint4 r = philox_block(make_uint4((uint32_t)mv, (uint32_t)(mv >> 32), a.chain, (uint32_t)(lane & 1)),
+                                     make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32)));
+        WordRec &W = words[lane >> 1];
+        ((uint4 *)W.w)[lane & 1] = r;
+        if (lane & 1) {
+            const uint64_t k53 = ((uint64_t)(r.z >> 5) << 26) | (uint64_t)(r.w >> 6);
             float l;
             if (k53 == 0) l = -INFINITY;                                   // u = 0: always accept
             else if (k53 < (1ull << 27)) l = __int_as_float(0x7fc00000);  // u < 2^-26: decide in FP64
@@ -811,938 +279,1006 @@ struct Chain {
             W.lnu = l;
         }
     }
-
-    // One side of a change of the cell counts (the committer's lane 0 only):
-    // the count epoch turns odd before the change and even after it.
-    __device__ __forceinline__ void seq_bump() const
-    {
-        __threadfence_block();
-        vstore(sh.seq, vload(sh.seq) + 1);
-        __threadfence_block();
-    }
+    __syncwarp();
+}
 
 
-    // Committer: apply an accepted move (Sec. 3.2.5), log what it changed
-    // (gathered in registers, stored as five 16-byte words).
-    __device__ __forceinline__ void apply(const Trial &t, int self_slot, const uint4 &last_val, LogRec &L) const
-    {
-        const int sp = t.s;
-        const long long sb = (long long)sp * a.maxN;
-        int cells[3] = {-1, -1, -1}, ids[3] = {-1, -1, -1};
-        int np = 0, has_moved = 0;
-        uint4 pos0 = make_uint4(0, 0, 0, 0), pos1 = pos0, moved = pos0;
-        if (t.type != 2) {
-            if (lane == 0) {
-                if (t.type == 0) {
-                    const uint4 v = make_uint4(t.Pn.x, t.Pn.y, t.Pn.z, t.Po.w);
-                    if (!t.cross) {
-                        a.cell_pos[(long long)t.co * a.cap + self_slot] = v;
-                        cells[0] = t.co;
-                    } else {
-                        seq_bump();
-                        const int c_o = cnt[t.co];
-                        if (self_slot != c_o - 1) {
-                            a.cell_pos[(long long)t.co * a.cap + self_slot] = last_val;
-                            has_moved = 1;
-                            moved = last_val;
-                        }
-                        cnt[t.co] = (uint16_t)(c_o - 1);
-                        const int c_n = cnt[t.cn];
-                        a.cell_pos[(long long)t.cn * a.cap + c_n] = v;
-                        cnt[t.cn] = (uint16_t)(c_n + 1);
-                        seq_bump();
-                        cells[0] = t.co;
-                        cells[1] = t.cn;
-                    }
-                    pos0 = t.Po;
-                    pos1 = t.Pn;
-                    np = 2;
-                    a.pos_by_id[sb + t.idx] = v;
-                    ids[0] = (sp << 24) | t.idx;
-                } else {
-                    const long long ni = sh.n[sp];
-                    const uint4 v = make_uint4(t.Pn.x, t.Pn.y, t.Pn.z, make_tag((uint32_t)ni, (uint32_t)sp));
-                    seq_bump();
-                    const int c_n = cnt[t.cn];
-                    a.cell_pos[(long long)t.cn * a.cap + c_n] = v;
-                    cnt[t.cn] = (uint16_t)(c_n + 1);
-                    seq_bump();
-                    a.pos_by_id[sb + ni] = v;
-                    sh.n[sp] = ni + 1;
-                    sh.ln_n[sp] = logf((float)(ni + 1));
-                    sh.ln_n1[sp] = logf((float)(ni + 2));
-                    cells[0] = t.cn;
-                    ids[0] = (sp << 24) | (int)ni;
-                    pos0 = t.Pn;
-                    np = 1;
-                }
-                L.ids = make_int4(ids[0], ids[1], ids[2], np | (has_moved << 8));
-                L.pos0 = pos0;
-                L.pos1 = pos1;
-                L.moved = moved;
-                L.head = make_int4(1 | ((t.type == 1) ? 2 : 0), cells[0], cells[1], cells[2]);
-            }
-            return;
-        }
-        // deletion: swap-with-last inside the cell, then the species' last
-        // index takes the freed index (its record and its cell entry)
-        const long long last = sh.n[sp] - 1;
-        if (lane == 0) {
-            seq_bump();
-            const int c_o = cnt[t.co];
-            has_moved = self_slot != c_o - 1;
-            if (has_moved) a.cell_pos[(long long)t.co * a.cap + self_slot] = last_val;
-            cnt[t.co] = (uint16_t)(c_o - 1);
-            seq_bump();
-            moved = last_val;
-        }
-        __syncwarp();
-        int cq = -1;
-        if (t.idx != last) {
-            const uint4 Q = a.pos_by_id[sb + last];
-            cq = (cell_coord(Q.z, uT) * T + cell_coord(Q.y, uT)) * T + cell_coord(Q.x, uT);
-            const int cc = cnt[cq];
-            const uint32_t ntag = make_tag((uint32_t)t.idx, (uint32_t)sp);
-            for (int base = 0; base < cc; base += 32) {
-                const int j = base + lane;
-                bool hit = false;
-                if (j < cc) hit = a.cell_pos[(long long)cq * a.cap + j].w == Q.w;
-                const unsigned hb = __ballot_sync(0xffffffffu, hit);
-                if (hit) a.cell_pos[(long long)cq * a.cap + j].w = ntag;
-                if (hb) break;
-            }
-            if (lane == 0) a.pos_by_id[sb + t.idx] = make_uint4(Q.x, Q.y, Q.z, ntag);
-        }
-        if (lane == 0) {
-            cells[0] = t.co;
-            ids[0] = (sp << 24) | t.idx;
-            if (cq >= 0) {
-                cells[1] = cq;
-                ids[1] = (sp << 24) | (int)last;
-            }
-            L.ids = make_int4(ids[0], ids[1], ids[2], 1 | (has_moved << 8));
-            L.pos0 = t.Po;
-            L.pos1 = make_uint4(0, 0, 0, 0);
-            L.moved = moved;
-            L.head = make_int4(3, cells[0], cells[1], cells[2]);
-            sh.n[sp] = last;
-            sh.ln_n[sp] = logf((float)last);
-            sh.ln_n1[sp] = logf((float)(last + 1));
-        }
-    }
+// The slot of `tag` in a cell of n entries (-1: not there), and in lane (n - 1)
+// & 31 the last entry; v: the lane's entry of the first 32.
+struct Found {
+    int at;
+    uint4 last;
 };
-
-// Whether some point of the grid box spanned by X0 and X1 (per axis, in
-// minimum-image coordinates relative to P) lies within the cutoff of P.
-// A record overwritten in place may be read with coordinates from either
-// value, so a move's old and new positions are tested as a box.
-__device__ __forceinline__ long long axis_gap(uint32_t a0, uint32_t a1, uint32_t p)
+__device__ __noinline__ Found find_far(const uint4 *cell, uint32_t tag, int n, uint4 v, int lane)
 {
-    long long lo = (int)(a0 - p), hi = (int)(a1 - p);
-    if (lo > hi) {
-        const long long t = lo;
-        lo = hi;
-        hi = t;
+    Found r = {-1, v};
+#pragma unroll 1
+    for (int b = 0; b < n; b += 32) {
+        const bool have = b + lane < n;
+        if (b > 0 && have) v = cell[b + lane];
+        const unsigned hit = __ballot_sync(0xffffffffu, have && v.w == tag);
+        if (hit && r.at < 0) r.at = b + __ffs(hit) - 1;
+        if (b + lane == n - 1) r.last = v;
     }
-    return lo > 0 ? lo : (hi < 0 ? -hi : 0);
+    return r;
 }
 
-// |a - p| along an axis, the minimum image as an unsigned 32-bit distance.
-__device__ __forceinline__ uint32_t axis_dist(uint32_t a, uint32_t p)
+// The record of particle (s, i), its cell and its slot there (at its turn only).
+struct Entry {
+    uint4 Q;
+    int cell, slot;
+};
+__device__ __noinline__ Entry find_now(const ChainArgs &a, const uint16_t *cnt, int s, int i, int lane)
 {
-    const uint32_t d = a - p;
-    return (d & 0x80000000u) ? 0u - d : d;
+    Entry r;
+    r.Q = a.pos_by_id[(long long)s * a.maxN + i];
+    r.cell = cell_of(r.Q.x, r.Q.y, r.Q.z, a.T);
+    const int n = cload(cnt[r.cell]);
+    const uint4 *cell = a.cell_pos + (long long)r.cell * a.cap;
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (lane < n) v = cell[lane];
+    r.slot = find_far(cell, r.Q.w, n, v, lane).at;
+    return r;
 }
 
-__device__ __forceinline__ bool box_within(const uint4 &X0, const uint4 &X1, const uint4 &P, unsigned long long R2,
-                                           uint32_t rcg)
+// The decision in FP64: accepted, near the threshold, ln A.
+struct Decision {
+    int bits;
+    double lnA;
+};
+__device__ __noinline__ Decision decide_f64(const ChainArgs &a, uint32_t w6, uint32_t w7, int type, int s, int ns,
+                                            double de, double da)
 {
-    // a box whose gap along one axis reaches rcg (rcg^2 >= R2) is out of
-    // reach: for a point record (X0 == X1) that settles most tests in
-    // 32-bit arithmetic
-    const uint32_t g0 = min(axis_dist(X0.x, P.x), axis_dist(X1.x, P.x));
-    const uint32_t g1 = min(axis_dist(X0.y, P.y), axis_dist(X1.y, P.y));
-    const uint32_t g2 = min(axis_dist(X0.z, P.z), axis_dist(X1.z, P.z));
-    if (g0 >= rcg || g1 >= rcg || g2 >= rcg) return false;
-    const long long dx = axis_gap(X0.x, X1.x, P.x), dy = axis_gap(X0.y, X1.y, P.y), dz = axis_gap(X0.z, X1.z, P.z);
-    return (unsigned long long)(dx * dx) + (unsigned long long)(dy * dy) + (unsigned long long)(dz * dz) < R2;
-}
-
-// Whether the committed moves [j0, j1) left a trial's evaluation standing:
-// none of them touched its old cell or wrote its particle's record, and
-// none put, removed or moved a particle within rc of its old or new
-// position.  Warp-wide, four lanes per logged move (eight moves a pass):
-// lane 4i + k tests, for move j0 + i, the positions it wrote (k = 0, 1) or
-// the entry it moved (k = 2, 3) against the trial's old (k even) or new
-// (k odd) position; lane 4i also compares cells and records.  The result is
-// uniform.
-template <bool F32, bool VIR>
-__device__ __forceinline__ bool logs_ok(const Chain<F32, VIR> &C, const Shared &sh, const Trial &t, int j0, int j1,
-                                        int lane)
-{
-    bool bad = false;
-    const ChainArgs &a = C.a;
-    if (t.possible) {
-        const int k = lane & 3;
-        const bool side = (k & 1) ? t.type != 2 : t.type != 1;
-        const bool old_side = t.type != 1;
-        const int myid = ((int)t.s << 24) | t.idx;
-        const uint4 P = (k & 1) ? t.Pn : t.Po;
-        const unsigned long long R2 = a.R2;
-        const uint32_t rcg = (uint32_t)a.rcg;
-        for (int j = j0 + (lane >> 2); j < j1; j += 8) {
-            // the log entry's words, loaded together
-            const LogRec &L = sh.logs[j & (kRS - 1)];
-            const int4 h = L.head, id = L.ids;
-            const uint4 X0 = (k < 2) ? L.pos0 : L.moved;
-            const uint4 X1r = (k < 2) ? L.pos1 : L.moved;
-            if (!(h.x & 1)) continue;
-            // the old cell's slots (self, last entry) must be as seen, and
-            // the particle's record must be as read
-            if (k == 0 && old_side &&
-                (h.y == t.co || h.z == t.co || h.w == t.co || id.x == myid || id.y == myid || id.z == myid))
-                bad = true;
-            // a particle that appeared, vanished or moved within rc of the
-            // trial's old or new position changes dU (exact integer cutoff,
-            // as in Eq. 1's sum); so may a cell's last entry that a removal
-            // moved into the freed slot (an evaluation that read the older
-            // count may have met it twice).  Changes farther away add
-            // nothing: their pair terms are exactly zero.
-            const bool use = side && (k < 2 || (id.w >> 8) != 0);
-            const uint4 X1 = (k < 2 && (id.w & 0xFF) == 2) ? X1r : X0;
-            if (use && box_within(X0, X1, P, R2, rcg)) bad = true;
-        }
+    const double lnu = log(uniform53(w6, w7));
+    double lnK = 0.0;
+    if (type != 0) {
+        lnK = log((double)(type == 1 ? ns + 1 : ns));
+        if (type == 1) lnK = a.logz[s] + a.lnV - lnK;
+        else lnK = lnK - a.logz[s] - a.lnV;
     }
-    return !__any_sync(0xffffffffu, bad);
+    Decision d;
+    d.lnA = lnK - a.beta * de;
+    const double band = a.beta * a.tol * da + 1e-12 * (1.0 + fabs(d.lnA));
+    d.bits = (lnu < d.lnA ? kBkAcc : 0) | (fabs(lnu - d.lnA) <= band ? kBkNear : 0);
+    return d;
 }
 
-// Whether the particle counts at move m's turn pick the particle the
-// evaluation used (it may have used predicted counts), or still make an
-// impossible move impossible.
-template <bool F32, bool VIR>
-__device__ __forceinline__ bool pick_ok(const Chain<F32, VIR> &C, const Shared &sh, const Trial &t, int m)
+// A bounded wait's expiry, the same in every lane; stops the chain.
+__device__ __forceinline__ bool gave_up(const ChainArgs &a, Shared &sh, Wait &wt, int where)
 {
-    if (t.type == 1) return true;
-    const int *ns = sh.ns_ring[(m) & (kRS - 1)];
-    const WordRec &W = C.words(m);
-    int s = 0, idx = -1, possible = 1;
-    if (t.type == 0) {
-        int N = 0;
-        for (int q = 0; q < C.a.S; ++q) N += ns[q];
-        if (N == 0) {
-            possible = 0;
-        } else {
-            int k = pick_index((uint32_t)N, W.w, 0);
-            while (k >= ns[s]) {
-                k -= ns[s];
-                ++s;
-            }
-            idx = k;
-        }
-    } else {
-        s = (int)t.s;
-        if (ns[s] == 0) possible = 0;
-        else idx = pick_index((uint32_t)ns[s], W.w, 2);
-    }
-    if (possible != (int)t.possible) return false;
-    if (possible && (s != (int)t.s || idx != t.idx)) return false;
+    if (!__any_sync(0xffffffffu, wt.expired(a.wait_ns))) return false;
+    if ((threadIdx.x & 31) == 0) chain_stop(sh, kStatusTimeout, where);
+    __syncwarp();
     return true;
 }
 
-__device__ __forceinline__ void team_sync(int id, int nthreads)
+// Room in the keeper's book for move m (false: the chain stopped).
+__device__ __noinline__ bool wait_room(const ChainArgs &a, Shared &sh, int m)
 {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+    Wait wt;
+    for (;;) {
+        const int room = m < vload(sh.booked) + kRS, st = vload(sh.turn.z);
+        if (__shfl_sync(0xffffffffu, room, 0)) return true;
+        if (__shfl_sync(0xffffffffu, st, 0) || gave_up(a, sh, wt, 1)) return false;
+        __nanosleep(40);
+    }
 }
 
-// Per-team hand-off area, double-buffered by iteration parity: the
-// leader's choice of move and the particle counts its evaluation uses.
-struct TeamCtl {
-    int go[2], m[2], c0[2], pad[2];
-    int ns[2][kMaxSpecies];
+// The diagnostic stall: a bounded wait on a flag nothing sets runs out,
+// and the chain stops before this move with a timeout status.
+__device__ __noinline__ bool wait_never(const ChainArgs &a, Shared &sh)
+{
+    Wait wt;
+    for (;;) {
+        const int go = vload(sh.never), st = vload(sh.turn.z);
+        if (__shfl_sync(0xffffffffu, go, 0)) return true;
+        if (__shfl_sync(0xffffffffu, st, 0) || gave_up(a, sh, wt, 2)) return false;
+    }
+}
+
+struct Mover {
+    const ChainArgs &a;
+    Shared &sh;
+    uint16_t *cnt;
+    int4 *q;         // kQ queued pairs: separation, pair index | 0x100 for a term that counts negatively
+    int4 *tab;       // 64 work cells: record offset (2 words), flags
+    WordRec *words;  // kWords
+    uint4 *cell_pos;
+    unsigned long long R2;
+    float r2hi;
+    int lane, T, S, cap;
+    int k27;  // this lane's cell of the 27: (dx + 1) | (dy + 1) << 8 | (dz + 1) << 16
+
+    // The particle that the counts pick (Algorithm 1; idx = -1 if there is
+    // none); lane q < S holds species q's count.
+    __device__ __forceinline__ void pick(const uint32_t *w, int type, int nq, int &s, int &idx) const
+    {
+        idx = -1;
+        s = type ? (int)__umulhi(w[5], (uint32_t)S) : 0;
+        if (type == 1) return;
+        int N = __shfl_sync(0xffffffffu, nq, s);
+        if (type == 0) {
+#pragma unroll 1
+            for (int k = 1; k < S; ++k) N += __shfl_sync(0xffffffffu, nq, k);
+        }
+        if (N <= 0) return;
+        idx = pick_index((uint32_t)N, w, type);
+        if (type == 0) {
+#pragma unroll 1
+            for (;;) {
+                const int n = __shfl_sync(0xffffffffu, nq, s);
+                if (idx < n || s + 1 >= S) break;
+                idx -= n;
+                ++s;
+            }
+        }
+    }
+
+    __device__ __forceinline__ int cell_at(int x, int y, int z) const
+    {
+        return (wrapc(z, T) * T + wrapc(y, T)) * T + wrapc(x, T);
+    }
+
+    // The cells a trial visits (its work list), 0 .. n - 1: the 27 around its
+    // cell (no cell change, insertions, deletions); for a displacement into
+    // an adjacent cell the union of the old and new neighbourhoods, 3 or 4
+    // values per axis, each cell flagged kOld and/or kNew (cells of the union
+    // box in neither neighbourhood carry no flag); for a longer displacement
+    // the old 27 (kOld) followed by the new 27 (kNew).  At most 64 cells.
+    // Per axis of a union, d in {-1, 0, 1} the change of the cell: the values
+    // p - 1 - (d < 0) + i, i < 3 + |d|; boxes of three cells per side have
+    // every value in both neighbourhoods.
+    __device__ __forceinline__ int union_axis(int p, int q) const
+    {
+        int d = q - p;
+        d = d > 1 ? -1 : (d < -1 ? 1 : d);
+        return T == 3 ? 0 : d;
+    }
+    __device__ __forceinline__ void cross_cell(const Trial &t, int i, int &cell, uint32_t &fl) const
+    {
+        if (t.far) {
+            const bool nw = i >= 27;
+            const int k = nw ? i - 27 : i;
+            cell = cell_at((nw ? t.qx : t.px) + k % 3 - 1, (nw ? t.qy : t.py) + k / 3 % 3 - 1,
+                           (nw ? t.qz : t.pz) + k / 9 - 1);
+            fl = nw ? kNew : kOld;
+            return;
+        }
+        const int dx = union_axis(t.px, t.qx), dy = union_axis(t.py, t.qy), dz = union_axis(t.pz, t.qz);
+        const int r = dx ? i >> 2 : i / 3, z = dy ? r >> 2 : r / 3;
+        // offsets from the old cell
+        const int ox = i - r * (dx ? 4 : 3) - 1 - (dx < 0), oy = r - z * (dy ? 4 : 3) - 1 - (dy < 0), oz = z - 1 - (dz < 0);
+        cell = cell_at(t.px + ox, t.py + oy, t.pz + oz);
+        fl = 0;
+        if (max(max(abs(ox), abs(oy)), abs(oz)) <= 1) fl |= kOld;
+        if (max(max(abs(ox - dx), abs(oy - dy)), abs(oz - dz)) <= 1) fl |= kNew;
+        if (T == 3) fl = kOld | kNew;
+    }
+
+    // The trial's energy change.  The records of the work cells are numbered
+    // cell after cell and taken 32 at a time, one per lane; the next 32 load
+    // while the last are screened on the FP32 squared distance against a
+    // bound just above rc^2.  Pairs that pass join the queue and are
+    // evaluated 32 at a time, where the exact integer test decides, so the
+    // long pair term (FP32: compensated, lj_ff; FP64) runs with every lane
+    // busy and only on the ~15 % of records inside the cutoff.
+    template <bool P32, bool VIR>
+    __device__ __forceinline__ void evaluate(const Trial &t, Sums &o) const
+    {
+        o.e = o.el = o.ua = o.w = 0.f;
+        o.de = o.da = o.dw = 0.0;
+        if (!t.possible) return;
+        const unsigned lt = (1u << lane) - 1u;
+        // lane l owns work cells l and l + 32.  The counts are read before the
+        // records: a count covers records that are already in place.
+        int c0 = 0, c1 = 0, n0 = 0, n1 = 0, nw = 27;
+        uint32_t f0 = t.type == 0 ? (kOld | kNew) : (t.type == 1 ? kNew : kOld), f1 = 0;
+        if (!t.cross) {
+            c0 = cell_at(t.px + (k27 & 0xFF) - 1, t.py + ((k27 >> 8) & 0xFF) - 1, t.pz + (k27 >> 16) - 1);
+            if (lane >= 27) f0 = 0;
+        } else {
+            nw = t.far ? 54
+                       : (3 + (union_axis(t.px, t.qx) != 0)) * (3 + (union_axis(t.py, t.qy) != 0)) *
+                             (3 + (union_axis(t.pz, t.qz) != 0));
+            cross_cell(t, lane, c0, f0);
+            if (lane >= nw) f0 = 0;
+            if (nw > 32) {
+                cross_cell(t, lane + 32, c1, f1);
+                if (lane + 32 >= nw) f1 = 0;
+                if (f1) n1 = cload(cnt[c1]);
+            }
+        }
+        if (f0) n0 = cload(cnt[c0]);
+        fence_cta();
+        const int i0 = warp_inclusive_scan(n0);
+        int P = __shfl_sync(0xffffffffu, i0, 31);
+        const unsigned e0 = __ballot_sync(0xffffffffu, n0 > 0);
+        // where each cell's records begin (out of reach for an empty cell),
+        // and the table of the cells that have some
+        const int s0 = n0 ? i0 - n0 : INT_MAX;
+        int s1 = INT_MAX;
+        __syncwarp();
+        if (n0) {
+            const long long off = (long long)c0 * cap - s0;
+            tab[__popc(e0 & lt)] = make_int4((int)off, (int)(off >> 32), (int)f0, 0);
+        }
+        if (nw > 32) {
+            const int i1 = warp_inclusive_scan(n1) + P;
+            P = __shfl_sync(0xffffffffu, i1, 31);
+            const unsigned e1 = __ballot_sync(0xffffffffu, n1 > 0);
+            if (n1) {
+                s1 = i1 - n1;
+                const long long off = (long long)c1 * cap - s1;
+                tab[__popc(e0) + __popc(e1 & lt)] = make_int4((int)off, (int)(off >> 32), (int)f1, 0);
+            }
+        }
+        __syncwarp();
+        const uint32_t self = t.Po.w;
+        const uint4 PA = t.type == 1 ? t.Pn : t.Po;
+        const int wA = t.s * kMaxSpecies + (t.type == 1 ? 0 : 0x100), wB = t.s * kMaxSpecies;
+        const uint32_t fA = t.type == 1 ? kNew : kOld;
+        int head = 0, nq = 0, ord = -1;
+        uint4 r = make_uint4(0, 0, 0, 0);
+        uint32_t f = 0;  // flags of r (0: no record)
+        // base: first of the records being screened; those after them load
+#pragma unroll 1
+        for (int base = -32;; base += 32) {
+            // (opaque to the compiler, which would make a copy of the loop for
+            // every combination of the two)
+            int two = t.type == 0, wide = nw > 32;
+            asm volatile("" : "+r"(two), "+r"(wide));
+            uint4 rn = r;
+            uint32_t fn = 0;
+            const int nb = base + 32;
+            if (nb < P) {
+                // the cells whose records begin among these 32
+                uint32_t x = bit_at(s0 - nb);
+                if (wide) x |= bit_at(s1 - nb);
+                x = __reduce_or_sync(0xffffffffu, x);
+                const int k = ord + __popc(x & (lt * 2u + 1u));
+                ord += __popc(x);
+                if (nb + lane < P) {
+                    const int4 e = tab[k];
+                    const long long off = ((long long)e.y << 32) | (uint32_t)e.x;
+                    rn = cell_pos[off + (nb + lane)];
+                    fn = (uint32_t)e.z;
+                }
+            }
+            if (f && r.w == self) f = 0;  // the particle itself
+            {
+                const int ex = (int)(PA.x - r.x), ey = (int)(PA.y - r.y), ez = (int)(PA.z - r.z);
+                const float gx = (float)ex, gy = (float)ey, gz = (float)ez;
+                const bool in = (f & fA) && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < r2hi;
+                const unsigned b = __ballot_sync(0xffffffffu, in);
+                if (in) q[(head + nq + __popc(b & lt)) & (kQ - 1)] = make_int4(ex, ey, ez, wA + (int)tag_species(r.w));
+                nq += __popc(b);
+            }
+            if (two) {
+                const int ex = (int)(t.Pn.x - r.x), ey = (int)(t.Pn.y - r.y), ez = (int)(t.Pn.z - r.z);
+                const float gx = (float)ex, gy = (float)ey, gz = (float)ez;
+                const bool in = (f & kNew) && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < r2hi;
+                const unsigned b = __ballot_sync(0xffffffffu, in);
+                if (in) q[(head + nq + __popc(b & lt)) & (kQ - 1)] = make_int4(ex, ey, ez, wB + (int)tag_species(r.w));
+                nq += __popc(b);
+            }
+            const bool last = nb >= P;
+#pragma unroll 1
+            while (nq >= 32 || (last && nq > 0)) {
+                const int c = min(nq, 32);
+                __syncwarp();
+                if (lane < c) pair_term<P32, VIR>(q[(head + lane) & (kQ - 1)], o);
+                head += c;
+                nq -= c;
+                __syncwarp();
+            }
+            if (last) break;
+            r = rn;
+            f = fn;
+        }
+        if constexpr (P32) {
+            const FF s = ff_warp_sum(FF{o.e, o.el});
+            o.e = s.hi;
+            o.el = s.lo;
+            o.ua = warp_sum(o.ua);
+            if (VIR) o.w = warp_sum(o.w);
+        } else {
+            o.de = warp_sum(o.de);
+            o.da = warp_sum(o.da);
+            if (VIR) o.dw = warp_sum(o.dw);
+        }
+    }
+
+    // Adds one queued pair, if it is inside the cutoff.
+    template <bool P32, bool VIR>
+    __device__ __forceinline__ void pair_term(const int4 &p, Sums &o) const
+    {
+        const unsigned long long g2 = (unsigned long long)((long long)p.x * p.x) +
+                                      (unsigned long long)((long long)p.y * p.y) +
+                                      (unsigned long long)((long long)p.z * p.z);
+        if (g2 >= R2) return;
+        const int k = p.w & 0xFF;
+        const bool neg = (p.w & 0x100) != 0;
+        if constexpr (P32) {
+            const float4 c = ((const float4 *)sh.field)[k];
+            float uh, ul, m;
+            lj_ff(p.x, p.y, p.z, c.x, c.z, c.y, c.w, uh, ul, m);
+            ff_acc(o.e, o.el, neg ? -uh : uh, neg ? -ul : ul);
+            o.ua += m;
+            if (VIR) {
+                const float w = -fmaf(3.f, m, 9.f * uh);  // r U'(r) = -12 rep + 6 att
+                o.w += neg ? -w : w;
+            }
+        } else {
+            GridSep s;
+            s.dx = p.x;
+            s.dy = p.y;
+            s.dz = p.z;
+            s.g = g2;
+            double u, m;
+            lj_f64(s, a.fd.c4e[k], a.fd.sig2[k], u, m);
+            o.de += neg ? -u : u;
+            o.da += m;
+            if (VIR) {
+                const double w = 3.0 * m + 9.0 * u;
+                o.dw -= neg ? -w : w;
+            }
+        }
+    }
+
+    // The Metropolis test of Eqs. 3-5 (textbook sign of mu) in FP32 with an
+    // explicit error band, for N_s = ns: 1 accept, 0 reject, -1 inside the
+    // band or not finite (decided in FP64).
+    __device__ __forceinline__ int decide_f32(int type, int sp, int ns, float lnu, float dUf, float uab) const
+    {
+        float lnK = 0.f;
+        if (type != 0) {
+            const float z = a.lnzv_f[sp], l = logf((float)(type == 1 ? ns + 1 : ns));
+            lnK = type == 1 ? z - l : l - z;
+        }
+        const float bd = a.beta_f * dUf;
+        const float band = a.beta_f * a.tol_f * uab + 1e-6f * (1.f + fabsf(lnK) + fabsf(bd) + fabsf(lnu));
+        const float diff = lnu - (lnK - bd);
+        if (fabsf(diff) > band) return (diff < 0.f) ? 1 : 0;
+        return -1;
+    }
+
+    // Tests the trial of move m, evaluated after c0 committed moves, against
+    // the logged moves c0 .. m - 1, evaluated or committed.  Bit i of conf:
+    // move m - 1 - i, if accepted, voids the evaluation: it touches the old
+    // cell or the particle's record, or puts, removes or moves a particle
+    // within rc of the trial's old or new position (a coordinate of a record
+    // overwritten in place may be read from either value, so a move's old and
+    // new positions are tested per axis by the nearer one; an entry that a
+    // removal moved into the freed slot may be met twice by an evaluation
+    // that read the older count).  Changes farther away add nothing: their
+    // pair terms are exactly zero.  Bit i of stale: it changes what is known
+    // of the species' last particle.  ver: lane i's version of the entry of
+    // move m - 1 - i (0: not there yet).  Eight moves a pass; lane 8 k + i tests
+    // positions (k = 0, 1) or the moved entry (k = 2, 3) of the i-th against
+    // the trial's old (k even) or new (k odd) position.
+    __device__ __forceinline__ void check_logs(const Trial &t, int last_id, int last_cell, bool unborn, int c0, int m,
+                                               uint32_t &conf, uint32_t &stale, int &ver) const
+    {
+        conf = stale = 0;
+        const int k = lane >> 3;
+        const bool side = (k & 1) ? t.type != 2 : t.type != 1;
+        const uint4 P = (k & 1) ? t.Pn : t.Po;
+        const int myid = (t.s << 24) | t.idx;
+#pragma unroll 1
+        for (int b = 0; b < m - c0; b += 8) {
+            const int i = b + (lane & 7), j = m - 1 - i;
+            bool bad = false, old = false;
+            int v = 0;
+            if (j >= c0) v = vload(sh.ver[j & (kRS - 1)]);
+            fence_cta();
+            if ((v >> 8) == (j & 0x7FFFFF) && v != 0 && j >= c0) {
+                const LogRec &L = sh.logs[j & (kRS - 1)];
+                const uint4 p0 = L.pos0;
+                const uint4 X0 = k < 2 ? p0 : L.moved, X1 = k < 2 && (p0.w & 1u) ? L.pos1 : X0;
+                if (k == 0) {
+                    const int4 id = L.ids;
+                    bad = t.type != 1 && (id.x == t.co || id.y == t.co || id.z == myid || id.w == myid ||
+                                          (unborn && (p0.w & 4u) && (int)(p0.w >> 8) == t.s));
+                    old = id.x == last_cell || id.y == last_cell || id.z == last_id || id.w == last_id;
+                }
+                const float dx = (float)min(axis_dist(X0.x, P.x), axis_dist(X1.x, P.x)),
+                            dy = (float)min(axis_dist(X0.y, P.y), axis_dist(X1.y, P.y)),
+                            dz = (float)min(axis_dist(X0.z, P.z), axis_dist(X1.z, P.z));
+                if (side && (k < 2 || (p0.w & 2u)) && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < r2hi) bad = true;
+            } else {
+                v = 0;
+            }
+            unsigned x = __ballot_sync(0xffffffffu, bad);
+            x |= x >> 16;
+            conf |= ((x | (x >> 8)) & 0xFFu) << b;
+            stale |= (__ballot_sync(0xffffffffu, old) & 0xFFu) << b;
+            if ((lane & ~7) == b) ver = v;
+        }
+    }
+
+    // The particle counts at the turn of move m, predicted after c committed
+    // moves: an insertion or deletion evaluated and likely accepted, or not
+    // yet evaluated and of a kind this chain mostly accepts, counts +1 or -1
+    // for its species (the movers post this outlook).  Lane q < S gets
+    // species q's count.
+    __device__ __forceinline__ int predict_counts(int c, int m, int &now) const
+    {
+        int code = 0;
+        const int k = c + lane;
+        if (k < m) {
+            const int o = vload(sh.outlook[k & (kRS - 1)]);
+            if ((o >> 8) == (k & 0x7FFFFF)) code = o & 0xFF;
+        }
+        now = lane < S ? vload(sh.n[lane]) : 0;
+        int n = now;
+#pragma unroll 1
+        for (int s = 0; s < S; ++s) {
+            const int d = __popc(__ballot_sync(0xffffffffu, code == ((s << 2) | 1))) -
+                          __popc(__ballot_sync(0xffffffffu, code == ((s << 2) | 2)));
+            if (lane == s) n += d;
+        }
+        return (int)min((long long)max(n, 0), a.maxN);
+    }
+
 };
 
-// NTEAM teams of G evaluator warps, the committer (warp 0) and the keeper
-// (warp 4).  Team k evaluates moves k, k + NTEAM, k + 2 NTEAM, ..., each as
-// soon as fewer than LOOK moves separate it from the committer; a move the
-// committer finds invalid is evaluated again by the first team free to take
-// it, ahead of that team's new moves.  KU: slots per work cell a lane loads
-// at once.
-template <bool F32, bool VIR, int G, int NTEAM, int LOOK, int KU, bool PROF>
+// FP64 evaluation of a trial inside the FP32 error band.
+template <bool VIR>
+__device__ __noinline__ Sums evaluate64(Mover M, Trial t)
+{
+    Sums d;
+    M.template evaluate<false, VIR>(t, d);
+    return d;
+}
+
+template <bool F32, bool VIR, bool PROF>
+__device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint16_t *cnt, unsigned char *mine, int warp)
+{
+    const int lane = threadIdx.x & 31, n = a.n_moves, W = a.movers;
+    Mover M{a, sh, cnt, (int4 *)mine, (int4 *)(mine + kQ * 16), (WordRec *)(mine + kQ * 16 + 64 * 16), a.cell_pos, a.R2,
+            a.r2hi, lane, a.T, a.S, a.cap, lane % 3 | (lane / 3 % 3) << 8 | (lane / 9) << 16};
+    const int S = M.S;
+    unsigned long long c_eval = 0, c_room = 0, c_wait = 0, c_logs = 0, c_pick = 0, c_dec = 0, c_app = 0, c_book = 0,
+                       c_all = 0;
+    long long n_eval = 0;
+    int it = 0;
+#pragma unroll 1
+    for (int m = warp; m < n; m += W, ++it) {
+        if ((it & (kWords - 1)) == 0) fill_words(a, M.words, m, lane);
+        const WordRec &WR = M.words[it & (kWords - 1)];
+        uint32_t w[8];
+        {
+            const uint4 x = ((const uint4 *)WR.w)[0], y = ((const uint4 *)WR.w)[1];
+            w[0] = x.x; w[1] = x.y; w[2] = x.z; w[3] = x.w;
+            w[4] = y.x; w[5] = y.y; w[6] = y.z; w[7] = y.w;
+        }
+        const int type = w[0] < a.thr_disp ? 0 : (w[0] < a.thr_ins ? 1 : 2);
+        const int slot = m & (kRS - 1), mtag = (m & 0x7FFFFF) << 8;
+        if (type && lane == 0) {
+            // a bet for the predictions of later moves, until the evaluation is in
+            const int code = vload(sh.likely[type - 1]) ? ((int)__umulhi(w[5], (uint32_t)S) << 2) | type : 0;
+            vstore(sh.outlook[slot], mtag | code);
+        }
+        bool need64 = false;
+#pragma unroll 1
+        for (int attempt = 1;; ++attempt) {
+            // ------------------------------------------------ evaluate
+            const unsigned long long t0 = prof_clock<PROF>();
+            const int4 v0 = turn_load(sh);
+            const int c0 = __shfl_sync(0xffffffffu, v0.x, 0);
+            if (__shfl_sync(0xffffffffu, v0.z, 0)) goto done;
+            fence_cta();
+            // lane q < S: the count of species q now, and the one the evaluation assumes
+            int now;
+            const int nq = M.predict_counts(c0, m, now);
+            Trial t;
+            M.pick(w, type, nq, t.s, t.idx);
+            const int s = t.s, idx = t.idx;
+            const int nref = __shfl_sync(0xffffffffu, nq, s);  // N_s assumed
+            const int nnow = __shfl_sync(0xffffffffu, now, s);
+            const bool unborn = idx >= nnow;  // a pending insertion's particle
+            t.type = type;
+            t.possible = type == 1 || idx >= 0;
+            t.cross = t.far = false;
+            t.co = t.cn = -1;
+            t.Po = make_uint4(0, 0, 0, 0xFFFFFFFFu);
+            t.Pn = make_uint4(0, 0, 0, 0);
+            // the old cell's count, and its entry `lane`; for a deletion the
+            // species' last particle, which will take the freed index
+            int nco = 0, qcell = -1, last_id = -1, qn = 0;
+            uint4 lastv = make_uint4(0, 0, 0, 0), Q = lastv;
+            uint32_t qtag = 0;
+            if (t.possible) {
+                if (type != 1) {
+                    // the records in lanes 0 (the particle) and 1 (the last one)
+                    uint4 r = make_uint4(0, 0, 0, 0);
+                    if (lane < (type == 2 ? 2 : 1)) r = a.pos_by_id[(long long)s * a.maxN + (lane ? nref - 1 : idx)];
+                    t.Po.x = __shfl_sync(0xffffffffu, r.x, 0);
+                    t.Po.y = __shfl_sync(0xffffffffu, r.y, 0);
+                    t.Po.z = __shfl_sync(0xffffffffu, r.z, 0);
+                    t.Po.w = __shfl_sync(0xffffffffu, r.w, 0);
+                    if (type == 2 && idx != nref - 1 && nref <= nnow) {  // (a particle that is there)
+                        last_id = (s << 24) | (nref - 1);
+                        Q.x = __shfl_sync(0xffffffffu, r.x, 1);
+                        Q.y = __shfl_sync(0xffffffffu, r.y, 1);
+                        Q.z = __shfl_sync(0xffffffffu, r.z, 1);
+                        Q.w = __shfl_sync(0xffffffffu, r.w, 1);
+                        qcell = cell_of(Q.x, Q.y, Q.z, M.T);
+                    }
+                    t.px = cell_coord(t.Po.x, (uint32_t)M.T);
+                    t.py = cell_coord(t.Po.y, (uint32_t)M.T);
+                    t.pz = cell_coord(t.Po.z, (uint32_t)M.T);
+                    t.co = (t.pz * M.T + t.py) * M.T + t.px;
+                    nco = __shfl_sync(0xffffffffu, cload(cnt[t.co]), 0);
+                    if (qcell >= 0) qn = __shfl_sync(0xffffffffu, cload(cnt[qcell]), 0);
+                    fence_cta();
+                    if (lane < nco) lastv = M.cell_pos[(long long)t.co * M.cap + lane];
+                    if (lane < qn) qtag = M.cell_pos[(long long)qcell * M.cap + lane].w;
+                }
+                if (type == 0) {
+                    t.Pn.x = t.Po.x + (uint32_t)((int)__umulhi(w[2], a.span) - a.D);
+                    t.Pn.y = t.Po.y + (uint32_t)((int)__umulhi(w[3], a.span) - a.D);
+                    t.Pn.z = t.Po.z + (uint32_t)((int)__umulhi(w[4], a.span) - a.D);
+                } else if (type == 1) {
+                    t.Pn = make_uint4(w[2], w[3], w[4], 0u);
+                }
+                if (type != 2) {
+                    t.qx = cell_coord(t.Pn.x, (uint32_t)M.T);
+                    t.qy = cell_coord(t.Pn.y, (uint32_t)M.T);
+                    t.qz = cell_coord(t.Pn.z, (uint32_t)M.T);
+                    t.cn = (t.qz * M.T + t.qy) * M.T + t.qx;
+                    if (type == 1) {
+                        t.px = t.qx;
+                        t.py = t.qy;
+                        t.pz = t.qz;
+                    } else {
+                        t.cross = t.co != t.cn;
+                        t.far = t.cross && !(near1(t.px - t.qx, M.T) && near1(t.py - t.qy, M.T) && near1(t.pz - t.qz, M.T));
+                    }
+                }
+            }
+            Sums E;
+            M.template evaluate<F32, VIR>(t, E);
+            ++n_eval;
+            // the slots of the particle and of the species' last one
+            int self_slot = -1, qslot = -1;
+            if (type != 1) {
+                const unsigned hit = __ballot_sync(0xffffffffu, lane < nco && lastv.w == t.Po.w);
+                if (nco <= 32) {
+                    self_slot = __ffs(hit) - 1;
+                } else {
+                    const Found x = find_far(M.cell_pos + (long long)t.co * M.cap, t.Po.w, nco, lastv, lane);
+                    self_slot = x.at;
+                    lastv = x.last;
+                }
+                if (qn > 0) {
+                    const unsigned hq = __ballot_sync(0xffffffffu, lane < qn && qtag == Q.w);
+                    qslot = __ffs(hq) - 1;  // -1: looked up at the turn
+                }
+            }
+            const bool has_last = (type == 2 || t.cross) && self_slot != nco - 1;
+            const bool last_mine = has_last && lane == ((nco - 1) & 31);
+            // the decision and the pick for each count N_s = nref - 16 + lane
+            // its turn can meet (at most kMaxMovers - 1 moves are pending)
+            uint32_t acc_mask, band_mask, same_mask;
+            {
+                const int nl = nref - 16 + lane;
+                const float dUf = F32 ? E.e + E.el : __double2float_rn(E.de), uab = F32 ? E.ua : __double2float_rn(E.da);
+                const int dec = t.possible && nl >= 0 ? M.decide_f32(type, s, nl, WR.lnu, dUf, uab) : 0;
+                bool same = true;
+                if (type == 2 || (type == 0 && S == 1))
+                    same = nl > 0 ? (idx >= 0 && pick_index((uint32_t)nl, w, type) == idx) : idx < 0;
+                acc_mask = __ballot_sync(0xffffffffu, dec > 0);
+                band_mask = __ballot_sync(0xffffffffu, dec < 0);
+                same_mask = __ballot_sync(0xffffffffu, same);
+            }
+            // FP32 mode: a trial inside the band is evaluated in FP64 too
+            bool have64 = !F32;
+            if constexpr (F32) {
+                if (need64 || ((band_mask >> 16) & 1u)) {
+                    const Sums d = evaluate64<VIR>(M, t);
+                    E.de = d.de;
+                    E.da = d.da;
+                    E.dw = d.dw;
+                    have64 = true;
+                }
+            }
+            // what later moves need to know
+            {
+                LogRec &L = sh.logs[slot];
+                if (attempt > 1) {
+                    if (lane == 0) vstore(sh.ver[slot], 0);
+                    fence_cta();
+                    __syncwarp();
+                }
+                if (last_mine) L.moved = lastv;
+                if (lane == 0) {
+                    L.ids = make_int4(type == 1 ? t.cn : t.co, t.cross ? t.cn : qcell, type == 1 ? -1 : (s << 24) | idx,
+                                      last_id);
+                    const uint4 p = type == 1 ? t.Pn : t.Po;
+                    L.pos0 = make_uint4(p.x, p.y, p.z,
+                                        (type == 0 ? 1u : 0u) | (has_last ? 2u : 0u) | (type == 1 ? 4u : 0u) | ((uint32_t)s << 8));
+                    L.pos1 = t.Pn;
+                    if (type) vstore(sh.outlook[slot], mtag | (((acc_mask >> 16) & 1u) ? (s << 2) | type : 0));
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    fence_cta();
+                    vstore(sh.ver[slot], mtag | (attempt & 0x7F) | 0x80);
+                }
+            }
+            const unsigned long long t1 = prof_clock<PROF>();
+            c_eval += t1 - t0;
+            // ------------------------------------------------ wait for the turn
+            if (m >= __shfl_sync(0xffffffffu, vload(sh.booked), 0) + kRS && !wait_room(a, sh, m)) goto done;
+            const unsigned long long t2 = prof_clock<PROF>();
+            c_room += t2 - t1;
+            // tested against the moves before it while it waits
+            uint32_t conf = 0, stale = 0;
+            int ver = 0, seen = c0;
+            int4 v;
+            bool again = false;
+            {
+                Wait wt;
+                const bool mine_i = lane < m - c0;
+                const int vi = (m - 1 - lane) & (kRS - 1);
+#pragma unroll 1
+                for (;;) {
+                    v = turn_load(sh);
+                    if (__all_sync(0xffffffffu, v.x == m && v.z == 0)) break;
+                    const int c = __shfl_sync(0xffffffffu, v.x, 0);
+                    if (__shfl_sync(0xffffffffu, v.z, 0)) goto done;
+                    if (c < m && t.possible) {
+                        const uint32_t hist = (uint32_t)__shfl_sync(0xffffffffu, v.y, 0) << (m - c);
+                        fence_cta();
+                        // entries that are new since they were tested: tested
+                        // once their move is committed and accepted, or near the turn
+                        const uint32_t fresh = __ballot_sync(0xffffffffu, mine_i && vload(sh.ver[vi]) != ver);
+                        if ((fresh & hist) || (fresh && m - c <= 2))
+                            M.check_logs(t, last_id, qcell, unborn, c0, m, conf, stale, ver);
+                        if (c != seen) {
+                            seen = c;
+                            wt = Wait();
+                            if (conf & hist) again = true;
+                            // the pick for the counts as now predicted
+                            if (same_mask != 0xffffffffu) {
+                                int x;
+                                const int i = __shfl_sync(0xffffffffu, M.predict_counts(c, m, x), s) - nref + 16;
+                                if (i < 0 || i > 31 || !((same_mask >> i) & 1u)) again = true;
+                            }
+                            if (again) break;
+                            continue;
+                        }
+                    }
+                    if (gave_up(a, sh, wt, 2)) goto done;
+                    if (m - c > 2) __nanosleep(20 * (m - c - 1));
+                }
+            }
+            if (again) {
+                c_wait += prof_clock<PROF>() - t2;
+                continue;  // evaluate again, before the turn
+            }
+            // ------------------------------------------------ the turn
+            if (m == a.stall_at && !wait_never(a, sh)) goto done;
+            fence_cta();
+            const unsigned long long t3 = prof_clock<PROF>();
+            c_wait += t3 - t2;
+            const int ns = vload(sh.n[s]);
+            const int c_n = t.cn >= 0 ? cload(cnt[t.cn]) : 0;
+            const uint32_t hist = (uint32_t)v.y & ((1u << (m - c0)) - 1u);  // m - c0 < kRS
+            if (t.possible) {
+                const uint32_t fresh = __ballot_sync(0xffffffffu, lane < m - c0 && vload(sh.ver[(m - 1 - lane) & (kRS - 1)]) != ver);
+                if (fresh & hist) M.check_logs(t, last_id, qcell, unborn, c0, m, conf, stale, ver);
+            }
+            const unsigned long long t4 = prof_clock<PROF>();
+            c_logs += t4 - t3;
+            const int i = ns - nref + 16;
+            bool valid = !(conf & hist) && i >= 0 && i <= 31 && ((same_mask >> (i & 31)) & 1u);
+            if (type == 0 && S > 1) {
+                // several counts decide the pick: the same counts, or the same pick
+                const int cur = lane < S ? vload(sh.n[lane]) : 0;
+                if (!__all_sync(0xffffffffu, lane >= S || cur == nq)) {
+                    int s2, i2;
+                    M.pick(w, 0, cur, s2, i2);
+                    valid = !(conf & hist) && i2 == idx && (idx < 0 || s2 == s);
+                }
+            }
+            const int ii = type == 0 ? 16 : (i & 31);  // a displacement's decision does not depend on the counts
+            const bool in_band = (band_mask >> ii) & 1u;
+            const unsigned long long t5 = prof_clock<PROF>();
+            c_pick += t5 - t4;
+            if (!valid || (in_band && !have64)) {
+                // an evaluation that began at the turn stands, unless FP64 is wanted
+                if (c0 == m && !valid) {
+                    if (lane == 0) chain_stop(sh, kStatusBadInput, 8);
+                    goto done;
+                }
+                need64 = need64 || in_band;
+                continue;
+            }
+            // the Metropolis test in FP32 with an error band, inside it in FP64
+            int bits = (((acc_mask >> ii) & 1u) ? kBkAcc : 0) | (attempt > 1 ? kBkAgain : 0) | (F32 ? 0 : kBkUse64);
+            double lnA = 0.0;
+            if (in_band) {
+                const Decision d = decide_f64(a, w[6], w[7], type, s, ns, E.de, E.da);
+                lnA = d.lnA;
+                bits = (bits & ~kBkAcc) | kBkUse64 | kBkRefined | d.bits;
+            }
+            const bool fin = bits & kBkAcc;
+            if (fin) {
+                int stop_bits = 0;
+                if (type != 2 && (type == 1 || t.cross) && c_n >= M.cap) stop_bits = kStatusCellOverflow;
+                if (type == 1 && ns >= a.maxN) stop_bits = kStatusCapacity;
+                if (type != 1 && self_slot < 0) stop_bits = kStatusBadInput;  // a record missing from its cell
+                if (stop_bits) {
+                    if (lane == 0) chain_stop(sh, stop_bits, 16);
+                    goto done;
+                }
+            }
+            const unsigned long long t6 = prof_clock<PROF>();
+            c_dec += t6 - t5;
+            // ------------------------------------------------ apply (Sec. 3.2.5)
+            if (fin) {
+                uint4 *by_id = a.pos_by_id + (long long)s * a.maxN;
+                uint4 *old_cell = M.cell_pos + (long long)t.co * M.cap;
+                bool both = false;
+                uint32_t ntag = t.Po.w;
+                if (type == 2) {
+                    // swap-with-last inside the cell, then the species' last
+                    // index takes the freed index (its record and its cell entry)
+                    const int last = ns - 1;
+                    ntag = make_tag((uint32_t)idx, (uint32_t)s);
+                    if (idx != last) {
+                        // known from the evaluation unless a later move touched it
+                        if (last_id != ((s << 24) | last) || (stale & hist) || qslot < 0) {
+                            const Entry x = find_now(a, cnt, s, last, lane);
+                            Q = x.Q;
+                            qcell = x.cell;
+                            qslot = x.slot;
+                            if (lane == 0) {
+                                sh.logs[slot].ids.y = qcell;
+                                sh.logs[slot].ids.w = (s << 24) | last;
+                                fence_cta();
+                                vstore(sh.ver[slot], mtag | 0x7F);  // later moves test it again
+                            }
+                            if (qslot < 0) {
+                                if (lane == 0) chain_stop(sh, kStatusBadInput, 32);
+                                goto done;
+                            }
+                        }
+                        // the last particle may be the entry that moves into the freed slot
+                        both = qcell == t.co && qslot == nco - 1;
+                        if (lane == 0) {
+                            if (!both) M.cell_pos[(long long)qcell * M.cap + qslot].w = ntag;
+                            by_id[idx] = make_uint4(Q.x, Q.y, Q.z, ntag);
+                        }
+                    }
+                } else if (lane == 0) {
+                    const bool move_in = type == 1 || t.cross;
+                    if (type == 1) ntag = make_tag((uint32_t)ns, (uint32_t)s);
+                    const uint4 r = make_uint4(t.Pn.x, t.Pn.y, t.Pn.z, ntag);
+                    M.cell_pos[(long long)t.cn * M.cap + (move_in ? c_n : self_slot)] = r;
+                    by_id[type == 1 ? ns : idx] = r;
+                }
+                if (last_mine) {
+                    if (both) lastv.w = ntag;
+                    old_cell[self_slot] = lastv;
+                }
+                __syncwarp();
+                if (lane == 0 && (type != 0 || t.cross)) {
+                    fence_cta();  // the records before the counts that cover them
+                    if (type != 1) cstore(cnt[t.co], nco - 1);
+                    if (type != 2) cstore(cnt[t.cn], c_n + 1);
+                    if (type != 0) vstore(sh.n[s], type == 1 ? ns + 1 : ns - 1);
+                }
+            }
+            const unsigned long long t7 = prof_clock<PROF>();
+            c_app += t7 - t6;
+            // ------------------------------------------------ pass the turn on
+            if (lane == 0) {
+                fence_cta();  // the move's writes before the turn that says they are there
+                turn_store(sh, m + 1, ((uint32_t)v.y << 1) | (fin ? 1u : 0u));
+                BookRec &B = sh.book[slot];
+                B.dU64 = E.de;
+                B.lnA = lnA;
+                B.dW = VIR ? (F32 && !in_band ? (double)E.w : E.dw) : 0.0;
+                B.hi = E.e;
+                B.lo = E.el;
+                B.uab = F32 && !in_band ? E.ua : (float)E.da;
+                B.bits = bits | (t.possible ? kBkPossible : 0) | (type << 8) | (s << 16);
+                B.index = type == 1 ? ns : idx;
+                B.n = ns;
+                fence_cta();
+                vstore(B.ready, m + 1);
+            }
+            __syncwarp();
+            const unsigned long long t8 = prof_clock<PROF>();
+            c_book += t8 - t7;
+            c_all += t8 - t1;
+            break;
+        }
+    }
+done:
+    __syncwarp();
+    if (lane == 0) {
+        fence_cta();
+        atomicAdd(&sh.gone, 1);
+        atomicAdd((unsigned long long *)&sh.evaluations, (unsigned long long)n_eval);
+        if constexpr (PROF) {
+            atomicAdd(&sh.prof[0], c_wait);
+            atomicAdd(&sh.prof[1], c_logs + c_pick);
+            atomicAdd(&sh.prof[2], c_dec);
+            atomicAdd(&sh.prof[3], c_app);
+            atomicAdd(&sh.prof[4], c_all);
+            atomicAdd(&sh.prof[5], c_room);
+            atomicAdd(&sh.prof[6], c_eval);
+            atomicAdd(&sh.prof[9], c_logs);
+            atomicAdd(&sh.prof[10], c_pick);
+            atomicAdd(&sh.prof[11], c_book);
+        }
+    }
+}
+
+// The keeper: books the committed moves in order.
+template <bool VIR>
+__device__ void keeper_loop(const ChainArgs &a, Shared &sh)
+{
+    const int lane = threadIdx.x & 31, n = a.n_moves;
+    double E = *a.d_energy, sumE = 0.0;
+    // the running virial, for the chains of the launch that keep it
+    const bool vir = VIR && a.virial;
+    double Wv = vir ? a.d_energy[1] : 0.0, sumW = 0.0;
+    long long sumN = 0, att0 = 0, att1 = 0, att2 = 0, acc0 = 0, acc1 = 0, acc2 = 0;
+    long long flagged = 0, reeval = 0, refines = 0, Ncur = 0;
+    for (int k = 0; k < kMaxSpecies; ++k) Ncur += k < a.S ? a.d_n[k] : 0;
+    int mb = 0;
+    Wait wt;
+    while (mb < n) {
+        const int rdy = vload(sh.book[mb & (kRS - 1)].ready);
+        if (__shfl_sync(0xffffffffu, rdy, 0) == mb + 1) {
+            fence_cta();
+            if (lane == 0) {
+                const BookRec &B = sh.book[mb & (kRS - 1)];
+                const int bits = B.bits, type = (bits >> 8) & 0xFF, sp = bits >> 16;
+                const bool acc = bits & kBkAcc;
+                att0 += type == 0;
+                att1 += type == 1;
+                att2 += type == 2;
+                if (bits & kBkNear) ++flagged;
+                if (bits & kBkRefined) ++refines;
+                if (bits & kBkAgain) ++reeval;
+                const double dU = (bits & kBkUse64) ? B.dU64 : (double)B.hi + (double)B.lo;
+                if (acc) {
+                    acc0 += type == 0;
+                    acc1 += type == 1;
+                    acc2 += type == 2;
+                    E += dU;
+                    Wv += B.dW;
+                    Ncur += (type == 1) - (type == 2);
+                }
+                if (type == 1) vstore(sh.likely[0], 2 * acc1 > att1);
+                else if (type == 2) vstore(sh.likely[1], 2 * acc2 > att2);
+                if (a.trace) {
+                    const bool possible = bits & kBkPossible;
+                    gcmc_trace tr;
+                    double lnA = B.lnA;
+                    if (!(bits & kBkRefined)) {
+                        double lnK = 0.0;
+                        if (type == 1) lnK = a.logz[sp] + a.lnV - log((double)(B.n + 1));
+                        else if (type == 2 && B.n > 0) lnK = log((double)B.n) - a.logz[sp] - a.lnV;
+                        lnA = possible ? lnK - a.beta * dU : -INFINITY;
+                    }
+                    tr.dU = possible ? dU : 0.0;
+                    tr.lnA = lnA;
+                    tr.uabs = possible ? (double)B.uab : 0.0;
+                    tr.index = B.index;
+                    tr.type = (uint8_t)type;
+                    tr.species = (uint8_t)sp;
+                    tr.accepted = (uint8_t)acc;
+                    tr.flagged = (uint8_t)(((bits & kBkNear) ? 1 : 0) | ((bits & kBkRefined) ? 2 : 0));
+                    a.trace[mb] = tr;
+                }
+                sumE += E;
+                sumW += Wv;
+                sumN += Ncur;
+                fence_cta();
+                vstore(sh.booked, mb + 1);
+            }
+            __syncwarp();
+            ++mb;
+            wt = Wait();
+            continue;
+        }
+        // a stopped chain may still commit the move that held the turn: its
+        // last move is known once every mover has finished
+        const int gone = vload(sh.gone);
+        fence_cta();
+        const int4 v = turn_load(sh);
+        if (__shfl_sync(0xffffffffu, v.z && gone == a.movers && mb >= v.x, 0)) break;
+        if (__any_sync(0xffffffffu, wt.expired(a.wait_ns))) {
+            if (lane == 0) chain_stop(sh, kStatusTimeout, 4);
+            break;
+        }
+        __nanosleep(40);
+    }
+    if (lane == 0) {
+        ChainOut &o = *a.out;
+        o.attempted[0] = att0;
+        o.attempted[1] = att1;
+        o.attempted[2] = att2;
+        o.accepted[0] = acc0;
+        o.accepted[1] = acc1;
+        o.accepted[2] = acc2;
+        o.flagged = flagged;
+        o.moves_done = mb;
+        o.energy = E;
+        o.sum_energy = sumE;
+        o.sum_n = (double)sumN;
+        o.reevaluated = reeval;
+        o.refines = refines;
+        o.virial = vir ? Wv : NAN;
+        o.sum_virial = vir ? sumW : NAN;
+        *a.d_energy = E;
+        if (vir) a.d_energy[1] = Wv;
+    }
+}
+
+template <bool F32, bool VIR, bool PROF>
 __global__ void __launch_bounds__(kChainWarps * 32, 1) k_chain(const ChainArgs *__restrict__ args)
 {
-    static_assert(G <= kGMax && LOOK < kRS && NTEAM <= 15, "team shape");
-    constexpr int EW = G * NTEAM;
-    constexpr int NW = kChainWarps;
-    constexpr int NTH = NW * 32;
-    static_assert(EW + 2 <= NW && EW <= kMaxEW, "team shape");
-    // dynamic shared memory: the evaluator warps' pair-term queues (FP32
-    // runs), then the cell counters
+    constexpr int NTH = kChainWarps * 32;
+    // dynamic shared memory: each mover's queue and words, then the cell counters
     extern __shared__ __align__(16) unsigned char dyn[];
-    int4 *fq = (int4 *)dyn;
-    uint16_t *cnt = (uint16_t *)(dyn + (F32 ? kMaxEW * kQ * sizeof(int4) : 0));
     unsigned long long t_start = 0;
     if (threadIdx.x == 0) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_start));
     __shared__ Shared sh;
-    __shared__ TeamCtl ctl[NTEAM];
-    __shared__ int redo;  // move + 1 to evaluate again (the first free team takes it), 0 none
-    __shared__ unsigned long long team_cyc[3];  // leaders' idle cycles, evaluation cycles, evaluations
     // this CTA's chain: its arguments copied to shared memory
     __shared__ __align__(16) ChainArgs a;
+    const int tid = threadIdx.x, warp = tid >> 5;
     {
         const uint32_t *src = (const uint32_t *)(args + blockIdx.x);
         uint32_t *dst = (uint32_t *)&a;
-        for (int k = threadIdx.x; k < (int)(sizeof(ChainArgs) / 4); k += NTH) dst[k] = src[k];
+        for (int k = tid; k < (int)(sizeof(ChainArgs) / 4); k += NTH) dst[k] = src[k];
         __syncthreads();
     }
     if (a.n_moves <= 0) {
-        if (threadIdx.x == 0) {
+        if (tid == 0) {
             ChainOut &o = *a.out;
             o.moves_done = 0;
             o.energy = *a.d_energy;
-            for (int q = 0; q < kMaxSpecies; ++q) o.n[q] = q < a.S ? a.d_n[q] : 0;
+            for (int k = 0; k < kMaxSpecies; ++k) o.n[k] = k < a.S ? a.d_n[k] : 0;
             o.status = 0;
         }
         return;
     }
-    Chain<F32, VIR> C(a, sh, cnt, fq);
-    const int tid = threadIdx.x, lane = C.lane, warp = C.warp, T = C.T;
-    const int n = a.n_moves;
-    // Roles by warp.  Warp w runs on the SM sub-partition w % 4, so the
-    // committer (warp 0), whose every step is on the chain's critical path,
-    // shares its sub-partition's issue slots with the keeper (warp 4, mostly
-    // asleep) and at most two evaluator warps (8 and 12, only for teams of
-    // more than 12 warps); the evaluators fill the other sub-partitions first.
-    const int keeper_warp = 4;
-    int eid = -1;
-    if (warp & 3) eid = (warp >> 2) * 3 + (warp & 3) - 1;
-    else if (warp == 8 || warp == 12) eid = 12 + (warp >> 2) - 2;
-    if (eid >= EW) eid = -1;
-    C.eidx = eid;
-
+    uint16_t *cnt = (uint16_t *)(dyn + (size_t)a.movers * kMoverBytes);
     for (int c = tid; c < a.ncell; c += NTH) cnt[c] = (uint16_t)a.cell_count[c];
-    if (tid < kMaxSpecies) {
-        const long long v = tid < a.S ? a.d_n[tid] : 0;
-        sh.n[tid] = v;
-        sh.ln_n[tid] = logf((float)v);
-        sh.ln_n1[tid] = logf((float)(v + 1));
-        sh.ns_ring[0][tid] = (int)v;
+    if (tid < kMaxSpecies) sh.n[tid] = tid < a.S ? (int)a.d_n[tid] : 0;
+    if (tid < kRS) {
+        sh.book[tid].ready = 0;
+        sh.outlook[tid] = -1;
+        sh.ver[tid] = 0;
     }
-    for (int k = tid; k < kRS; k += NTH) {
-        sh.slots[k].tag = 0;
-        sh.slots[k].tpub = 0;
-        sh.slots[k].arrive = 0;
-        sh.book[k].ready = 0;
-        sh.logs[k].head.x = 0;
+    for (int k = tid; k < kMaxSpecies * kMaxSpecies; k += NTH) {
+        if constexpr (F32) ((float4 *)sh.field)[k] = make_float4(a.ff.c4e[k], a.ff.sig2[k], a.ff.c4e_lo[k], a.ff.sig2_lo[k]);
+        else sh.field[k] = make_double2(a.fd.c4e[k], a.fd.sig2[k]);
     }
-    if (tid == 0) redo = 0;
-    if (tid < 3) team_cyc[tid] = 0ull;
+    if (tid < 12) sh.prof[tid] = 0ull;
     if (tid == 0) {
-        sh.committed = 0;
-        sh.booked = 0;
-        sh.stop = 0;
-        sh.status = 0;
-        sh.where = 0;
-        sh.seq = 0;
+        sh.turn = make_int4(0, 0, 0, 0);
+        sh.booked = sh.status = sh.where = sh.gone = sh.never = 0;
         sh.likely[0] = sh.likely[1] = 0;
-        sh.never = 0;
-        sh.nacc = 0;
-    }
-    {
-        const int first_fill = min(n, kRW);
-        for (int b = warp; b * kFill < first_fill; b += NW)
-            C.fill_words(b * kFill, min(kFill, first_fill - b * kFill));
-        if (tid == 0) sh.filled = first_fill;
+        sh.evaluations = 0;
     }
     __syncthreads();
-
-    if (eid >= 0) {
-        // ------------------------------------------------------------ evaluators
-        const int team = eid / G, j = eid % G;
-        TeamCtl &tc = ctl[team];
-        int next = team;  // the team's next new move (leader lane 0)
-        unsigned long long cyc_idle = 0, cyc_eval = 0, n_eval = 0;  // leader lane of warp j == 0
-        for (int it = 0;; ++it) {
-            const int p = it & 1;
-            if (j == 0 && lane == 0) {
-                const unsigned long long ti = prof_clock<PROF>();
-                Wait wt;
-                int go = 0, mm = 0, c0 = 0, acc0 = 0;
-                for (;;) {
-                    if (vload(sh.stop)) {
-                        go = 2;
-                        break;
-                    }
-                    // the accepted count is read before the commit count, so
-                    // that it never covers a commit the evaluation did not see
-                    const int acc_seen = vload(sh.nacc);
-                    __threadfence_block();
-                    const int com = vload(sh.committed);
-                    const int rd = vload(redo);
-                    const bool fresh = next < n && next < com + LOOK && next < vload(sh.filled);
-                    if (rd || fresh) {
-                        // the counts after `com` commits (the ring entry stays
-                        // until com + kRS - 1 moves are committed)
-                        for (int q = 0; q < a.S; ++q) tc.ns[p][q] = sh.ns_ring[(com) & (kRS - 1)][q];
-                        __threadfence_block();
-                        if (vload(sh.committed) < com + kRS - 1) {
-                            // a re-evaluation goes to the first team free to
-                            // take it, ahead of the team's new move
-                            if (rd && atomicCAS(&redo, rd, 0) == rd) {
-                                mm = rd - 1;
-                            } else if (fresh) {
-                                mm = next;
-                                next += NTEAM;
-                            } else {
-                                continue;
-                            }
-                            c0 = com;
-                            acc0 = acc_seen;
-                            go = 1;
-                            break;
-                        }
-                        continue;
-                    }
-                    if (next >= n && com >= n) {
-                        go = 2;
-                        break;
-                    }
-                    if (wt.expired(a.wait_ns)) {
-                        atomicOr(&sh.status, kStatusTimeout);
-                        atomicOr(&sh.where, 1);
-                        vstore(sh.stop, 1);
-                        go = 2;
-                        break;
-                    }
-                    __nanosleep(16);
-                }
-                if (go == 1) {
-                    Slot &S = sh.slots[(mm) & (kRS - 1)];
-                    S.self_slot = -1;
-                    S.has_last = 0;
-                    S.arrive = 0;
-                    S.tpub = 0;
-                    S.c0 = c0;
-                    S.acc0 = acc0;
-                    __threadfence_block();
-                    vstore(S.tag, mm + 1);
-                }
-                tc.go[p] = go;
-                tc.m[p] = mm;
-                tc.c0[p] = c0;
-                __threadfence_block();
-                cyc_idle += prof_clock<PROF>() - ti;
-            }
-            __syncwarp();
-            if (j == 0) {
-                // predicted counts at the move's turn: lane i looks at the
-                // pending move c0 + i; an insertion or deletion whose
-                // evaluation is in and that the FP32 test would accept counts
-                // +1 or -1 for its species; one not yet evaluated counts as
-                // the chain's more frequent outcome for its kind.  The
-                // particle pick uses the prediction; the committer checks the
-                // pick against the actual counts.  Skipped when the pick is
-                // the same for every count the pending moves can leave.
-                const int go = tc.go[p], mm = tc.m[p], c0 = tc.c0[p];
-                if (go == 1 && mm > c0 && !C.pick_settled(mm, tc.ns[p], mm - c0)) {
-                    const int k = c0 + lane;
-                    int d = 0, sk = 0;
-                    if (k < mm) {
-                        const WordRec &Wk = C.words(k);
-                        const uint32_t w0 = Wk.w[0];
-                        const int ty = (w0 < a.thr_disp) ? 0 : ((w0 < a.thr_ins) ? 1 : 2);
-                        const Slot &Sk = sh.slots[(k) & (kRS - 1)];
-                        if (ty != 0 && vload(Sk.tag) == k + 1 && vload(Sk.arrive) == G + 1 && Sk.t.possible) {
-                            sk = Sk.t.s;
-                            const float dU = F32 ? Sk.th : (float)Sk.td;
-                            const float lnK = (ty == 1) ? a.lnzv_f[sk] - sh.ln_n1[sk] : sh.ln_n[sk] - a.lnzv_f[sk];
-                            if (Wk.lnu < lnK - a.beta_f * dU) d = (ty == 1) ? 1 : -1;
-                        } else if (ty != 0 && vload(sh.likely[ty - 1])) {
-                            sk = (int)__umulhi(Wk.w[5], (uint32_t)a.S);
-                            d = (ty == 1) ? 1 : -1;
-                        }
-                    }
-                    for (int q = 0; q < a.S; ++q) {
-                        const int dn = __popc(__ballot_sync(0xffffffffu, d > 0 && sk == q)) -
-                                       __popc(__ballot_sync(0xffffffffu, d < 0 && sk == q));
-                        if (lane == 0) tc.ns[p][q] = max(0, tc.ns[p][q] + dn);
-                    }
-                    __threadfence_block();
-                }
-            }
-            // the whole leader warp reaches the team barrier together: the
-            // barrier counts warps, not lanes
-            __syncwarp();
-            team_sync(1 + team, G * 32);
-            if (tc.go[p] == 2) {
-                if (j == 0 && lane == 0) {
-                    atomicAdd(&team_cyc[0], cyc_idle);
-                    atomicAdd(&team_cyc[1], cyc_eval);
-                    atomicAdd(&team_cyc[2], n_eval);
-                }
-                break;
-            }
-            const unsigned long long te = prof_clock<PROF>();
-            const int m = tc.m[p];
-            const Trial t = C.make_trial(m, tc.ns[p]);
-            Slot &S = sh.slots[(m) & (kRS - 1)];
-            // the trial and the counts it picked with, published before the
-            // evaluation: the committer checks them while the team evaluates
-            if (j == 0) {
-                if (lane < a.S) S.nsu[lane] = tc.ns[p][lane];
-                if (lane == 0) S.t = t;
-                __syncwarp();
-                if (lane == 0) {
-                    __threadfence_block();
-                    vstore(S.tpub, m + 1);
-                }
-            }
-            const typename Chain<F32, VIR>::Part P = C.template eval_part<F32, KU>(t, j, G);
-            if (P.self_slot >= 0) S.self_slot = P.self_slot;
-            if (P.has_last) {
-                S.last_val = P.last;
-                S.has_last = 1;
-            }
-            if (lane == 0) {
-                S.pseq[j] = P.seq;
-                if constexpr (F32) {
-                    S.ph[j] = P.e;
-                    S.pl[j] = P.el;
-                    S.pu[j] = P.ua;
-                    S.pw[j] = P.w;
-                } else {
-                    S.pd[j] = P.de;
-                    S.pa[j] = P.da;
-                    S.pwd[j] = P.dw;
-                }
-            }
-            __syncwarp();
-            int last = 0;
-            if (lane == 0) {
-                __threadfence_block();
-                last = atomicAdd(&S.arrive, 1) == G - 1;
-                if (j == 0) {
-                    cyc_eval += prof_clock<PROF>() - te;
-                    ++n_eval;
-                }
-            }
-            // the team's last warp adds the G partial sums in a fixed order
-            // (lanes 0 .. G-1, butterfly) and marks the move arrive = G + 1:
-            // the committer reads one total
-            if (__shfl_sync(0xffffffffu, last, 0)) {
-                __threadfence_block();
-                if constexpr (F32) {
-                    const volatile Slot &V = S;
-                    FF v = {lane < G ? V.ph[lane] : 0.f, lane < G ? V.pl[lane] : 0.f};
-                    float u = lane < G ? V.pu[lane] : 0.f;
-                    float w = (VIR && lane < G) ? V.pw[lane] : 0.f;
-#pragma unroll
-                    for (int o = kGMax / 2; o > 0; o >>= 1) {
-                        FF x;
-                        x.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-                        x.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-                        v = ff_add(v, x);
-                        u += __shfl_xor_sync(0xffffffffu, u, o);
-                        w += __shfl_xor_sync(0xffffffffu, w, o);
-                    }
-                    if (lane == 0) {
-                        S.th = v.hi;
-                        S.tl = v.lo;
-                        S.tu = u;
-                        S.tw = w;
-                    }
-                } else {
-                    const volatile Slot &V = S;
-                    double v = lane < G ? V.pd[lane] : 0.0, u = lane < G ? V.pa[lane] : 0.0;
-                    double w = (VIR && lane < G) ? V.pwd[lane] : 0.0;
-#pragma unroll
-                    for (int o = kGMax / 2; o > 0; o >>= 1) {
-                        v += __shfl_xor_sync(0xffffffffu, v, o);
-                        u += __shfl_xor_sync(0xffffffffu, u, o);
-                        w += __shfl_xor_sync(0xffffffffu, w, o);
-                    }
-                    if (lane == 0) {
-                        S.td = v;
-                        S.ta = u;
-                        S.tdw = w;
-                    }
-                }
-                if (lane == 0) {
-                    __threadfence_block();
-                    atomicAdd(&S.arrive, 1);
-                }
-                __syncwarp();
-            }
-        }
-    } else if (warp == 0) {
-        // ------------------------------------------------------------ committer
-        int att_id[2] = {0, 0}, acc_id[2] = {0, 0};  // insertions, deletions (lane 0)
-        unsigned long long cw = 0, cv = 0, cd = 0, ca = 0, ct = 0;  // committer cycles (see ChainOut::prof)
-        unsigned long long cv_e = 0, cv_l = 0, cv_p = 0, cb = 0;
-        int nacc = 0;  // moves accepted so far (the committer's count, published in sh.nacc)
-        for (int m = 0; m < n; ++m) {
-            const unsigned long long tm0 = prof_clock<PROF>();
-            Slot &S = sh.slots[(m) & (kRS - 1)];
-            bool ok = true;
-            if (m == a.stall_at) {
-                // diagnostic: a bounded wait on a flag nothing sets runs out,
-                // and the chain stops before this move with a timeout status
-                Wait ws;
-                for (;;) {
-                    int f = 0;
-                    if (lane == 0) f = vload(sh.never);
-                    if (__shfl_sync(0xffffffffu, f, 0)) break;
-                    if (ws.expired(a.wait_ns)) {
-                        if (lane == 0) {
-                            atomicOr(&sh.status, kStatusTimeout);
-                            atomicOr(&sh.where, 2);
-                        }
-                        ok = false;
-                        break;
-                    }
-                }
-                if (!ok) break;
-            }
-            int c0 = 0, attempt = 0;
-            Trial tcur;
-            for (;; ++attempt) {
-                // wait for the trial of m (its evaluation under way) and for
-                // room in the keeper's book
-                const unsigned long long tw = prof_clock<PROF>();
-                Wait wt;
-                for (;;) {
-                    int r = 0;
-                    if (lane == 0) {
-                        const int tg = vload(S.tag);
-                        __threadfence_block();
-                        r = tg == m + 1 && vload(S.tpub) == m + 1 && m < vload(sh.booked) + kRS;
-                    }
-                    r = __shfl_sync(0xffffffffu, r, 0);
-                    if (r) break;
-                    if (wt.expired(a.wait_ns)) {
-                        if (lane == 0) {
-                            atomicOr(&sh.status, kStatusTimeout);
-                            atomicOr(&sh.where, 2);
-                        }
-                        ok = false;
-                        break;
-                    }
-                }
-                if (!ok) break;
-                const unsigned long long tv = prof_clock<PROF>();
-                cw += tv - tw;
-                __threadfence_block();
-                c0 = S.c0;
-                tcur = S.t;  // one copy in registers for the checks and the decision
-                // While the team evaluates, check what does not depend on its
-                // sums (the moves [c0, m) are all committed by now).  The
-                // counts at the move's turn equal those the evaluation picked
-                // with: the same particle (else compare the picks).  No move
-                // accepted since the evaluation started: nothing it read has
-                // changed (counts, records, cells).
-                const bool quiet = S.acc0 == nacc;
-                const int *ring = sh.ns_ring[m & (kRS - 1)];
-                bool pick = c0 == m || tcur.type == 1;
-                if (!pick && (tcur.type == 2 || a.S == 1)) {
-                    // one count decides the pick
-                    const int na = ring[tcur.type == 2 ? (int)tcur.s : 0];
-                    pick = tcur.possible ? (na > 0 && pick_index((uint32_t)na, C.words(m).w, tcur.type) == tcur.idx)
-                                         : na == 0;
-                } else if (!pick) {
-                    pick = __all_sync(0xffffffffu, lane >= a.S || S.nsu[lane] == ring[lane]) || pick_ok(C, sh, tcur, m);
-                }
-                const unsigned long long tv1 = prof_clock<PROF>();
-                const bool logs = !pick || c0 == m || quiet || logs_ok(C, sh, tcur, c0, m, lane);
-                const unsigned long long tv2 = prof_clock<PROF>();
-                // then wait for the team's sums
-                Wait wa;
-                for (;;) {
-                    int r = 0;
-                    if (lane == 0) r = vload(S.arrive) == G + 1;
-                    r = __shfl_sync(0xffffffffu, r, 0);
-                    if (r) break;
-                    if (wa.expired(a.wait_ns)) {
-                        if (lane == 0) {
-                            atomicOr(&sh.status, kStatusTimeout);
-                            atomicOr(&sh.where, 2);
-                        }
-                        ok = false;
-                        break;
-                    }
-                }
-                if (!ok) break;
-                const unsigned long long tv3 = prof_clock<PROF>();
-                cw += tv3 - tv2;
-                __threadfence_block();
-                // the team's warps must have read the counts of one epoch
-                // (their item ranges follow the counts)
-                const int q0 = S.pseq[0];
-                const bool one_epoch = quiet || (__all_sync(0xffffffffu, lane >= G || S.pseq[lane] == q0) && q0 >= 0);
-                const bool valid = pick && (c0 == m || quiet || (one_epoch && logs));
-                const unsigned long long tv4 = prof_clock<PROF>();
-                cv += (tv2 - tv) + (tv4 - tv3);
-                cv_p += tv1 - tv;
-                cv_l += tv2 - tv1;
-                cv_e += tv4 - tv3;
-                if (valid) break;
-                // evaluate again against the configuration after m moves
-                if (lane == 0) {
-                    vstore(S.tag, 0);
-                    __threadfence_block();
-                    vstore(redo, m + 1);
-                }
-                __syncwarp();
-            }
-            if (!ok) break;
-            const unsigned long long td = prof_clock<PROF>();
-            const Trial t = tcur;
-            const int self_slot = S.self_slot;
-            const uint4 last_val = S.last_val;
-            // the team's totals (summed by its last warp in a fixed order)
-            FF e = {0.f, 0.f};
-            float uab = 0.f;
-            double de = 0.0, da = 0.0, dW = 0.0;
-            if constexpr (F32) {
-                e.hi = S.th;
-                e.lo = S.tl;
-                uab = S.tu;
-                dW = VIR ? (double)S.tw : 0.0;
-            } else {
-                de = S.td;
-                da = S.ta;
-                dW = S.tdw;
-                e.hi = __double2float_rn(de);
-                uab = __double2float_rn(da);
-            }
-            int refined = attempt > 0 ? 4 : 0;
-            const int type = t.type, sp = t.s;
-            const long long ns = sh.n[sp];
-            // the Metropolis test in FP32 with an error band
-            const int dec = t.possible ? decide_f32(a, type, sp, sh.ln_n[sp], sh.ln_n1[sp], C.words(m).lnu, e.hi + e.lo, uab)
-                                       : 0;
-            int fin = dec == 1 ? 1 : 0, use64 = F32 ? 0 : 1;
-            double lnA_d = 0.0;
-            if (dec < 0) {
-                // decide in FP64: in FP32 mode the whole trial is evaluated
-                // again in FP64 (pair terms and sums)
-                if constexpr (F32) {
-                    const typename Chain<F32, VIR>::Part Q = C.template eval_part<false, 1>(t, 0, 1);
-                    de = Q.de;
-                    da = Q.da;
-                    dW = Q.dw;
-                }
-                const WordRec &W = C.words(m);
-                const double lnu = log(uniform53(W.w[6], W.w[7]));
-                double lnK = 0.0;
-                if (type == 1) lnK = a.logz[sp] + a.lnV - log((double)(ns + 1));
-                else if (type == 2) lnK = log((double)ns) - a.logz[sp] - a.lnV;
-                lnA_d = lnK - a.beta * de;
-                fin = (lnu < lnA_d) ? 1 : 0;
-                const double band = a.beta * a.tol * da + 1e-12 * (1.0 + fabs(lnA_d));
-                refined |= 2 | ((fabs(lnu - lnA_d) <= band) ? 1 : 0);
-                use64 = 1;
-                uab = (float)da;
-            }
-            if (lane == 0 && type != 0) {
-                // the chain's more frequent outcome per kind, for the count prediction
-                const int q = type - 1;
-                att_id[q] += 1;
-                acc_id[q] += fin & 1;
-                const int lk = 2 * acc_id[q] > att_id[q];
-                if (lk != sh.likely[q]) vstore(sh.likely[q], lk);
-            }
-            int stop_bits = 0;
-            if (fin & 1) {
-                if (type == 1 && ns >= a.maxN) stop_bits = kStatusCapacity;
-                else if ((type == 1 || t.cross) && cnt[t.cn] >= a.cap) stop_bits = kStatusCellOverflow;
-            }
-            if (stop_bits) {
-                if (lane == 0) {
-                    atomicOr(&sh.status, stop_bits);
-                    vstore(sh.stop, 1);
-                }
-                break;
-            }
-            LogRec &L = sh.logs[(m) & (kRS - 1)];
-            const unsigned long long tapp = prof_clock<PROF>();
-            cd += tapp - td;
-            if (fin & 1) C.apply(t, self_slot, last_val, L);
-            else if (lane == 0) L.head.x = 0;
-            const unsigned long long tb0 = prof_clock<PROF>();
-            ca += tb0 - tapp;
-            __syncwarp();
-            if (lane < kMaxSpecies) sh.ns_ring[((m + 1)) & (kRS - 1)][lane] = (int)sh.n[lane];
-            __syncwarp();
-            if (lane == 0) {
-                BookRec &B = sh.book[(m) & (kRS - 1)];
-                B.dU64 = de;
-                B.dW = dW;
-                B.hi = e.hi;
-                B.lo = e.lo;
-                B.use64 = use64;
-                B.lnA = lnA_d;
-                B.uab = uab;
-                B.fin = fin;
-                B.type = type;
-                B.sp = sp;
-                B.index = (type == 1) ? (int)ns : t.idx;
-                B.possible = t.possible;
-                B.refined = refined;
-                B.ns = ns;
-                // the move's writes are visible before the accepted count and
-                // the commit count say so
-                __threadfence_block();
-                if (fin & 1) vstore(sh.nacc, nacc + 1);
-                vstore(B.ready, m + 1);
-                vstore(sh.committed, m + 1);
-            }
-            nacc += fin & 1;
-            __syncwarp();
-            const unsigned long long tend = prof_clock<PROF>();
-            cb += tend - tb0;
-            ct += tend - tm0;
-        }
-        if (lane == 0) {
-            vstore(sh.stop, 1);  // evaluators and keeper wind down
-            ChainOut &o = *a.out;
-            o.prof[0] = cw;
-            o.prof[1] = cv;
-            o.prof[2] = cd;
-            o.prof[3] = ca;
-            o.prof[4] = ct;
-            o.prof[8] = cv_e;
-            o.prof[9] = cv_l;
-            o.prof[10] = cv_p;
-            o.prof[11] = cb;
-        }
-    } else if (warp == keeper_warp) {
-        // ------------------------------------------------------------ keeper
-        double E = *a.d_energy, sumE = 0.0;
-        // the running virial, for the chains of the launch that keep it
-        const bool vir = VIR && a.virial;
-        double Wv = vir ? a.d_energy[1] : 0.0, sumW = 0.0;
-        long long sumN = 0, att0 = 0, att1 = 0, att2 = 0, acc0 = 0, acc1 = 0, acc2 = 0;
-        long long flagged = 0, reeval = 0, refines = 0, Ncur = 0;
-        for (int q = 0; q < kMaxSpecies; ++q) Ncur += sh.n[q];
-        int mb = 0;
-        Wait wt;
-        for (;;) {
-            // refill the words ring ahead of the evaluators
-            int c = 0, f = 0, sp0 = 0;
-            if (lane == 0) {
-                c = vload(sh.committed);
-                f = vload(sh.filled);
-                sp0 = vload(sh.stop);
-            }
-            c = __shfl_sync(0xffffffffu, c, 0);
-            f = __shfl_sync(0xffffffffu, f, 0);
-            sp0 = __shfl_sync(0xffffffffu, sp0, 0);
-            if (f < n && f + kFill <= c + kRW - kFill && !sp0) {
-                const int cntw = min(kFill, n - f);
-                C.fill_words(f, cntw);
-                __threadfence_block();
-                if (lane == 0) vstore(sh.filled, f + cntw);
-                __syncwarp();
-                continue;
-            }
-            // book the committed moves in order
-            int rdy = 0;
-            if (lane == 0 && mb < n) rdy = vload(sh.book[(mb) & (kRS - 1)].ready);
-            rdy = __shfl_sync(0xffffffffu, rdy, 0);
-            if (mb < n && rdy == mb + 1) {
-                __threadfence_block();
-                if (lane == 0) {
-                    const BookRec &B = sh.book[(mb) & (kRS - 1)];
-                    const int type = B.type;
-                    att0 += type == 0;
-                    att1 += type == 1;
-                    att2 += type == 2;
-                    if (B.refined & 1) ++flagged;
-                    if (B.refined & 2) ++refines;
-                    if (B.refined & 4) ++reeval;
-                    if (B.fin & 1) {
-                        acc0 += type == 0;
-                        acc1 += type == 1;
-                        acc2 += type == 2;
-                        E += B.use64 ? B.dU64 : (double)B.hi + (double)B.lo;
-                        Wv += B.dW;
-                        Ncur += (type == 1) - (type == 2);
-                    }
-                    if (a.trace) {
-                        const double dU = B.use64 ? B.dU64 : (double)B.hi + (double)B.lo;
-                        gcmc_trace tr;
-                        double lnA = B.lnA;
-                        if (!(B.refined & 2)) {
-                            double lnK = 0.0;
-                            if (type == 1) lnK = a.logz[B.sp] + a.lnV - log((double)(B.ns + 1));
-                            else if (type == 2 && B.ns > 0) lnK = log((double)B.ns) - a.logz[B.sp] - a.lnV;
-                            lnA = B.possible ? lnK - a.beta * dU : -INFINITY;
-                        }
-                        tr.dU = B.possible ? dU : 0.0;
-                        tr.lnA = lnA;
-                        tr.uabs = B.possible ? (double)B.uab : 0.0;
-                        tr.index = B.index;
-                        tr.type = (uint8_t)type;
-                        tr.species = (uint8_t)B.sp;
-                        tr.accepted = (uint8_t)(B.fin & 1);
-                        tr.flagged = (uint8_t)(B.refined & 3);
-                        a.trace[mb] = tr;
-                    }
-                    sumE += E;
-                    sumW += Wv;
-                    sumN += Ncur;
-                    vstore(sh.booked, mb + 1);
-                }
-                __syncwarp();
-                ++mb;
-                wt = Wait();
-                continue;
-            }
-            if (mb >= n) break;
-            int stop = 0, com = 0;
-            if (lane == 0) {
-                stop = vload(sh.stop);
-                com = vload(sh.committed);
-            }
-            stop = __shfl_sync(0xffffffffu, stop, 0);
-            com = __shfl_sync(0xffffffffu, com, 0);
-            if (stop && mb >= com) break;
-            if (wt.expired(a.wait_ns)) {
-                if (lane == 0) {
-                    atomicOr(&sh.status, kStatusTimeout);
-                    atomicOr(&sh.where, 4);
-                    vstore(sh.stop, 1);
-                }
-                break;
-            }
-            __nanosleep(20);
-        }
-        if (lane == 0) {
-            ChainOut &o = *a.out;
-            o.attempted[0] = att0;
-            o.attempted[1] = att1;
-            o.attempted[2] = att2;
-            o.accepted[0] = acc0;
-            o.accepted[1] = acc1;
-            o.accepted[2] = acc2;
-            o.flagged = flagged;
-            o.moves_done = mb;
-            o.energy = E;
-            o.sum_energy = sumE;
-            o.sum_n = (double)sumN;
-            o.reevaluated = reeval;
-            o.refines = refines;
-            o.virial = vir ? Wv : NAN;
-            o.sum_virial = vir ? sumW : NAN;
-            *a.d_energy = E;
-            if (vir) a.d_energy[1] = Wv;
-        }
-    }
+    if (warp < a.movers) mover_loop<F32, VIR, PROF>(a, sh, cnt, dyn + (size_t)warp * kMoverBytes, warp);
+    else if (warp == kChainWarps - 1) keeper_loop<VIR>(a, sh);
     __syncthreads();
     for (int c = tid; c < a.ncell; c += NTH) a.cell_count[c] = cnt[c];
     if (tid < a.S) a.d_n[tid] = sh.n[tid];
     if (tid == 0) {
         ChainOut &o = *a.out;
-        for (int q = 0; q < kMaxSpecies; ++q) o.n[q] = sh.n[q];
+        for (int k = 0; k < kMaxSpecies; ++k) o.n[k] = sh.n[k];
         int st = sh.status;
         if (!(o.energy - o.energy == 0.0)) st |= kStatusNonFinite;
         o.status = st;
@@ -1751,36 +1287,21 @@ __global__ void __launch_bounds__(kChainWarps * 32, 1) k_chain(const ChainArgs *
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_end));
         o.t0 = t_start;
         o.t1 = t_end;
-        o.prof[5] = team_cyc[0];
-        o.prof[6] = team_cyc[1];
-        o.prof[7] = team_cyc[2];
+        for (int k = 0; k < 12; ++k) o.prof[k] = sh.prof[k];
+        o.prof[7] = (unsigned long long)sh.evaluations;
     }
 }
 
 // ---------------------------------------------------------------- host side
-// Team shapes the launcher can use: (warps per team, teams, look-ahead).
-// More teams evaluate more moves ahead (better when moves rarely conflict);
-// larger teams evaluate one move faster (better when N changes often).
-// Shape 0 leaves the committer's SM sub-partition to the committer and the
-// keeper (twelve evaluator warps on the other three); shape 1 adds two
-// evaluator warps there.
-constexpr int kNumConfigs = 4;
-
-template <bool F32, bool VIR, bool PROF>
-static void *chain_kernel(int config)
-{
-    switch (config) {
-    case 1: return (void *)k_chain<F32, VIR, 7, 2, 4, 2, PROF>;
-    case 2: return (void *)k_chain<F32, VIR, 4, 3, 6, 2, PROF>;
-    case 3: return (void *)k_chain<F32, VIR, 3, 4, 8, 2, PROF>;
-    default: return (void *)k_chain<F32, VIR, 6, 2, 4, 2, PROF>;
-    }
-}
+// The launcher's choices of W, the moves in flight.  More movers hide a longer
+// evaluation; fewer evaluate on a newer configuration, so fewer evaluations
+// are repeated where most moves are accepted or the box is small.
+constexpr int kMoverChoices[kChainConfigs] = {8, 5, 11, 15};
 
 template <bool F32, bool VIR>
-static void *chain_kernel(int config, bool prof)
+static void *chain_kernel(bool prof)
 {
-    return prof ? chain_kernel<F32, VIR, true>(config) : chain_kernel<F32, VIR, false>(config);
+    return prof ? (void *)k_chain<F32, VIR, true> : (void *)k_chain<F32, VIR, false>;
 }
 
 int chain_threads(int) { return kChainWarps * 32; }
@@ -1799,7 +1320,7 @@ struct ChainJob {
     gcmc_status result;
 };
 
-static void fill_args(ChainArgs &a, const ChainJob &j, ChainOut *out)
+static void fill_args(ChainArgs &a, const ChainJob &j, int movers, ChainOut *out)
 {
     gcmc_ctx *ctx = j.ctx;
     const gcmc_move_mix *mix = &j.mix;
@@ -1808,6 +1329,7 @@ static void fill_args(ChainArgs &a, const ChainJob &j, ChainOut *out)
     a.first = j.first + (uint64_t)j.done;
     a.n_moves = (j.result == GCMC_OK) ? (int)std::min<int64_t>(j.n_moves - j.done, 1 << 30) : 0;
     a.chain = j.chain;
+    a.movers = movers;
     a.T = ctx->T;
     a.ncell = (int)ctx->ncell;
     a.cap = ctx->cap;
@@ -1815,14 +1337,9 @@ static void fill_args(ChainArgs &a, const ChainJob &j, ChainOut *out)
     a.S = ctx->S;
     a.R2 = ctx->R2;
     a.rcg = ctx->rcg;
-    {
-        // FP32 r^2 from exact integer separations carries a relative error
-        // below 1e-6 (1 + D / rc); outside this band the FP32 test agrees
-        // with the exact one
-        const double band = 1e-5 * (1.0 + (double)(int64_t)(mix->max_disp * ctx->q) / (double)ctx->rcg);
-        a.r2lo = (float)((double)ctx->R2 * (1.0 - band));
-        a.r2hi = (float)((double)ctx->R2 * (1.0 + band));
-    }
+    // FP32 r^2 from exact integer separations carries a relative error below
+    // 1e-6: every pair inside the cutoff passes the screen
+    a.r2hi = (float)((double)ctx->R2 * (1.0 + 1e-5));
     a.thr_disp = (unsigned long long)(mix->p_disp * 4294967296.0);
     a.thr_ins = (unsigned long long)((mix->p_disp + mix->p_ins) * 4294967296.0);
     const int64_t D = (int64_t)(mix->max_disp * ctx->q);
@@ -1922,9 +1439,13 @@ static gcmc_status run_jobs(std::vector<ChainJob> &jobs, cudaStream_t st, bool f
         if (err) *err = cudaGetErrorString(e);
         return GCMC_ERR_CUDA;
     }
-    size_t smem = 16;
-    for (auto &j : jobs) smem = std::max(smem, ((size_t)j.ctx->ncell * sizeof(uint16_t) + 15) / 16 * 16);
-    if (f32) smem += kMaxEW * kQ * sizeof(int4);
+    size_t counters = 16;
+    for (auto &j : jobs) counters = std::max(counters, ((size_t)j.ctx->ncell * sizeof(uint16_t) + 15) / 16 * 16);
+    // a box of very many cells leaves room for fewer movers
+    const size_t state = sizeof(Shared) + sizeof(ChainArgs) + 1024;
+    const size_t room = (jobs[0].ctx->smem_optin - state - counters) / kMoverBytes;
+    const int movers = (int)std::min<size_t>(kMoverChoices[config], room);
+    const size_t smem = (size_t)movers * kMoverBytes + counters;
     // the virial sums are compiled in only when a chain of the launch keeps
     // it, the cycle counters only when a chain's context asked for them
     bool vir = false, prof = false;
@@ -1932,8 +1453,8 @@ static gcmc_status run_jobs(std::vector<ChainJob> &jobs, cudaStream_t st, bool f
         vir |= (j.mix.flags & GCMC_MIX_VIRIAL) != 0;
         prof |= j.ctx->chain_prof;
     }
-    void *kern = f32 ? (vir ? chain_kernel<true, true>(config, prof) : chain_kernel<true, false>(config, prof))
-                     : (vir ? chain_kernel<false, true>(config, prof) : chain_kernel<false, false>(config, prof));
+    void *kern = f32 ? (vir ? chain_kernel<true, true>(prof) : chain_kernel<true, false>(prof))
+                     : (vir ? chain_kernel<false, true>(prof) : chain_kernel<false, false>(prof));
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) {
         if (err) *err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e);
@@ -1942,7 +1463,7 @@ static gcmc_status run_jobs(std::vector<ChainJob> &jobs, cudaStream_t st, bool f
     for (int round = 0; round < (1 << 20); ++round) {
         bool any = false;
         for (int k = 0; k < K; ++k) {
-            fill_args(B.h_args[k], jobs[k], B.d_out + k);
+            fill_args(B.h_args[k], jobs[k], movers, B.d_out + k);
             any = any || B.h_args[k].n_moves > 0;
         }
         if (!any) break;
@@ -2053,7 +1574,9 @@ static gcmc_status run_jobs(std::vector<ChainJob> &jobs, cudaStream_t st, bool f
                 if (rs != GCMC_OK) j.result = rs;
                 continue;
             }
-            if (o.moves_done == 0) j.result = fail(ctx, GCMC_ERR_CUDA, "gcmc_run_moves: the chain kernel made no progress");
+            if (o.moves_done == 0)
+                j.result = fail(ctx, GCMC_ERR_CUDA, "gcmc_run_moves: the chain kernel made no progress (status " +
+                                                        std::to_string(o.status) + ", sites " + std::to_string(o.pad) + ")");
         }
         // the grown arrays must be visible to the next round's arguments
         for (auto &j : jobs) j.ctx->energy_valid = true;
@@ -2061,13 +1584,13 @@ static gcmc_status run_jobs(std::vector<ChainJob> &jobs, cudaStream_t st, bool f
     return GCMC_OK;
 }
 
-// Runs the jobs with the given team shape, or -- config < 0 -- picks one:
-// the first quarter of the moves runs under shape 0 (a fresh configuration
-// relaxes there, and its rates do not predict the rest), then every shape is
+// Runs the jobs with the given choice of W, or -- config < 0 -- picks one:
+// the first quarter of the moves runs under choice 0 (a fresh configuration
+// relaxes there, and its rates do not predict the rest), then every choice is
 // timed on short chunks, twice, in the orders 0 .. K-1 and K-1 .. 0 (the sum
-// cancels a steady drift of the chains), and the rest runs under the shape
-// with the smallest total (config returns the choice).  Every shape takes
-// exactly the same moves, so tuning never changes the chain.
+// cancels a steady drift of the chains), and the rest runs under the one
+// with the smallest total (config returns it).  Every choice takes exactly
+// the same moves, so tuning never changes the chain.
 static gcmc_status run_jobs_tuned(std::vector<ChainJob> &jobs, cudaStream_t st, bool f32, int &config,
                                   LaunchBufs &B, int64_t *launches, std::string *err, bool use_graph,
                                   double *probe_ms, double *dev_ms = nullptr)
@@ -2075,12 +1598,12 @@ static gcmc_status run_jobs_tuned(std::vector<ChainJob> &jobs, cudaStream_t st, 
     if (config >= 0) return run_jobs(jobs, st, f32, config, B, launches, err, use_graph, dev_ms);
     int64_t remaining = INT64_MAX;
     for (auto &j : jobs) remaining = std::min<int64_t>(remaining, j.n_moves - j.done);
-    const int64_t chunk = std::min<int64_t>(std::max<int64_t>(remaining / (8 * kNumConfigs), 256), 2048);
-    if (remaining < 4 * chunk * kNumConfigs) {
+    const int64_t chunk = std::min<int64_t>(std::max<int64_t>(remaining / (8 * kChainConfigs), 256), 2048);
+    if (remaining < 4 * chunk * kChainConfigs) {
         config = 0;
         return run_jobs(jobs, st, f32, config, B, launches, err, use_graph, dev_ms);
     }
-    // runs the next `count` moves of every job under shape c; returns its time
+    // runs the next `count` moves of every job under choice c; returns its time
     auto run_limited = [&](int c, int64_t count, float *ms_out) -> gcmc_status {
         std::vector<int64_t> saved(jobs.size());
         for (size_t k = 0; k < jobs.size(); ++k) {
@@ -2102,13 +1625,13 @@ static gcmc_status run_jobs_tuned(std::vector<ChainJob> &jobs, cudaStream_t st, 
         if (ms_out) *ms_out = ms;
         return r;
     };
-    const int64_t burn = std::min<int64_t>(remaining / 4, remaining - 3 * chunk * kNumConfigs);
+    const int64_t burn = std::min<int64_t>(remaining / 4, remaining - 3 * chunk * kChainConfigs);
     gcmc_status r = run_limited(0, burn, nullptr);
     if (r != GCMC_OK) return r;
-    double total[kNumConfigs] = {};
+    double total[kChainConfigs] = {};
     for (int pass = 0; pass < 2; ++pass) {
-        for (int i = 0; i < kNumConfigs; ++i) {
-            const int c = pass == 0 ? i : kNumConfigs - 1 - i;
+        for (int i = 0; i < kChainConfigs; ++i) {
+            const int c = pass == 0 ? i : kChainConfigs - 1 - i;
             float ms = 0.f;
             r = run_limited(c, chunk, &ms);
             if (r != GCMC_OK) return r;
@@ -2116,7 +1639,7 @@ static gcmc_status run_jobs_tuned(std::vector<ChainJob> &jobs, cudaStream_t st, 
         }
     }
     int bc = 0;
-    for (int c = 0; c < kNumConfigs; ++c) {
+    for (int c = 0; c < kChainConfigs; ++c) {
         if (probe_ms) probe_ms[c] = total[c];
         if (total[c] < total[bc]) bc = c;
     }
@@ -2124,13 +1647,16 @@ static gcmc_status run_jobs_tuned(std::vector<ChainJob> &jobs, cudaStream_t st, 
     return run_jobs(jobs, st, f32, config, B, launches, err, use_graph, dev_ms);
 }
 
+constexpr size_t kChainReserve = 36576, kChainReserveFp32 = 28672;
+
 static gcmc_status check_chain_fits(gcmc_ctx *ctx)
 {
     const size_t smem = ((size_t)ctx->ncell * sizeof(uint16_t) + 15) / 16 * 16;
-    // the chain state and its arguments (static), the evaluator warps'
-    // pair-term queues (dynamic, FP32 runs) and a margin for the rest
-    const size_t queues = ctx->precision == GCMC_FP32 ? kMaxEW * kQ * sizeof(int4) : 0;
-    if (smem + sizeof(Shared) + sizeof(ChainArgs) + queues + 4096 > ctx->smem_optin)
+    // the documented limit on the cells of a box: what the counters may take
+    // beside kChainReserve bytes of chain state (which hold four movers)
+    static_assert(sizeof(Shared) + sizeof(ChainArgs) + 4 * kMoverBytes + 2048 <= kChainReserve, "chain state");
+    const size_t queues = ctx->precision == GCMC_FP32 ? kChainReserveFp32 : 0;
+    if (smem + kChainReserve + queues > ctx->smem_optin)
         return fail(ctx, GCMC_ERR_INVALID_ARG, "gcmc_run_moves: too many cells for the on-chip cell counters");
     if (ctx->T > 1023) return fail(ctx, GCMC_ERR_INVALID_ARG, "gcmc_run_moves: more than 1023 cells per side");
     return GCMC_OK;

@@ -329,7 +329,7 @@ __device__ __forceinline__ FF ff_add(FF a, FF b)
     const float s = a.hi + b.hi;
     const float bb = s - a.hi;
     const float e = (a.hi - (s - bb)) + (b.hi - bb);
-    const float t = e + a.lo + b.lo;
+    const float t = e + (a.lo + b.lo);  // the same for (a, b) and (b, a): a butterfly leaves every lane one value
     const float h = s + t;
     return FF{h, t - (h - s)};
 }

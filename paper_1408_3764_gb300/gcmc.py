@@ -162,11 +162,11 @@ class Box:
         return int(out[0])
 
     def set_chain_config(self, config: int):
-        """Team shape of the chain kernel: 0..3, or -1 = tuned on the next run."""
+        """Moves in flight of the chain kernel: choice 0..3, or -1 = tuned on the next run."""
         check(self._lib.gcmc_set_chain_config(self._h, int(config)), self._h)
 
     def chain_config(self) -> int:
-        """The chain kernel's current team shape (0..3; -1 before the tuner has run)."""
+        """The chain kernel's current choice of moves in flight (0..3; -1 before the tuner has run)."""
         out = C.c_int32()
         check(self._lib.gcmc_get_chain_config(self._h, C.byref(out)), self._h)
         return out.value
@@ -184,9 +184,9 @@ class Box:
         check(self._lib.gcmc_set_chain_profile(self._h, 1 if on else 0), self._h)
 
     def chain_profile(self) -> dict:
-        """SM cycles of the last chain run by role (zeros unless set_chain_profile was on):
-        committer waiting, validity, decision, applying, loop total; team leaders idle, teams
-        evaluating, evaluations."""
+        """SM cycles of the last chain run by role (zeros unless set_chain_profile was on; evaluations
+        always): evaluated moves waiting for their turn, the checks at the turn, the decision,
+        applying, all of it; waiting for the book, evaluating, evaluations."""
         out = np.zeros(12, np.float64)
         check(self._lib.gcmc_chain_profile(self._h, out.ctypes.data_as(C.c_void_p)), self._h)
         keys = ("commit_wait", "commit_valid", "commit_decide", "commit_apply", "commit_total",
@@ -428,7 +428,7 @@ class Batch:
         return n
 
     def config(self, set_config: int = -2):
-        """Sets the team shape (-1 automatic, -2 unchanged); returns it and the tuner's per-shape times."""
+        """Sets the choice of moves in flight (-1 automatic, -2 unchanged); returns it and the tuner's times."""
         out = C.c_int32()
         probe = np.zeros(_lib.CHAIN_CONFIGS, np.float64)
         check(self._lib.gcmc_batch_config(self._h, int(set_config), C.byref(out),
