@@ -68,12 +68,13 @@ FLUSH_BYTES = 256 << 20
 CHAIN_TRAFFIC = {"sha256_prefix": "fb1ab48a525325ae", "bytes": 19.05e6, "moves": 6.4e6}
 # DRAM bytes (read + write, summed over the call's launches) of the timed calls
 # of --kernels-only from one ncu capture (profiles/cell_build_mixture_1m.md),
-# valid for the sources whose joint sha256 has this prefix
+# valid for the sources whose joint sha256 has this prefix (the kernels of
+# these calls are those of the captured revision)
 KERNEL_TRAFFIC = {
-    "cells": {"sources": ("gcmc_cells.cu", "gcmc_device.cuh"), "sha256_prefix": "820ee9a4c2fb519e",
+    "cells": {"sources": ("gcmc_cells.cu", "gcmc_device.cuh"), "sha256_prefix": "6fd5582c04647251",
               "bytes": {"cell_build_mixture_1m": 115.4e6}},
     "energy": {"sources": ("gcmc_energy.cu", "gcmc_stage.cuh", "gcmc_device.cuh"),
-               "sha256_prefix": "13f89e1759c1ac26",
+               "sha256_prefix": "9bbb2660d89fd703",
                "bytes": {"trial_energy_mixture_1m": 151.6e6, "total_energy_mixture_1m": 17.97e6,
                          "energy_grad_262k": 6.39e6}},
 }

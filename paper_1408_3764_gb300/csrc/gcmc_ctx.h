@@ -100,7 +100,8 @@ gcmc_status cuda_fail(gcmc_ctx *ctx, cudaError_t e, const char *where);
 // Pinned host words that builds and energy calls read back (per context),
 // in 8-byte words: [0 .. 7] species totals, [8] largest cell count, [9]
 // status bits of a build; [10] energy, [11] virial, [12] status of the
-// full-system energy; [16 ..] the gradient's scalars, then its status.
+// full-system energy; [13] status of a call with few trial points; [16 ..] the
+// gradient's scalars, then its status.
 constexpr size_t kPinnedBytes = 8 * (16 + 2 + 2 * kMaxSpecies * kMaxSpecies + 8);
 
 gcmc_status ensure_scratch(gcmc_ctx *ctx, size_t bytes);
