@@ -74,7 +74,7 @@ KERNEL_TRAFFIC = {
     "cells": {"sources": ("gcmc_cells.cu", "gcmc_device.cuh"), "sha256_prefix": "6fd5582c04647251",
               "bytes": {"cell_build_mixture_1m": 115.4e6}},
     "energy": {"sources": ("gcmc_energy.cu", "gcmc_stage.cuh", "gcmc_device.cuh"),
-               "sha256_prefix": "9bbb2660d89fd703",
+               "sha256_prefix": "e9196cbdcf852df9",
                "bytes": {"trial_energy_mixture_1m": 151.6e6, "total_energy_mixture_1m": 17.97e6,
                          "energy_grad_262k": 6.39e6}},
 }

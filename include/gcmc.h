@@ -300,6 +300,12 @@ gcmc_status gcmc_total_energy_noalloc(gcmc_ctx *ctx, double *energy);
 gcmc_status gcmc_energy_grad(gcmc_ctx *ctx, float *dpos, double *deps, double *dsigma,
                              double *energy, double *virial);
 
+/* gcmc_energy_grad with dpos[k] = dE/dr_k of input particle k of the last
+ * gcmc_build_cells (device, N x 3 FP32) or NULL.
+ * Errors: STATE (no build, or moves since the last one), CUDA. */
+gcmc_status gcmc_energy_grad_input_order(gcmc_ctx *ctx, float *dpos, double *deps, double *dsigma,
+                                         double *energy, double *virial);
+
 /* Particle counts per species (host, n_species int64; zeros before the
  * first build).  Errors: INVALID_ARG (NULL). */
 gcmc_status gcmc_counts(gcmc_ctx *ctx, int64_t *n_per_species);

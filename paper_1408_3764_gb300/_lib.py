@@ -82,6 +82,7 @@ SIGNATURES = {
     "gcmc_total_energy": (C.c_int, [_vp, C.POINTER(C.c_double)]),
     "gcmc_total_energy_noalloc": (C.c_int, [_vp, _vp]),
     "gcmc_energy_grad": (C.c_int, [_vp, _vp, _vp, _vp, _vp, _vp]),
+    "gcmc_energy_grad_input_order": (C.c_int, [_vp, _vp, _vp, _vp, _vp, _vp]),
     "gcmc_counts": (C.c_int, [_vp, _vp]),
     "gcmc_get_state": (C.c_int, [_vp, _vp, _vp, _vp, _vp]),
     "gcmc_set_state": (C.c_int, [_vp, _vp, _vp, _vp, _vp, C.c_double]),

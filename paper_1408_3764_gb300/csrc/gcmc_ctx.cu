@@ -404,6 +404,15 @@ gcmc_status gcmc_energy_grad(gcmc_ctx *ctx, float *dpos, double *deps, double *d
     return energy_grad(ctx, dpos, deps, dsigma, energy, virial);
 }
 
+gcmc_status gcmc_energy_grad_input_order(gcmc_ctx *ctx, float *dpos, double *deps, double *dsigma,
+                                         double *energy, double *virial)
+{
+    if (!ctx) return GCMC_ERR_INVALID_ARG;
+    if (!ctx->built || !ctx->order_valid)
+        return fail(ctx, GCMC_ERR_STATE, "gcmc_energy_grad_input_order: no fresh build");
+    return energy_grad(ctx, dpos, deps, dsigma, energy, virial, true);
+}
+
 gcmc_status gcmc_counts(gcmc_ctx *ctx, int64_t *n)
 {
     if (!ctx || !n) return GCMC_ERR_INVALID_ARG;

@@ -135,8 +135,8 @@ gcmc_status total_energy_begin(gcmc_ctx *ctx, bool virial_only = false);
 gcmc_status total_energy_finish(gcmc_ctx *ctx, double *energy, bool virial_only = false);
 gcmc_status total_energy_noalloc(gcmc_ctx *ctx, double *energy_dev);
 gcmc_status energy_grad(gcmc_ctx *ctx, float *dpos, double *deps, double *dsigma, double *energy,
-                        double *virial);
-gcmc_status energy_grad_begin(gcmc_ctx *ctx, float *dpos);
+                        double *virial, bool input_order = false);
+gcmc_status energy_grad_begin(gcmc_ctx *ctx, float *dpos, bool input_order = false);
 gcmc_status energy_grad_finish(gcmc_ctx *ctx, double *deps, double *dsigma, double *energy, double *virial);
 // Writes the configuration as real coordinates (the centres of the grid
 // points, which quantise back to them) and species, species-major.

@@ -749,7 +749,8 @@ static void sum_partials(gcmc_ctx *ctx, const double *partial, int64_t n, int wi
 // particle; every pair is met from both of its particles (the forces of a
 // particle are summed by one warp, so nothing is scattered).  The per-cell
 // scalars go to `partial` rows of width 2 + 2 S^2: [E, virial, deps...,
-// dsigma...].  NS: partner species in registers (1, 2, or kMaxSpecies).
+// dsigma...].  order: the forces are stored at the particles' input rows (the
+// last build's order), otherwise species-major.  NS: partner species in registers (1, 2, or kMaxSpecies).
 // FP32 mode: FP32 pair terms from the exact integer r^2, forces summed in
 // FP32 per lane and FP64 across the warp, the scalars summed in
 // compensated FP32; FP64 mode: FP64 throughout.
@@ -824,7 +825,8 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_cell_grad(const uint4 *__rest
                                                              uint64_t R2, float r2lo, float r2hi, bool wrap, int S,
                                                              const __grid_constant__ FieldF ff,
                                                              const __grid_constant__ FieldD fd, double inv_h,
-                                                             const int64_t *__restrict__ d_n, float *__restrict__ dpos,
+                                                             const int64_t *__restrict__ d_n,
+                                                             const int32_t *__restrict__ order, float *__restrict__ dpos,
                                                              double *__restrict__ partial, int *__restrict__ status)
 {
     constexpr int kW = 2 + 2 * kMaxSpecies * kMaxSpecies;
@@ -971,7 +973,7 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_cell_grad(const uint4 *__rest
                 if (dpos) {
                     for (int i = threadIdx.x; i < pn; i += blockDim.x) {
                         const uint32_t tg = home[i].w;
-                        const int64_t row = base_s[tag_species(tg)] + tag_index(tg);
+                        const int64_t row = order ? order[h0 + pb + i] : base_s[tag_species(tg)] + tag_index(tg);
                         if constexpr (F32) {
                             const float ih = (float)inv_h;
                             dpos[3 * row + 0] = (fpartf[i][0].x + fpartf[i][0].y) * ih;
@@ -1205,7 +1207,7 @@ gcmc_status total_energy(gcmc_ctx *ctx, double *energy, bool virial_only)
     return total_energy_finish(ctx, energy, virial_only);
 }
 
-gcmc_status energy_grad_begin(gcmc_ctx *ctx, float *dpos)
+gcmc_status energy_grad_begin(gcmc_ctx *ctx, float *dpos, bool input_order)
 {
     gcmc_status st = make_compact(ctx);
     if (st != GCMC_OK) return st;
@@ -1228,7 +1230,7 @@ gcmc_status energy_grad_begin(gcmc_ctx *ctx, float *dpos)
         if (st != GCMC_OK) return st;                                                                         \
         k_cell_grad<F, NSP><<<nb, kNbWarps * 32, sizeof(NbShared), ctx->stream>>>(                            \
             ctx->cpos, ctx->cell_start, ctx->T, ctx->ncell, ctx->R2, r2lo, r2hi, wrap, S, ctx->ff, ctx->fd,    \
-            1.0 / ctx->h, ctx->d_n, dpos, part, ctx->d_status);                                               \
+            1.0 / ctx->h, ctx->d_n, input_order ? ctx->order : nullptr, dpos, part, ctx->d_status);           \
     } while (0)
     if (ctx->precision == GCMC_FP32) {
         if (S == 1) GCMC_GRAD(true, 1);
@@ -1269,9 +1271,9 @@ gcmc_status energy_grad_finish(gcmc_ctx *ctx, double *deps, double *dsigma, doub
 }
 
 gcmc_status energy_grad(gcmc_ctx *ctx, float *dpos, double *deps, double *dsigma, double *energy,
-                        double *virial)
+                        double *virial, bool input_order)
 {
-    gcmc_status st = energy_grad_begin(ctx, dpos);
+    gcmc_status st = energy_grad_begin(ctx, dpos, input_order);
     if (st != GCMC_OK) return st;
     GCMC_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return energy_grad_finish(ctx, deps, dsigma, energy, virial);

