@@ -782,21 +782,25 @@ struct GradDrain {
         const unsigned long long g = (unsigned long long)((long long)ex * ex) +
                                      (unsigned long long)((long long)ey * ey) +
                                      (unsigned long long)((long long)ez * ez);
-        R r2, c4e, sig2;
+        R c4e, s2, coef;
         if constexpr (F32) {
-            r2 = fmaf(__uint2float_rn((uint32_t)(g >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)g));
+            const float r2 = fmaf(__uint2float_rn((uint32_t)(g >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)g));
             c4e = ff.c4e[k];
-            sig2 = ff.sig2[k];
+            s2 = ff.sig2[k] / r2;
+            coef = r2;
         } else {
-            r2 = (double)g;
+            const double r2 = u64_to_f64(g);
+            double y;
             c4e = fd.c4e[k];
-            sig2 = fd.sig2[k];
+            s2 = div_by_g(fd.sig2[k], r2, g, y);
+            if (g == 0ull) s2 = __longlong_as_double(0x7ff0000000000000ll);
+            coef = fma(fma(-r2, y, 1.0), y, y);  // 1 / r^2
         }
-        const R s2 = sig2 / r2;
         const R s6 = s2 * s2 * s2;
         const R rep = c4e * s6 * s6, att = c4e * s6;
         const R rdu = (R)(-12) * rep + (R)6 * att;  // r U'(r)
-        const R coef = rdu / r2;
+        if constexpr (F32) coef = rdu / coef;
+        else coef *= rdu;
         fx += coef * (R)ex;
         fy += coef * (R)ey;
         fz += coef * (R)ez;
