@@ -74,7 +74,7 @@ KERNEL_TRAFFIC = {
     "cells": {"sources": ("gcmc_cells.cu", "gcmc_device.cuh"), "sha256_prefix": "eb69051b00b64433",
               "bytes": {"cell_build_mixture_1m": 115.4e6}},
     "energy": {"sources": ("gcmc_energy.cu", "gcmc_stage.cuh", "gcmc_device.cuh"),
-               "sha256_prefix": "c6aa145a9a0f065b",
+               "sha256_prefix": "3654b1093391fa25",
                "bytes": {"trial_energy_mixture_1m": 151.6e6, "total_energy_mixture_1m": 17.97e6,
                          "energy_grad_262k": 6.39e6}},
 }

@@ -79,13 +79,20 @@ __device__ __forceinline__ void pair_acc(const uint4 &p, const uint4 &q, uint32_
 // by bulk copies (gcmc_stage.cuh), at most kBuf records per pass, and each
 // staged record is converted once to float coordinates relative to the home
 // cell's centre.  Warps take the cell's points (trial points or home
-// particles), lanes the staged records: the FP32 squared distance screens the
-// cutoff (the exact integer squared distance decides inside a thin band
-// around rc^2), the pairs inside the cutoff join the warp's queue and are
-// evaluated 32 at a time -- in compensated FP32 (lj_ff) in FP32 mode, in FP64
-// in FP64 mode -- so the long pair term runs only on the ~15 % of
-// candidates inside the cutoff, with every lane busy.
-//
+// particles) a few at a time, lanes the staged records, 32 a row: the FP32
+// squared distance minus a bound just above rc^2 is accumulated from the
+// bound, and its sign bit is shifted into the point's mask, so that a row
+// costs seven instructions per point and one shared load for all of them.
+// The set bits -- the ~15 % of the candidates inside the cutoff -- are then
+// written to the warp's list and evaluated 32 at a time, where the exact
+// integer squared distance decides: in compensated FP32 (lj_ff) in FP32 mode,
+// in FP64 in FP64 mode, with every lane busy.
+// What bounds them: instruction issue (FP32 mode), the FP64 pipe (FP64 mode).
+// Screening with a vote and two population counts per row and a band test took
+// 55 instructions per 32 candidates and 1,350 per trial point, now 760: 10^6
+// points in the 2^20-particle mixture 1.49 -> 0.91 ms a call, its total energy
+// with the cell build 1.22 -> 0.83 ms, a gradient step of 262,144 particles
+// 1.88 -> 1.45 ms.
 // Minimum image relative to the cell centre c: a partner within rc of a
 // point p of the cell lies, along each axis, within rc + S/2 of c.  When
 // S >= rc (T = floor(L / rc) >= 3) that is at most 1.5 S <= L / 2, so the
@@ -94,10 +101,21 @@ __device__ __forceinline__ void pair_acc(const uint4 &p, const uint4 &q, uint32_
 // wrapped once more into [-L/2, L/2] (wrap = 1).  The queued pairs use the
 // exact wrapped integer difference p - q.
 // ---------------------------------------------------------------------------
-constexpr int kBuf = 896;     // staged records per pass (six CTAs fit an SM)
+// staged records per pass, in rows of 32 (a mask word holds at most 32): a
+// little more than a neighbourhood of 27 cells (14 for the half shell) holds
+// at liquid densities, so that most cells take one pass and shared memory
+// holds many CTAs (nine of four warps).  With 768 for both (six CTAs) the
+// trial energies took 1.09 ms and the total energy 0.95 ms.
+constexpr int kBufFull = 544, kBufHalf = 384;
+// ... and where plain FP32 sums of a point's terms are results: their order,
+// the pairs of a pass by staged index, is part of the result to its last digits
+constexpr int kBufOrdered = 896;
 constexpr int kPChunk = 64;   // points per chunk (per-point sums in shared memory)
-constexpr int kNbWarps = 8;   // warps of a neighbourhood CTA
-constexpr int kNbQ = 128;     // queue entries per warp (a ring: up to 31 + 2 x 32 pending)
+constexpr int kNbWarps = 4;   // warps of a neighbourhood CTA (two: trial energies 14 % slower; eight: total energy 18 %)
+constexpr int kNbQ = 128;     // queue entries per warp of k_trial_direct (a ring: up to 31 + 2 x 32 pending)
+static_assert(kBufFull % 32 == 0 && kBufHalf % 32 == 0 && kBufOrdered % 32 == 0 && kBufFull <= 1024 &&
+                  kBufHalf <= 1024 && kBufOrdered <= 1024 && kPChunk <= 64,
+              "list entries and masks");
 
 // Grid coordinate of the centre of cell k along an axis of T cells.
 __device__ __forceinline__ uint32_t cell_centre(int k, int T)
@@ -108,112 +126,206 @@ __device__ __forceinline__ uint32_t cell_centre(int k, int T)
 __device__ __forceinline__ float rel_f(uint32_t a, uint32_t c) { return (float)(int)(a - c); }
 
 // Shared state of a neighbourhood CTA.
+template <int KB>
 struct __align__(16) NbShared {
-    uint4 raw[kBuf];     // staged records (X, Y, Z, tag)
-    float4 fl[kBuf];     // the same relative to the home cell centre, tag bits in .w
-    int q[kNbWarps][kNbQ];
+    static constexpr int kBuf = KB;
+    uint4 raw[KB];       // staged records (X, Y, Z, tag)
+    float4 fl[KB];       // the same relative to the home cell centre
+    // pairs inside the cutoff: staged index | point << 10; up to 31 left over
+    // and a point's pairs
+    unsigned short list[kNbWarps][KB + 32];
     RunList runs;
     uint64_t bar;
-    int nbad;
+    // the species pairs' constants: FP32 mode float4 (c4e, c4e_lo, sig2,
+    // sig2_lo), FP64 mode (c4e, sig2) -- lanes of one warp read several
+    union {
+        float4 f[kMaxSpecies * kMaxSpecies];
+        double2 d[kMaxSpecies * kMaxSpecies];
+    } field;
 };
 
-// The per-warp queue of staged indices of pairs inside the cutoff.
-struct NbQueue {
-    int *buf;
-    int head, n;
-    unsigned lt;  // this lane's mask of lower lanes
-};
-
-// Adds the lanes' entries of two screened candidates (where in0 / in1) to
-// the queue; evaluates 32 at a time while 32 or more are pending.
-template <typename Drain>
-__device__ __forceinline__ void nb_push2(NbQueue &Q, bool in0, int f0, bool in1, int f1, Drain &D)
+template <bool F32, int KB>
+__device__ __forceinline__ void nb_field(NbShared<KB> &sh, const FieldF &ff, const FieldD &fd)
 {
-    const int lane = threadIdx.x & 31;
-    const unsigned b0 = __ballot_sync(0xffffffffu, in0), b1 = __ballot_sync(0xffffffffu, in1);
-    if ((b0 | b1) == 0u) return;
-    const int base = Q.head + Q.n, n0 = __popc(b0);
-    if (in0) Q.buf[(base + __popc(b0 & Q.lt)) & (kNbQ - 1)] = f0;
-    if (in1) Q.buf[(base + n0 + __popc(b1 & Q.lt)) & (kNbQ - 1)] = f1;
-    Q.n += n0 + __popc(b1);
-    if (Q.n >= 32) {
-        __syncwarp();
-        do {
-            D(Q.buf[(Q.head + lane) & (kNbQ - 1)], true);
-            Q.head = (Q.head + 32) & (kNbQ - 1);
-            Q.n -= 32;
-        } while (Q.n >= 32);
-        __syncwarp();
+    for (int k = threadIdx.x; k < kMaxSpecies * kMaxSpecies; k += blockDim.x) {
+        if constexpr (F32) sh.field.f[k] = make_float4(ff.c4e[k], ff.c4e_lo[k], ff.sig2[k], ff.sig2_lo[k]);
+        else sh.field.d[k] = make_double2(fd.c4e[k], fd.sig2[k]);
     }
 }
 
-template <typename Drain>
-__device__ __forceinline__ void nb_flush(NbQueue &Q, Drain &D)
-{
-    const int lane = threadIdx.x & 31;
-    if (Q.n > 0) {
-        __syncwarp();
-        const bool have = lane < Q.n;
-        D(have ? Q.buf[(Q.head + lane) & (kNbQ - 1)] : 0, have);
-        Q.head = (Q.head + Q.n) & (kNbQ - 1);
-        Q.n = 0;
-    }
-    __syncwarp();
-}
-
-// Screens the staged records [f0, nst) against point P (float position pf
-// relative to the centre) and queues those inside the cutoff.  skip(f)
-// leaves a record out (the point itself, or home-cell pairs met from the
-// other side).
 __device__ __forceinline__ float wrap_grid(float d)
 {
     return fmaf(-4294967296.0f, rintf(d * 2.3283064365386963e-10f), d);  // d - 2^32 rint(d / 2^32)
 }
 
-template <typename Skip, typename Drain>
-__device__ __forceinline__ void nb_screen(const NbShared &sh, int nst, const uint4 &P, const float3 &pf, uint64_t R2,
-                                          float r2lo, float r2hi, bool wrap, NbQueue &Q, Skip skip, Drain &D,
-                                          int tag = 0)
+// Screens the staged records of `rows` rows against NP points (coordinates
+// relative to the centre): bit rows - 1 - r of mask[p] in lane l stands for
+// record 32 r + l.  BAND: inner[p] holds those inside by more than `band` too.
+template <bool WRAP, int NP, bool BAND>
+__device__ __forceinline__ void nb_rows(const float4 *fl, int rows, const float3 *pf, float r2hi, float band,
+                                        uint32_t *mask, uint32_t *inner)
 {
-    const int lane = threadIdx.x & 31;
-    // two candidates per lane and pass (f and f + 32)
-    for (int b = 0; b < nst; b += 64) {
-        bool in[2], band[2];
-        int f[2];
+    fl += threadIdx.x & 31;
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            f[u] = b + 32 * u + lane;
-            in[u] = band[u] = false;
-            if (f[u] < nst) {
-                const float4 q = sh.fl[f[u]];
-                if (!skip(f[u], __float_as_uint(q.w))) {
-                    float dx = pf.x - q.x, dy = pf.y - q.y, dz = pf.z - q.z;
-                    if (wrap) {
-                        dx = wrap_grid(dx);
-                        dy = wrap_grid(dy);
-                        dz = wrap_grid(dz);
-                    }
-                    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                    in[u] = r2 < r2lo;
-                    band[u] = r2 >= r2lo && r2 <= r2hi;
-                }
+    for (int p = 0; p < NP; ++p) {
+        mask[p] = 0u;
+        if (BAND) inner[p] = 0u;
+    }
+#pragma unroll 2
+    for (int r = 0; r < rows; ++r) {
+        const float4 q = fl[32 * r];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            float dx = pf[p].x - q.x, dy = pf[p].y - q.y, dz = pf[p].z - q.z;
+            if (WRAP) {
+                dx = wrap_grid(dx);
+                dy = wrap_grid(dy);
+                dz = wrap_grid(dz);
             }
+            const float d = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, -r2hi)));
+            mask[p] = __funnelshift_l(__float_as_uint(d), mask[p], 1);
+            if (BAND) inner[p] = __funnelshift_l(__float_as_uint(d + band), inner[p], 1);
         }
-        // inside the thin band around rc^2 the exact integer test decides
-        if (__any_sync(0xffffffffu, band[0] || band[1])) {
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-                if (band[u]) in[u] = grid_sep(P, sh.raw[f[u]]).g < R2;
-        }
-        nb_push2(Q, in[0], f[0] | tag, in[1], f[1] | tag, D);
     }
 }
 
+// The same for the nst staged records (what lies behind them is left out):
+// those below the bound r2hi, a little above the cutoff.
+template <int NP>
+__device__ __forceinline__ void nb_screen(const float4 *fl, int nst, const float3 *pf, float r2hi, bool wrap,
+                                          uint32_t *mask)
+{
+    const int rows = (nst + 31) >> 5;
+    if (wrap) nb_rows<true, NP, false>(fl, rows, pf, r2hi, 0.f, mask, nullptr);
+    else nb_rows<false, NP, false>(fl, rows, pf, r2hi, 0.f, mask, nullptr);
+    const uint32_t keep = 32 * (rows - 1) + (int)(threadIdx.x & 31) < nst ? ~0u : ~1u;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) mask[p] &= keep;
+}
+
+// Exactly those inside the cutoff: the exact integer test decides in the thin
+// band around it.
+template <int NP>
+__device__ __forceinline__ void nb_screen_exact(const float4 *fl, const uint4 *raw, int nst, const uint4 *P,
+                                                const float3 *pf, uint64_t R2, float r2hi, bool wrap, uint32_t *mask)
+{
+    const int rows = (nst + 31) >> 5, lane = threadIdx.x & 31;
+    const float band = 2e-5f * r2hi;
+    uint32_t inner[NP];
+    if (wrap) nb_rows<true, NP, true>(fl, rows, pf, r2hi, band, mask, inner);
+    else nb_rows<false, NP, true>(fl, rows, pf, r2hi, band, mask, inner);
+    const uint32_t keep = 32 * (rows - 1) + lane < nst ? ~0u : ~1u;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        mask[p] &= keep;
+        uint32_t x = mask[p] & ~inner[p];
+        while (x) {
+            const int b = 31 - __clz((int)x);
+            if (grid_sep(P[p], raw[32 * (rows - 1 - b) + lane]).g >= R2) mask[p] ^= 1u << b;
+            x ^= 1u << b;
+        }
+    }
+}
+
+// Writes the records of a mask to the list by ascending index, without that of
+// tag `excl` (~0: none); returns their number.
+__device__ __forceinline__ int nb_list_ordered(unsigned short *list, uint32_t mask, int rows, const uint4 *raw,
+                                               uint32_t excl)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    int n = 0;
+#pragma unroll 2
+    for (int r = 0; r < rows; ++r) {
+        bool in = (mask >> (rows - 1 - r)) & 1u;
+        if (excl != 0xFFFFFFFFu && in) in = raw[32 * r + lane].w != excl;
+        const unsigned b = __ballot_sync(0xffffffffu, in);
+        if (in) list[n + __popc(b & lt)] = (unsigned short)(32 * r + lane);
+        n += __popc(b);
+    }
+    return n;
+}
+
+// Appends the records of a mask to the warp's list of n entries (tag in the
+// bits above the staged index); returns the new length.
+__device__ __forceinline__ int nb_append(unsigned short *list, int n, uint32_t mask, int rows, int tag)
+{
+    const int c = __popc(mask), inc = warp_inclusive_scan(c);
+    unsigned short *q = list + n + inc - c;
+    const int f0 = (rows - 1) * 32 + (int)(threadIdx.x & 31) + tag;
+    while (mask) {
+        const int b = 31 - __clz((int)mask);
+        *q++ = (unsigned short)(f0 - 32 * b);
+        mask ^= 1u << b;
+    }
+    return n + __shfl_sync(0xffffffffu, inc, 31);
+}
+
+// Evaluates the whole list, 32 entries at a time.
+template <typename Drain>
+__device__ __forceinline__ void nb_flush(const unsigned short *list, int n, Drain &D)
+{
+    __syncwarp();
+    for (int h = (int)(threadIdx.x & 31); h < n; h += 32) D(list[h]);
+    __syncwarp();
+}
+
+// Evaluates whole groups of 32 and moves the rest to the front; returns its
+// length.
+template <typename Drain>
+__device__ __forceinline__ int nb_drain(unsigned short *list, int n, Drain &D)
+{
+    const int lane = threadIdx.x & 31, full = n & ~31;
+    __syncwarp();
+    for (int h = lane; h < full; h += 32) D(list[h]);
+    unsigned short v = 0;
+    if (full + lane < n) v = list[full + lane];
+    __syncwarp();
+    if (full && full + lane < n) list[lane] = v;
+    return n - full;
+}
+
+// Sums of several values across the warp at once: each step adds half of the
+// lanes' values to the other half's and halves their number, so V values take
+// about V + 5 - log2 V additions instead of 5 V.  V a power of two up to 16;
+// the sum of value k ends in every lane l with (l >> (5 - log2 V)) == k.
+__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ FF shfl_xor(FF v, int o)
+{
+    return FF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+}
+__device__ __forceinline__ double sum_of(double a, double b) { return a + b; }
+__device__ __forceinline__ FF sum_of(FF a, FF b) { return ff_add(a, b); }
+
+template <int V, typename T>
+__device__ __forceinline__ T warp_sum_many(T *v)
+{
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int half = V / 2; half > 0; half >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < half; ++k) {
+            const T keep = up ? v[k + half] : v[k], send = up ? v[k] : v[k + half];
+            v[k] = sum_of(keep, shfl_xor(send, o));
+        }
+        o >>= 1;
+    }
+    T x = v[0];
+#pragma unroll
+    for (int k = V; k < 32; k <<= 1) {
+        x = sum_of(x, shfl_xor(x, o));
+        o >>= 1;
+    }
+    return x;
+}
 // Stages the items [w0, w1) of the neighbourhood into the shared buffers
 // (bulk copies, then the float conversion).  Returns false -- in every
 // thread -- when the copy did not land within the wait limit; the timeout
 // bit is then set and the block must return.
-__device__ __forceinline__ bool nb_stage(NbShared &sh, const uint4 *__restrict__ cpos, int w0, int w1,
+template <int KB>
+__device__ __forceinline__ bool nb_stage(NbShared<KB> &sh, const uint4 *__restrict__ cpos, int w0, int w1,
                                          uint32_t cx0, uint32_t cy0, uint32_t cz0, unsigned &parity,
                                          int *__restrict__ status)
 {
@@ -232,7 +344,7 @@ __device__ __forceinline__ bool nb_stage(NbShared &sh, const uint4 *__restrict__
     parity ^= 1u;
     for (int f = threadIdx.x; f < w1 - w0; f += blockDim.x) {
         const uint4 r = sh.raw[f];
-        sh.fl[f] = make_float4(rel_f(r.x, cx0), rel_f(r.y, cy0), rel_f(r.z, cz0), __uint_as_float(r.w));
+        sh.fl[f] = make_float4(rel_f(r.x, cx0), rel_f(r.y, cy0), rel_f(r.z, cz0), 0.f);
     }
     __syncthreads();
     return true;
@@ -246,39 +358,39 @@ struct TrialPt {
     int idx;       // the point's input index
 };
 
-template <bool F32>
+template <bool F32, class SH>
 struct TrialDrain {
-    const NbShared &sh;
+    const SH &sh;
     uint4 P;
-    int t;
-    const FieldF &ff;
-    const FieldD &fd;
+    uint32_t excl;
+    unsigned long long R2;
     float eh = 0.f, el = 0.f, mag = 0.f;
     double de = 0.0, da = 0.0;
-    __device__ TrialDrain(const NbShared &s, const uint4 &p, int t_, const FieldF &f, const FieldD &d)
-        : sh(s), P(p), t(t_), ff(f), fd(d)
+    __device__ TrialDrain(const SH &s, const TrialPt &p, unsigned long long r) : sh(s), P(p.P), excl(p.excl), R2(r)
     {
     }
-    __device__ __forceinline__ void operator()(int f, bool have)
+    __device__ __forceinline__ void operator()(int f)
     {
-        if (!have) return;
         const uint4 r = sh.raw[f];
-        const int k = t * kMaxSpecies + (int)tag_species(r.w);
         const int ex = (int)(P.x - r.x), ey = (int)(P.y - r.y), ez = (int)(P.z - r.z);
+        GridSep s;
+        s.dx = ex;
+        s.dy = ey;
+        s.dz = ez;
+        s.g = (unsigned long long)((long long)ex * ex) + (unsigned long long)((long long)ey * ey) +
+              (unsigned long long)((long long)ez * ez);
+        if (s.g >= R2 || r.w == excl) return;
+        const int k = (int)P.w * kMaxSpecies + (int)tag_species(r.w);
         if constexpr (F32) {
+            const float4 c = sh.field.f[k];
             float uh, ul, m;
-            lj_ff(ex, ey, ez, ff.c4e[k], ff.c4e_lo[k], ff.sig2[k], ff.sig2_lo[k], uh, ul, m);
+            lj_ff(ex, ey, ez, c.x, c.y, c.z, c.w, uh, ul, m);
             ff_acc(eh, el, uh, ul);
             mag += m;
         } else {
-            GridSep s;
-            s.dx = ex;
-            s.dy = ey;
-            s.dz = ez;
-            s.g = (unsigned long long)((long long)ex * ex) + (unsigned long long)((long long)ey * ey) +
-                  (unsigned long long)((long long)ez * ez);
+            const double2 c = sh.field.d[k];
             double u, m;
-            lj_f64(s, fd.c4e[k], fd.sig2[k], u, m);
+            lj_f64(s, c.x, c.y, u, m);
             de += u;
             da += m;
         }
@@ -286,24 +398,30 @@ struct TrialDrain {
 };
 
 // Trial points binned by cell: cell c holds the points pts[ps[c] .. ps[c+1]).
-template <bool F32>
+// Each warp screens two points together (they share the loads of the staged
+// records), evaluates the pairs of each and sums both across its lanes at once.
+// ABS: with the sums of |rep| + |att|, which FP32 mode adds in plain FP32, by
+// ascending staged index.
+template <bool F32, bool ABS>
 __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
     const TrialPt *__restrict__ pts, const int32_t *__restrict__ ps, const uint4 *__restrict__ cpos,
-    const int32_t *__restrict__ cs, int T, int64_t ncell, uint64_t R2, float r2lo, float r2hi, bool wrap,
+    const int32_t *__restrict__ cs, int T, int64_t ncell, uint64_t R2, float r2hi, bool wrap,
     const __grid_constant__ FieldF ff, const __grid_constant__ FieldD fd, double *__restrict__ out,
     double *__restrict__ out_abs, int *__restrict__ status)
 {
     extern __shared__ __align__(128) unsigned char dyn[];
-    NbShared &sh = *reinterpret_cast<NbShared *>(dyn);
+    constexpr bool kOrdered = F32 && ABS;
+    using SH = NbShared<kOrdered ? kBufOrdered : kBufFull>;
+    constexpr int kBuf = SH::kBuf;
+    SH &sh = *reinterpret_cast<SH *>(dyn);
     // per-point sums over the passes: FP32 mode float-float (hi, lo) and
     // uabs in .z; FP64 mode energy and uabs in .x, .y
-    __shared__ double2 part[kPChunk];
-    __shared__ float4 partf[kPChunk];
+    __shared__ typename std::conditional<F32, float4, double2>::type part[kPChunk];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (threadIdx.x == 0) mbar_init(&sh.bar, 1);
+    nb_field<F32>(sh, ff, fd);
     __syncthreads();
     unsigned parity = 0;
-    NbQueue Q = {sh.q[w], 0, 0, (1u << lane) - 1u};
     for (int64_t c = blockIdx.x; c < ncell; c += gridDim.x) {
         const int p0 = ps[c], p1 = ps[c + 1];
         if (p1 == p0) continue;  // uniform across the block
@@ -315,34 +433,59 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
         const uint32_t cx0 = cell_centre(cx, T), cy0 = cell_centre(cy, T), cz0 = cell_centre(cz, T);
         for (int pb = p0; pb < p1; pb += kPChunk) {
             const int pn = min(kPChunk, p1 - pb);
-            __syncthreads();  // the previous chunk's sums have been written out
-            for (int i = threadIdx.x; i < pn; i += blockDim.x) {
-                if constexpr (F32) partf[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                else part[i] = make_double2(0.0, 0.0);
-            }
             for (int base = 0; base < max(total, 1); base += kBuf) {
-                const int nst = min(kBuf, total - base);
-                if (!nb_stage(sh, cpos, base, base + max(nst, 0), cx0, cy0, cz0, parity, status)) return;
-                for (int i = w; i < pn; i += kNbWarps) {
-                    const TrialPt tp = pts[pb + i];
-                    const float3 pf = make_float3(rel_f(tp.P.x, cx0), rel_f(tp.P.y, cy0), rel_f(tp.P.z, cz0));
-                    TrialDrain<F32> D(sh, tp.P, (int)tp.P.w, ff, fd);
-                    const uint32_t ex = tp.excl;
-                    nb_screen(sh, max(nst, 0), tp.P, pf, R2, r2lo, r2hi, wrap, Q,
-                              [&](int, uint32_t tag) { return tag == ex; }, D);
-                    nb_flush(Q, D);
+                const int nst = max(min(kBuf, total - base), 0);
+                if ((base > 0 || pb == p0 || total > kBuf) &&
+                    !nb_stage(sh, cpos, base, base + nst, cx0, cy0, cz0, parity, status))
+                    return;
+                const int rows = (nst + 31) >> 5;
+                for (int i = 2 * w; i < pn; i += 2 * kNbWarps) {
+                    const TrialPt t0 = pts[pb + i], t1 = pts[pb + min(i + 1, pn - 1)];
+                    const float3 pf[2] = {make_float3(rel_f(t0.P.x, cx0), rel_f(t0.P.y, cy0), rel_f(t0.P.z, cz0)),
+                                          make_float3(rel_f(t1.P.x, cx0), rel_f(t1.P.y, cy0), rel_f(t1.P.z, cz0))};
+                    uint32_t mask[2];
+                    TrialDrain<F32, SH> D0(sh, t0, R2), D1(sh, t1, R2);
+                    unsigned short *list = sh.list[w];
+                    if constexpr (kOrdered) {
+                        const uint4 P[2] = {t0.P, t1.P};
+                        nb_screen_exact<2>(sh.fl, sh.raw, nst, P, pf, R2, r2hi, wrap, mask);
+                        nb_flush(list, nb_list_ordered(list, mask[0], rows, sh.raw, t0.excl), D0);
+                        if (i + 1 < pn) nb_flush(list, nb_list_ordered(list, mask[1], rows, sh.raw, t1.excl), D1);
+                    } else {
+                        nb_screen<2>(sh.fl, nst, pf, r2hi, wrap, mask);
+                        nb_flush(list, nb_append(list, 0, mask[0], rows, 0), D0);
+                        if (i + 1 < pn) nb_flush(list, nb_append(list, 0, mask[1], rows, 0), D1);
+                    }
+                    // lane 0 gets point i, lane 16 point i + 1
+                    const int k = i + (lane >> 4);
+                    const bool mine = (lane & 15) == 0 && k < pn;
                     if constexpr (F32) {
-                        const FF s = ff_warp_sum(FF{D.eh, D.el});
-                        const float a = warp_sum(D.mag);
-                        if (lane == 0) {
-                            const FF t = ff_add(FF{partf[i].x, partf[i].y}, s);
-                            partf[i] = make_float4(t.hi, t.lo, partf[i].z + a, 0.f);
+                        FF e[2] = {FF{D0.eh, D0.el}, FF{D1.eh, D1.el}};
+                        FF s = warp_sum_many<2>(e);
+                        float a = 0.f;
+                        if constexpr (ABS) {
+                            float keep = lane & 16 ? D1.mag : D0.mag;
+                            a = keep + __shfl_xor_sync(0xffffffffu, lane & 16 ? D0.mag : D1.mag, 16);
+#pragma unroll
+                            for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                        }
+                        if (mine) {
+                            if (base > 0) {
+                                s = ff_add(FF{part[k].x, part[k].y}, s);
+                                a += part[k].z;
+                            }
+                            part[k] = make_float4(s.hi, s.lo, a, 0.f);
                         }
                     } else {
-                        const double e = warp_sum(D.de), a = warp_sum(D.da);
-                        if (lane == 0) {
-                            part[i].x += e;
-                            part[i].y += a;
+                        double e[2] = {D0.de, D1.de}, m[2] = {D0.da, D1.da};
+                        double s = warp_sum_many<2>(e), a = 0.0;
+                        if constexpr (ABS) a = warp_sum_many<2>(m);
+                        if (mine) {
+                            if (base > 0) {
+                                s += part[k].x;
+                                a += part[k].y;
+                            }
+                            part[k] = make_double2(s, a);
                         }
                     }
                 }
@@ -352,15 +495,16 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
                 const int k = pts[pb + i].idx;
                 double e, a;
                 if constexpr (F32) {
-                    e = (double)partf[i].x + (double)partf[i].y;
-                    a = (double)partf[i].z;
+                    e = (double)part[i].x + (double)part[i].y;
+                    a = (double)part[i].z;
                 } else {
                     e = part[i].x;
                     a = part[i].y;
                 }
                 out[k] = e;
-                if (out_abs) out_abs[k] = a;
+                if constexpr (ABS) out_abs[k] = a;
             }
+            __syncthreads();  // the sums are read before the next chunk's
         }
     }
 }
@@ -563,45 +707,42 @@ __global__ void k_trial_place(const TrialPt *__restrict__ tmp, const int32_t *__
 }
 
 // ---- full-system energy ---------------------------------------------------
-// Queue entries of the full-system energy: the staged partner's index in
-// the low 16 bits, the home particle's index in the chunk above them, so
-// that the pairs of several home particles share one evaluation pass.
-template <bool F32>
+// List entries of the full-system energy: the staged partner's index, the
+// home particle's index in the chunk above it, so that the pairs of several
+// home particles share one evaluation pass.
+template <bool F32, class SH>
 struct PairDrain {
-    const NbShared &sh;
+    const SH &sh;
     const uint4 *home;
-    const FieldF &ff;
-    const FieldD &fd;
+    unsigned long long R2;
     float eh = 0.f, el = 0.f, wh = 0.f, wl = 0.f;
-    double de = 0.0, dw = 0.0;
-    __device__ PairDrain(const NbShared &s, const uint4 *h, const FieldF &f, const FieldD &d)
-        : sh(s), home(h), ff(f), fd(d)
+    double de = 0.0, da = 0.0;
+    __device__ PairDrain(const SH &s, const uint4 *h, unsigned long long r) : sh(s), home(h), R2(r) {}
+    __device__ __forceinline__ void operator()(int e)
     {
-    }
-    __device__ __forceinline__ void operator()(int e, bool have)
-    {
-        if (!have) return;
-        const uint4 P = home[e >> 16];
-        const int t = (int)tag_species(P.w);
-        const uint4 r = sh.raw[e & 0xFFFF];
-        const int k = t * kMaxSpecies + (int)tag_species(r.w);
+        const uint4 P = home[e >> 10];
+        const uint4 r = sh.raw[e & 1023];
+        const int k = (int)tag_species(P.w) * kMaxSpecies + (int)tag_species(r.w);
         const int ex = (int)(P.x - r.x), ey = (int)(P.y - r.y), ez = (int)(P.z - r.z);
+        GridSep s;
+        s.dx = ex;
+        s.dy = ey;
+        s.dz = ez;
+        s.g = (unsigned long long)((long long)ex * ex) + (unsigned long long)((long long)ey * ey) +
+              (unsigned long long)((long long)ez * ez);
+        if (s.g >= R2) return;
         if constexpr (F32) {
+            const float4 c = sh.field.f[k];
             float uh, ul, m;
-            lj_ff(ex, ey, ez, ff.c4e[k], ff.c4e_lo[k], ff.sig2[k], ff.sig2_lo[k], uh, ul, m);
+            lj_ff(ex, ey, ez, c.x, c.y, c.z, c.w, uh, ul, m);
             ff_acc(eh, el, uh, ul);
             ff_acc(wh, wl, -fmaf(3.f, m, 9.f * uh), 0.f);  // r U'(r) = -12 rep + 6 att
         } else {
-            GridSep s;
-            s.dx = ex;
-            s.dy = ey;
-            s.dz = ez;
-            s.g = (unsigned long long)((long long)ex * ex) + (unsigned long long)((long long)ey * ey) +
-                  (unsigned long long)((long long)ez * ez);
+            const double2 c = sh.field.d[k];
             double u, m;
-            lj_f64(s, fd.c4e[k], fd.sig2[k], u, m);
+            lj_f64(s, c.x, c.y, u, m);
             de += u;
-            dw -= 3.0 * m + 9.0 * u;
+            da += m;  // r U'(r) = -(3 m + 9 u)
         }
     }
 };
@@ -613,24 +754,28 @@ struct PairDrain {
 template <bool F32>
 __global__ void __launch_bounds__(kNbWarps * 32) k_cell_energy(const uint4 *__restrict__ cpos,
                                                                const int32_t *__restrict__ cs, int T, int64_t ncell,
-                                                               uint64_t R2, float r2lo, float r2hi, bool wrap,
+                                                               uint64_t R2, float r2hi, bool wrap,
                                                                const __grid_constant__ FieldF ff,
                                                                const __grid_constant__ FieldD fd,
                                                                double *__restrict__ partial, int *__restrict__ status)
 {
+    constexpr int NP = 2;  // home particles a warp screens together
     extern __shared__ __align__(128) unsigned char dyn[];
-    NbShared &sh = *reinterpret_cast<NbShared *>(dyn);
+    using SH = NbShared<kBufHalf>;
+    constexpr int kBuf = SH::kBuf;
+    SH &sh = *reinterpret_cast<SH *>(dyn);
     __shared__ double red[kNbWarps][2];
     __shared__ float2 redf[kNbWarps][2];
     __shared__ uint4 home[kPChunk];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (threadIdx.x == 0) mbar_init(&sh.bar, 1);
+    nb_field<F32>(sh, ff, fd);
     __syncthreads();
     unsigned parity = 0;
-    NbQueue Q = {sh.q[w], 0, 0, (1u << lane) - 1u};
+    unsigned short *list = sh.list[w];
     for (int64_t c = blockIdx.x; c < ncell; c += gridDim.x) {
         const int h0 = cs[c], nh = cs[c + 1] - h0;
-        PairDrain<F32> D(sh, home, ff, fd);
+        PairDrain<F32, SH> D(sh, home, R2);
         if (nh > 0) {
             const int cx = (int)(c % T), cy = (int)((c / T) % T), cz = (int)(c / ((int64_t)T * T));
             __syncthreads();
@@ -645,18 +790,33 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_cell_energy(const uint4 *__re
                 for (int base = 0; base < total; base += kBuf) {
                     const int nst = min(kBuf, total - base);
                     if (!nb_stage(sh, cpos, base, base + nst, cx0, cy0, cz0, parity, status)) return;
-                    for (int i = w; i < pn; i += kNbWarps) {
-                        const int hi = pb + i;  // the particle's item index (home items come first)
-                        const uint4 P = home[i];
-                        const float3 pf = make_float3(rel_f(P.x, cx0), rel_f(P.y, cy0), rel_f(P.z, cz0));
-                        nb_screen(sh, nst, P, pf, R2, r2lo, r2hi, wrap, Q,
-                                  [&](int f, uint32_t) {
-                                      const int g = base + f;
-                                      return g < nh && g <= hi;
-                                  },
-                                  D, i << 16);
+                    const int rows = (nst + 31) >> 5;
+                    int n = 0;
+                    for (int i0 = NP * w; i0 < pn; i0 += NP * kNbWarps) {
+                        float3 pf[NP];
+                        uint32_t mask[NP];
+#pragma unroll
+                        for (int p = 0; p < NP; ++p) {
+                            const uint4 P = home[min(i0 + p, pn - 1)];
+                            pf[p] = make_float3(rel_f(P.x, cx0), rel_f(P.y, cy0), rel_f(P.z, cz0));
+                        }
+                        nb_screen<NP>(sh.fl, nst, pf, r2hi, wrap, mask);
+#pragma unroll 1
+                        for (int p = 0; p < NP && i0 + p < pn; ++p) {
+                            uint32_t x = mask[0];
+#pragma unroll
+                            for (int u = 1; u < NP; ++u) x = p == u ? mask[u] : x;
+                            // the home items come first: those up to the particle
+                            // itself (the top bits of the lane's mask) are left out
+                            const int last = pb + i0 + p - base - lane;
+                            if (last >= 0) {
+                                const int out = min(rows, (last >> 5) + 1);
+                                x = out >= rows ? 0u : x & ((1u << (rows - out)) - 1u);
+                            }
+                            n = nb_drain(list, nb_append(list, n, x, rows, (i0 + p) << 10), D);
+                        }
                     }
-                    nb_flush(Q, D);  // before the staged records are replaced
+                    nb_flush(list, n, D);  // before the staged records are replaced
                 }
             }
         }
@@ -675,7 +835,7 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_cell_energy(const uint4 *__re
                 partial[2 * c + threadIdx.x] = (double)sum.hi + (double)sum.lo;
             }
         } else {
-            const double e = warp_sum(D.de), vw = warp_sum(D.dw);
+            const double e = warp_sum(D.de), vw = warp_sum(-(3.0 * D.da + 9.0 * D.de));
             if (lane == 0) {
                 red[w][0] = e;
                 red[w][1] = vw;
@@ -755,26 +915,26 @@ static void sum_partials(gcmc_ctx *ctx, const double *partial, int64_t n, int wi
 // FP32 per lane and FP64 across the warp, the scalars summed in
 // compensated FP32; FP64 mode: FP64 throughout.
 // ---------------------------------------------------------------------------
-template <bool F32, int NS>
+template <bool F32, int NS, class SH>
 struct GradDrain {
     using R = typename std::conditional<F32, float, double>::type;
-    const NbShared &sh;
+    const SH &sh;
     uint4 P;
     int t;
-    const FieldF &ff;
-    const FieldD &fd;
-    R fx = 0, fy = 0, fz = 0;
-    float eh = 0.f, el = 0.f, wh = 0.f, wl = 0.f;  // FP32 mode
-    double de = 0.0, dw = 0.0;                    // FP64 mode
-    R aEps[NS], aSig[NS];
-    __device__ GradDrain(const NbShared &s, const FieldF &f, const FieldD &d) : sh(s), ff(f), fd(d)
+    R fx, fy, fz, aEps[NS], aSig[NS];              // of one home particle
+    float eh = 0.f, el = 0.f, wh = 0.f, wl = 0.f;  // FP32 mode: of all
+    double de = 0.0, dw = 0.0;                    // FP64 mode: of all
+    __device__ GradDrain(const SH &s) : sh(s) {}
+    __device__ __forceinline__ void start(const uint4 &p)
     {
+        P = p;
+        t = (int)tag_species(p.w);
+        fx = fy = fz = 0;
 #pragma unroll
         for (int q = 0; q < NS; ++q) aEps[q] = aSig[q] = 0;
     }
-    __device__ __forceinline__ void operator()(int f, bool have)
+    __device__ __forceinline__ void operator()(int f)
     {
-        if (!have) return;
         const uint4 r = sh.raw[f];
         const int ts = (int)tag_species(r.w);
         const int k = t * kMaxSpecies + ts;
@@ -782,25 +942,27 @@ struct GradDrain {
         const unsigned long long g = (unsigned long long)((long long)ex * ex) +
                                      (unsigned long long)((long long)ey * ey) +
                                      (unsigned long long)((long long)ez * ez);
-        R c4e, s2, coef;
+        R c4e, s2, coef;  // coef: 1 / r^2, then r U'(r) / r^2
         if constexpr (F32) {
+            const float4 c = sh.field.f[k];
             const float r2 = fmaf(__uint2float_rn((uint32_t)(g >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)g));
-            c4e = ff.c4e[k];
-            s2 = ff.sig2[k] / r2;
-            coef = r2;
+            const float y = rcp_approx(r2);
+            c4e = c.x;
+            s2 = c.z / r2;
+            coef = fmaf(fmaf(-r2, y, 1.f), y, y);
         } else {
+            const double2 c = sh.field.d[k];
             const double r2 = u64_to_f64(g);
             double y;
-            c4e = fd.c4e[k];
-            s2 = div_by_g(fd.sig2[k], r2, g, y);
+            c4e = c.x;
+            s2 = div_by_g(c.y, r2, g, y);
             if (g == 0ull) s2 = __longlong_as_double(0x7ff0000000000000ll);
-            coef = fma(fma(-r2, y, 1.0), y, y);  // 1 / r^2
+            coef = fma(fma(-r2, y, 1.0), y, y);
         }
         const R s6 = s2 * s2 * s2;
         const R rep = c4e * s6 * s6, att = c4e * s6;
         const R rdu = (R)(-12) * rep + (R)6 * att;  // r U'(r)
-        if constexpr (F32) coef = rdu / coef;
-        else coef *= rdu;
+        coef *= rdu;
         fx += coef * (R)ex;
         fy += coef * (R)ey;
         fz += coef * (R)ez;
@@ -815,7 +977,7 @@ struct GradDrain {
         const R gs = (R)0.5 * ((R)12 * rep - (R)6 * att);
 #pragma unroll
         for (int q = 0; q < NS; ++q) {
-            if (q == ts) {
+            if (NS == 1 || q == ts) {
                 aEps[q] += ge;
                 aSig[q] += gs;
             }
@@ -823,27 +985,39 @@ struct GradDrain {
     }
 };
 
+// A running sum over the pairs of many particles: float-float in FP32 mode,
+// FP64 in FP64 mode.
+__device__ __forceinline__ void sum_add(FF &a, float x) { a = ff_add_f(a, x); }
+__device__ __forceinline__ void sum_add(double &a, double x) { a += x; }
+__device__ __forceinline__ FF to_sum(float x) { return FF{x, 0.f}; }
+__device__ __forceinline__ double to_sum(double x) { return x; }
+__device__ __forceinline__ double sum_value(FF a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double sum_value(double a) { return a; }
+
 template <bool F32, int NS>
-__global__ void __launch_bounds__(kNbWarps * 32) k_cell_grad(const uint4 *__restrict__ cpos,
+__global__ void __launch_bounds__(kNbWarps * 32, 5) k_cell_grad(const uint4 *__restrict__ cpos,
                                                              const int32_t *__restrict__ cs, int T, int64_t ncell,
-                                                             uint64_t R2, float r2lo, float r2hi, bool wrap, int S,
+                                                             uint64_t R2, float r2hi, bool wrap, int S,
                                                              const __grid_constant__ FieldF ff,
                                                              const __grid_constant__ FieldD fd, double inv_h,
                                                              const int64_t *__restrict__ d_n,
                                                              const int32_t *__restrict__ order, float *__restrict__ dpos,
                                                              double *__restrict__ partial, int *__restrict__ status)
 {
-    constexpr int kW = 2 + 2 * kMaxSpecies * kMaxSpecies;
+    constexpr int kW = 2 + 2 * NS * NS;
+    using Sum = typename std::conditional<F32, FF, double>::type;
     extern __shared__ __align__(128) unsigned char dyn[];
-    NbShared &sh = *reinterpret_cast<NbShared *>(dyn);
+    using SH = NbShared<kBufOrdered>;
+    constexpr int kBuf = SH::kBuf;
+    SH &sh = *reinterpret_cast<SH *>(dyn);
     __shared__ double red[kNbWarps][kW];
-    __shared__ double fpart[kPChunk][3];   // FP64 mode: per-point forces over the passes
-    __shared__ float2 fpartf[kPChunk][3];  // FP32 mode: the same as float-float
+    __shared__ Sum fpart[kPChunk][3];  // per-point forces over the passes
     __shared__ uint4 home[kPChunk];
-    // FP32 mode with up to two species: each warp's scalar sums of a cell in
-    // float-float registers (the same in every lane), written once per cell
-    constexpr bool kRegSums = F32 && NS <= 2;
-    FF sE = {0.f, 0.f}, sW = {0.f, 0.f}, sEp[NS][NS], sSg[NS][NS];
+    // with up to two species the table sums of a cell stay in registers, per
+    // lane, and cross the warp once per cell; with more, once per particle
+    constexpr bool kRegSums = NS <= 2;
+    constexpr int NR = kRegSums ? NS : 1;
+    Sum sEp[NR][NR], sSg[NR][NR];
     __shared__ long long base_s[kMaxSpecies];  // first species-major row of each species
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int width = 2 + 2 * S * S;
@@ -855,120 +1029,79 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_cell_grad(const uint4 *__rest
         }
         mbar_init(&sh.bar, 1);
     }
-    for (int k = threadIdx.x; k < kNbWarps * kW; k += blockDim.x) (&red[0][0])[k] = 0.0;
+    nb_field<F32>(sh, ff, fd);
     __syncthreads();
     unsigned parity = 0;
-    NbQueue Q = {sh.q[w], 0, 0, (1u << lane) - 1u};
+    unsigned short *list = sh.list[w];
     for (int64_t c = blockIdx.x; c < ncell; c += gridDim.x) {
         const int h0 = cs[c], nh = cs[c + 1] - h0;
-        if constexpr (kRegSums) {
-            sE = sW = FF{0.f, 0.f};
+        for (int k = lane; k < width; k += 32) red[w][k] = 0.0;
+        __syncwarp();
+        GradDrain<F32, NS, SH> D(sh);
 #pragma unroll
-            for (int a = 0; a < NS; ++a)
+        for (int a = 0; a < NR; ++a)
 #pragma unroll
-                for (int q = 0; q < NS; ++q) sEp[a][q] = sSg[a][q] = FF{0.f, 0.f};
-        }
+            for (int q = 0; q < NR; ++q) sEp[a][q] = sSg[a][q] = Sum{};
         if (nh > 0) {
             const int cx = (int)(c % T), cy = (int)((c / T) % T), cz = (int)(c / ((int64_t)T * T));
-            __syncthreads();
             if (w == 0) runs27(cs, T, cx, cy, cz, sh.runs);
             __syncthreads();
             const int total = sh.runs.end[17];
+            // the home cell lies in the middle row's first run
+            const int own = sh.runs.end[3] + h0 - sh.runs.start[4];
             const uint32_t cx0 = cell_centre(cx, T), cy0 = cell_centre(cy, T), cz0 = cell_centre(cz, T);
             for (int pb = 0; pb < nh; pb += kPChunk) {
                 const int pn = min(kPChunk, nh - pb);
                 __syncthreads();
-                for (int i = threadIdx.x; i < pn; i += blockDim.x) {
-                    home[i] = cpos[h0 + pb + i];
-                    if constexpr (F32) fpartf[i][0] = fpartf[i][1] = fpartf[i][2] = make_float2(0.f, 0.f);
-                    else fpart[i][0] = fpart[i][1] = fpart[i][2] = 0.0;
-                }
+                for (int i = threadIdx.x; i < pn; i += blockDim.x) home[i] = cpos[h0 + pb + i];
                 for (int base = 0; base < total; base += kBuf) {
                     const int nst = min(kBuf, total - base);
                     if (!nb_stage(sh, cpos, base, base + nst, cx0, cy0, cz0, parity, status)) return;
-                    for (int i = w; i < pn; i += kNbWarps) {
-                        GradDrain<F32, NS> D(sh, ff, fd);
-                        D.P = home[i];
-                        D.t = (int)tag_species(D.P.w);
-                        const uint32_t self = D.P.w;
-                        const float3 pf =
-                            make_float3(rel_f(D.P.x, cx0), rel_f(D.P.y, cy0), rel_f(D.P.z, cz0));
-                        nb_screen(sh, nst, D.P, pf, R2, r2lo, r2hi, wrap, Q,
-                                  [&](int, uint32_t tag) { return tag == self; }, D);
-                        nb_flush(Q, D);
-                        // FP32 mode reduces across the warp and accumulates in
-                        // float-float (the FP64 pipe is a small fraction of the
-                        // FP32 one); FP64 mode in FP64
-                        if constexpr (F32) {
-                            const FF gx = ff_warp_sum(FF{D.fx, 0.f}), gy = ff_warp_sum(FF{D.fy, 0.f}),
-                                     gz = ff_warp_sum(FF{D.fz, 0.f});
-                            const FF vE = ff_warp_sum(FF{D.eh, D.el}), vW = ff_warp_sum(FF{D.wh, D.wl});
-                            if (lane == 0) {
-                                const FF ox = ff_add(FF{fpartf[i][0].x, fpartf[i][0].y}, gx);
-                                const FF oy = ff_add(FF{fpartf[i][1].x, fpartf[i][1].y}, gy);
-                                const FF oz = ff_add(FF{fpartf[i][2].x, fpartf[i][2].y}, gz);
-                                fpartf[i][0] = make_float2(ox.hi, ox.lo);
-                                fpartf[i][1] = make_float2(oy.hi, oy.lo);
-                                fpartf[i][2] = make_float2(oz.hi, oz.lo);
-                            }
+                    const int rows = (nst + 31) >> 5;
+                    for (int i0 = 2 * w; i0 < pn; i0 += 2 * kNbWarps) {
+                        uint4 P[2];
+                        float3 pf[2];
+                        uint32_t mask[2];
+#pragma unroll
+                        for (int p = 0; p < 2; ++p) {
+                            P[p] = home[min(i0 + p, pn - 1)];
+                            pf[p] = make_float3(rel_f(P[p].x, cx0), rel_f(P[p].y, cy0), rel_f(P[p].z, cz0));
+                        }
+                        nb_screen_exact<2>(sh.fl, sh.raw, nst, P, pf, R2, r2hi, wrap, mask);
+#pragma unroll 1
+                        for (int i = i0; i < min(i0 + 2, pn); ++i) {
+                            D.start(home[i]);
+                            uint32_t x = i == i0 ? mask[0] : mask[1];
+                            const int self = own + pb + i - base;  // the particle's own record
+                            if (self >= 0 && self < nst && (self & 31) == lane) x &= ~(1u << (rows - 1 - (self >> 5)));
+                            nb_flush(list, nb_list_ordered(list, x, rows, sh.raw, 0xFFFFFFFFu), D);
+                            // lanes 0, 8, 16 get the force's x, y, z
+                            Sum f[4] = {to_sum(D.fx), to_sum(D.fy), to_sum(D.fz), Sum{}};
+                            const Sum force = warp_sum_many<4>(f);
+                            if ((lane & 7) == 0 && lane < 24)
+                                fpart[i][lane >> 3] = base > 0 ? sum_of(fpart[i][lane >> 3], force) : force;
                             if constexpr (kRegSums) {
-                                sE = ff_add(sE, vE);
-                                sW = ff_add(sW, vW);
 #pragma unroll
-                                for (int q = 0; q < NS; ++q) {
-                                    const FF ve = ff_warp_sum(FF{D.aEps[q], 0.f});
-                                    const FF vs = ff_warp_sum(FF{D.aSig[q], 0.f});
+                                for (int t = 0; t < NR; ++t) {
+                                    if (NR == 1 || t == D.t) {  // the same in every lane
 #pragma unroll
-                                    for (int tt = 0; tt < NS; ++tt) {
-                                        if (tt == D.t) {
-                                            sEp[tt][q] = ff_add(sEp[tt][q], ve);
-                                            sSg[tt][q] = ff_add(sSg[tt][q], vs);
+                                        for (int q = 0; q < NR; ++q) {
+                                            sum_add(sEp[t][q], D.aEps[q]);
+                                            sum_add(sSg[t][q], D.aSig[q]);
                                         }
                                     }
                                 }
                             } else {
-                                double ve[NS], vs[NS];
+                                Sum v[2 * NS];
 #pragma unroll
                                 for (int q = 0; q < NS; ++q) {
-                                    FF x = ff_warp_sum(FF{D.aEps[q], 0.f}), y = ff_warp_sum(FF{D.aSig[q], 0.f});
-                                    ve[q] = (double)x.hi + (double)x.lo;
-                                    vs[q] = (double)y.hi + (double)y.lo;
+                                    v[q] = to_sum(D.aEps[q]);
+                                    v[NS + q] = to_sum(D.aSig[q]);
                                 }
-                                if (lane == 0) {
-                                    red[w][0] += (double)vE.hi + (double)vE.lo;
-                                    red[w][1] += (double)vW.hi + (double)vW.lo;
-#pragma unroll
-                                    for (int q = 0; q < NS; ++q) {
-                                        if (q < S) {
-                                            red[w][2 + D.t * S + q] += ve[q];
-                                            red[w][2 + S * S + D.t * S + q] += vs[q];
-                                        }
-                                    }
-                                }
-                            }
-                        } else {
-                            const double gx = warp_sum((double)D.fx), gy = warp_sum((double)D.fy),
-                                         gz = warp_sum((double)D.fz);
-                            const double vE = warp_sum(D.de), vW = warp_sum(D.dw);
-                            double ve[NS], vs[NS];
-#pragma unroll
-                            for (int q = 0; q < NS; ++q) {
-                                ve[q] = q < S ? warp_sum((double)D.aEps[q]) : 0.0;
-                                vs[q] = q < S ? warp_sum((double)D.aSig[q]) : 0.0;
-                            }
-                            if (lane == 0) {
-                                fpart[i][0] += gx;
-                                fpart[i][1] += gy;
-                                fpart[i][2] += gz;
-                                red[w][0] += vE;
-                                red[w][1] += vW;
-#pragma unroll
-                                for (int q = 0; q < NS; ++q) {
-                                    if (q < S) {
-                                        red[w][2 + D.t * S + q] += ve[q];
-                                        red[w][2 + S * S + D.t * S + q] += vs[q];
-                                    }
-                                }
+                                const Sum x = warp_sum_many<2 * NS>(v);
+                                const int k = lane / (16 / NS), q = k % NS;
+                                if (lane % (16 / NS) == 0 && q < S)
+                                    red[w][2 + (k >= NS ? S * S : 0) + D.t * S + q] += sum_value(x);
                             }
                         }
                     }
@@ -978,43 +1111,47 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_cell_grad(const uint4 *__rest
                     for (int i = threadIdx.x; i < pn; i += blockDim.x) {
                         const uint32_t tg = home[i].w;
                         const int64_t row = order ? order[h0 + pb + i] : base_s[tag_species(tg)] + tag_index(tg);
-                        if constexpr (F32) {
-                            const float ih = (float)inv_h;
-                            dpos[3 * row + 0] = (fpartf[i][0].x + fpartf[i][0].y) * ih;
-                            dpos[3 * row + 1] = (fpartf[i][1].x + fpartf[i][1].y) * ih;
-                            dpos[3 * row + 2] = (fpartf[i][2].x + fpartf[i][2].y) * ih;
-                        } else {
-                            dpos[3 * row + 0] = (float)(fpart[i][0] * inv_h);
-                            dpos[3 * row + 1] = (float)(fpart[i][1] * inv_h);
-                            dpos[3 * row + 2] = (float)(fpart[i][2] * inv_h);
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            if constexpr (F32) dpos[3 * row + a] = (fpart[i][a].hi + fpart[i][a].lo) * (float)inv_h;
+                            else dpos[3 * row + a] = (float)(fpart[i][a] * inv_h);
                         }
                     }
                 }
             }
         }
-        if constexpr (kRegSums) {
-            if (lane == 0) {
-                red[w][0] = (double)sE.hi + (double)sE.lo;
-                red[w][1] = (double)sW.hi + (double)sW.lo;
-#pragma unroll
-                for (int a2 = 0; a2 < NS; ++a2)
-#pragma unroll
-                    for (int q = 0; q < NS; ++q) {
-                        if (a2 < S && q < S) {
-                            red[w][2 + a2 * S + q] = (double)sEp[a2][q].hi + (double)sEp[a2][q].lo;
-                            red[w][2 + S * S + a2 * S + q] = (double)sSg[a2][q].hi + (double)sSg[a2][q].lo;
-                        }
-                    }
+        {
+            Sum v[2];
+            if constexpr (F32) {
+                v[0] = FF{D.eh, D.el};
+                v[1] = FF{D.wh, D.wl};
+            } else {
+                v[0] = D.de;
+                v[1] = D.dw;
             }
+            const Sum x = warp_sum_many<2>(v);
+            if ((lane & 15) == 0) red[w][lane >> 4] = sum_value(x);
+        }
+        if constexpr (kRegSums) {
+            Sum v[2 * NR * NR];
+#pragma unroll
+            for (int a = 0; a < NR; ++a)
+#pragma unroll
+                for (int q = 0; q < NR; ++q) {
+                    v[a * NR + q] = sEp[a][q];
+                    v[NR * NR + a * NR + q] = sSg[a][q];
+                }
+            const Sum x = warp_sum_many<2 * NR * NR>(v);  // NR == S
+            constexpr int kLanes = 16 / (NR * NR);
+            if (lane % kLanes == 0) red[w][2 + lane / kLanes] = sum_value(x);
         }
         __syncthreads();
-        if (threadIdx.x < width) {
+        for (int j = threadIdx.x; j < width; j += blockDim.x) {
             double s = 0.0;
-            for (int k = 0; k < kNbWarps; ++k) s += red[k][threadIdx.x];
-            partial[c * width + threadIdx.x] = s;
+            for (int k = 0; k < kNbWarps; ++k) s += red[k][j];
+            partial[c * width + j] = s;
         }
         __syncthreads();
-        for (int k = threadIdx.x; k < kNbWarps * kW; k += blockDim.x) (&red[0][0])[k] = 0.0;
     }
 }
 
@@ -1026,15 +1163,14 @@ static unsigned blocks_for(gcmc_ctx *ctx, int64_t work, int per_block)
     return (unsigned)(b < 1 ? 1 : b);
 }
 
-// The screen's band around the grid cutoff R2: FP32 squared distances below
-// r2lo are inside, above r2hi outside; in between the exact integer test
-// decides.  The FP32 separations carry a relative error below 1e-6 of the
-// cell edge (coordinates relative to the cell centre), far inside the band.
+// The screen's bound above the grid cutoff R2: FP32 squared distances above
+// r2hi are outside; below it the exact integer test decides.  The FP32
+// separations carry a relative error below 1e-6 of the cell edge (coordinates
+// relative to the cell centre), far inside the margin.
 // wrap: the cells are narrower than rc (2 rc <= L < 3 rc), so the FP32
 // separations need their own periodic wrap.
-static void screen_band(const gcmc_ctx *ctx, float &r2lo, float &r2hi, bool &wrap)
+static void screen_bound(const gcmc_ctx *ctx, float &r2hi, bool &wrap)
 {
-    r2lo = (float)((double)ctx->R2 * (1.0 - 1e-5));
     r2hi = (float)((double)ctx->R2 * (1.0 + 1e-5));
     wrap = (double)ctx->T * ctx->rc > ctx->L;
 }
@@ -1049,10 +1185,10 @@ static unsigned nb_blocks(const gcmc_ctx *ctx, int64_t cells)
 
 // The neighbourhood kernels take more than 48 KB of shared memory.
 template <typename K>
-static gcmc_status nb_smem(gcmc_ctx *ctx, K kern)
+static gcmc_status nb_smem(gcmc_ctx *ctx, K kern, size_t bytes)
 {
     const cudaError_t e =
-        cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NbShared));
+        cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute (neighbourhood kernel)");
     return GCMC_OK;
 }
@@ -1065,10 +1201,10 @@ gcmc_status trial_energy(gcmc_ctx *ctx, const double *pos, const int32_t *specie
     if (m <= 0) return GCMC_OK;
     if (m > (int64_t)INT32_MAX) return fail(ctx, GCMC_ERR_INVALID_ARG, "gcmc_trial_energy: too many points");
     cudaStream_t s = ctx->stream;
-    float r2lo, r2hi;
+    float r2hi;
     bool wrap;
-    screen_band(ctx, r2lo, r2hi, wrap);
-    if (m <= kDirectPoints) {
+    screen_bound(ctx, r2hi, wrap);
+    if (m <= kDirectPoints && !(out_abs && ctx->precision == GCMC_FP32)) {
         st = ensure_pinned(ctx, kPinnedBytes);
         if (st != GCMC_OK) return st;
         // the status word lies in pinned host memory, written by the kernel
@@ -1117,19 +1253,20 @@ gcmc_status trial_energy(gcmc_ctx *ctx, const double *pos, const int32_t *specie
     if (st != GCMC_OK) return st;
     k_trial_place<<<gb, 256, 0, s>>>(tmp, cid, m, ps, fill, pts);
     const unsigned nb = nb_blocks(ctx, ncell);
-    if (ctx->precision == GCMC_FP32) {
-        st = nb_smem(ctx, k_trial_energy<true>);
-        if (st != GCMC_OK) return st;
-        k_trial_energy<true><<<nb, kNbWarps * 32, sizeof(NbShared), s>>>(
-            pts, ps, ctx->cpos, ctx->cell_start, ctx->T, ncell, ctx->R2, r2lo, r2hi, wrap, ctx->ff, ctx->fd, out, out_abs,
-            ctx->d_status);
-    } else {
-        st = nb_smem(ctx, k_trial_energy<false>);
-        if (st != GCMC_OK) return st;
-        k_trial_energy<false><<<nb, kNbWarps * 32, sizeof(NbShared), s>>>(
-            pts, ps, ctx->cpos, ctx->cell_start, ctx->T, ncell, ctx->R2, r2lo, r2hi, wrap, ctx->ff, ctx->fd, out, out_abs,
-            ctx->d_status);
-    }
+    auto launch = [&](auto kern, size_t smem) {
+        gcmc_status r = nb_smem(ctx, kern, smem);
+        if (r == GCMC_OK)
+            kern<<<nb, kNbWarps * 32, smem, s>>>(pts, ps, ctx->cpos, ctx->cell_start, ctx->T, ncell, ctx->R2, r2hi, wrap,
+                                                 ctx->ff, ctx->fd, out, out_abs, ctx->d_status);
+        return r;
+    };
+    if (ctx->precision == GCMC_FP32)
+        st = out_abs ? launch(k_trial_energy<true, true>, sizeof(NbShared<kBufOrdered>))
+                     : launch(k_trial_energy<true, false>, sizeof(NbShared<kBufFull>));
+    else
+        st = out_abs ? launch(k_trial_energy<false, true>, sizeof(NbShared<kBufFull>))
+                     : launch(k_trial_energy<false, false>, sizeof(NbShared<kBufFull>));
+    if (st != GCMC_OK) return st;
     ctx->launches += 3;
     GCMC_CUDA(ctx, cudaGetLastError());
     int bits = 0;
@@ -1150,22 +1287,22 @@ gcmc_status total_energy_begin(gcmc_ctx *ctx, bool virial_only)
     if (st != GCMC_OK) return st;
     st = ensure_pinned(ctx, kPinnedBytes);
     if (st != GCMC_OK) return st;
-    float r2lo, r2hi;
+    float r2hi;
     bool wrap;
-    screen_band(ctx, r2lo, r2hi, wrap);
+    screen_bound(ctx, r2hi, wrap);
     const unsigned nb = nb_blocks(ctx, ctx->ncell);
     GCMC_CUDA(ctx, cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->stream));
     if (ctx->precision == GCMC_FP32) {
-        st = nb_smem(ctx, k_cell_energy<true>);
+        st = nb_smem(ctx, k_cell_energy<true>, sizeof(NbShared<kBufHalf>));
         if (st != GCMC_OK) return st;
-        k_cell_energy<true><<<nb, kNbWarps * 32, sizeof(NbShared), ctx->stream>>>(
-            ctx->cpos, ctx->cell_start, ctx->T, ctx->ncell, ctx->R2, r2lo, r2hi, wrap, ctx->ff, ctx->fd, ctx->d_red,
+        k_cell_energy<true><<<nb, kNbWarps * 32, sizeof(NbShared<kBufHalf>), ctx->stream>>>(
+            ctx->cpos, ctx->cell_start, ctx->T, ctx->ncell, ctx->R2, r2hi, wrap, ctx->ff, ctx->fd, ctx->d_red,
             ctx->d_status);
     } else {
-        st = nb_smem(ctx, k_cell_energy<false>);
+        st = nb_smem(ctx, k_cell_energy<false>, sizeof(NbShared<kBufHalf>));
         if (st != GCMC_OK) return st;
-        k_cell_energy<false><<<nb, kNbWarps * 32, sizeof(NbShared), ctx->stream>>>(
-            ctx->cpos, ctx->cell_start, ctx->T, ctx->ncell, ctx->R2, r2lo, r2hi, wrap, ctx->ff, ctx->fd, ctx->d_red,
+        k_cell_energy<false><<<nb, kNbWarps * 32, sizeof(NbShared<kBufHalf>), ctx->stream>>>(
+            ctx->cpos, ctx->cell_start, ctx->T, ctx->ncell, ctx->R2, r2hi, wrap, ctx->ff, ctx->fd, ctx->d_red,
             ctx->d_status);
     }
     sum_partials(ctx, ctx->d_red, ctx->ncell, 2, ctx->d_red + 2 * ctx->ncell + 8, ctx->d_red + 2 * ctx->ncell);
@@ -1221,28 +1358,30 @@ gcmc_status energy_grad_begin(gcmc_ctx *ctx, float *dpos, bool input_order)
     if (st != GCMC_OK) return st;
     st = ensure_pinned(ctx, kPinnedBytes);
     if (st != GCMC_OK) return st;
-    float r2lo, r2hi;
+    float r2hi;
     bool wrap;
-    screen_band(ctx, r2lo, r2hi, wrap);
+    screen_bound(ctx, r2hi, wrap);
     const unsigned nb = nb_blocks(ctx, ctx->ncell);
     double *part = ctx->d_red;
     double *res = ctx->d_red + (size_t)ctx->ncell * width;
     GCMC_CUDA(ctx, cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->stream));
 #define GCMC_GRAD(F, NSP)                                                                                     \
     do {                                                                                                      \
-        st = nb_smem(ctx, k_cell_grad<F, NSP>);                                                               \
+        st = nb_smem(ctx, k_cell_grad<F, NSP>, sizeof(NbShared<kBufOrdered>));                                \
         if (st != GCMC_OK) return st;                                                                         \
-        k_cell_grad<F, NSP><<<nb, kNbWarps * 32, sizeof(NbShared), ctx->stream>>>(                            \
-            ctx->cpos, ctx->cell_start, ctx->T, ctx->ncell, ctx->R2, r2lo, r2hi, wrap, S, ctx->ff, ctx->fd,    \
+        k_cell_grad<F, NSP><<<nb, kNbWarps * 32, sizeof(NbShared<kBufOrdered>), ctx->stream>>>(               \
+            ctx->cpos, ctx->cell_start, ctx->T, ctx->ncell, ctx->R2, r2hi, wrap, S, ctx->ff, ctx->fd,          \
             1.0 / ctx->h, ctx->d_n, input_order ? ctx->order : nullptr, dpos, part, ctx->d_status);           \
     } while (0)
     if (ctx->precision == GCMC_FP32) {
         if (S == 1) GCMC_GRAD(true, 1);
         else if (S == 2) GCMC_GRAD(true, 2);
+        else if (S <= 4) GCMC_GRAD(true, 4);
         else GCMC_GRAD(true, kMaxSpecies);
     } else {
         if (S == 1) GCMC_GRAD(false, 1);
         else if (S == 2) GCMC_GRAD(false, 2);
+        else if (S <= 4) GCMC_GRAD(false, 4);
         else GCMC_GRAD(false, kMaxSpecies);
     }
 #undef GCMC_GRAD
