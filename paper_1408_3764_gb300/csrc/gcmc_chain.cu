@@ -615,7 +615,7 @@ struct Mover {
             s.dz = p.z;
             s.g = g2;
             double u, m;
-            lj_f64(s, a.fd.c4e[k], a.fd.sig2[k], u, m);
+            lj_f64(s, a.fd.rep[k], a.fd.att[k], u, m);
             o.de += neg ? -u : u;
             o.da += m;
             if (VIR) {

@@ -91,6 +91,26 @@ static void free_device(gcmc_ctx *ctx)
     ctx->scratch_bytes = ctx->d_red_len = ctx->h_pinned_bytes = 0;
 }
 
+// 4 eps (sigma / h)^12 and 4 eps (sigma / h)^6 with h = L / 2^32, rounded once:
+// double-length products (Dekker), as every pair of the species shares the
+// error.
+struct Double2 {
+    double hi, lo;
+};
+static Double2 mul2(Double2 a, Double2 b)
+{
+    const double p = a.hi * b.hi;
+    return Double2{p, std::fma(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi)};
+}
+static void pair_constants(double eps, double sigma, double L, double &rep, double &att)
+{
+    const double s = sigma * 4294967296.0, r = s / L;
+    const Double2 x{r, std::fma(-r, L, s) / L};
+    const Double2 x3 = mul2(mul2(x, x), x), x6 = mul2(x3, x3), x12 = mul2(x6, x6);
+    rep = 4.0 * eps * x12.hi + 4.0 * eps * x12.lo;
+    att = 4.0 * eps * x6.hi + 4.0 * eps * x6.lo;
+}
+
 }  // namespace gcmc
 
 using namespace gcmc;
@@ -149,6 +169,7 @@ gcmc_status gcmc_create(const gcmc_params *p, void *stream, gcmc_ctx **out)
             const double sg = s * ctx->q;
             ctx->fd.c4e[a * kMaxSpecies + b] = 4.0 * e;
             ctx->fd.sig2[a * kMaxSpecies + b] = sg * sg;
+            pair_constants(e, s, p->L, ctx->fd.rep[a * kMaxSpecies + b], ctx->fd.att[a * kMaxSpecies + b]);
             ctx->ff.c4e[a * kMaxSpecies + b] = (float)(4.0 * e);
             ctx->ff.sig2[a * kMaxSpecies + b] = (float)(sg * sg);
             ctx->ff.c4e_lo[a * kMaxSpecies + b] = (float)(4.0 * e - (double)(float)(4.0 * e));

@@ -196,6 +196,8 @@ struct FieldF {
 struct FieldD {
     double c4e[kMaxSpecies * kMaxSpecies];
     double sig2[kMaxSpecies * kMaxSpecies];
+    double rep[kMaxSpecies * kMaxSpecies];  // 4 eps (sigma / h)^12
+    double att[kMaxSpecies * kMaxSpecies];  // 4 eps (sigma / h)^6
 };
 
 // Pair energy in FP32 from an exact grid separation known to be inside the
@@ -303,51 +305,77 @@ __device__ __forceinline__ void ff_acc(float &hi, float &lo, float xh, float xl)
     lo = __fadd_rn(lo, __fadd_rn(e, xl));
 }
 
-// g (< 2^63) as the nearest double, from its halves: 2^84 + 2^32 gh and
-// 2^52 + gl are assembled from bits, their offsets cancel exactly in the
-// first subtraction, and the last addition rounds once.
+// g (0 < g < 2^63) rounded to a double, in integer operations (the FP64 pipe
+// bounds the kernels that need it): the leading bit moved to bit 62, the low
+// ten bits rounded off, the exponent added above the 53-bit mantissa, whose
+// own leading bit -- or a carry of the rounding -- counts into it.
 __device__ __forceinline__ double u64_to_f64(unsigned long long g)
 {
-    const double hi = __hiloint2double(0x45300000, (int)(uint32_t)(g >> 32));
-    const double lo = __hiloint2double(0x43300000, (int)(uint32_t)g);
-    return (hi - 19342813118337666422669312.0) + lo;  // 2^84 + 2^52
+    const int n = __clzll((long long)g) - 1;
+    const unsigned long long m = ((g << n) + 0x200ull) >> 10;  // times 2^(10 - n)
+    return __longlong_as_double((long long)(m + ((unsigned long long)(1084 - n) << 52)));
 }
 
-// a / r2 for r2 = u64_to_f64(g) >= 1 and a > 0, and an approximate reciprocal
-// (to about 2^-44) in y: a seed from the FP32 reciprocal (to about 2^-22,
-// widened by moving its bits), one Newton step, and the quotient corrected by
-// its residual, which leaves one rounding.
-__device__ __forceinline__ double div_by_g(double a, double r2, unsigned long long g, double &y)
+// An approximate 1 / r2 for r2 = u64_to_f64(g): the FP32 reciprocal (to about
+// 2^-22), widened by moving its bits.
+__device__ __forceinline__ double rcp_seed(unsigned long long g)
 {
     const uint32_t b = __float_as_uint(
         rcp_approx(fmaf(__uint2float_rn((uint32_t)(g >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)g))));
-    const double y0 = __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+
+// a / r2 for r2 = u64_to_f64(g) >= 1 and a > 0, and an approximate reciprocal
+// (to about 2^-44) in y: the seed, one Newton step, and the quotient corrected
+// by its residual, which leaves one rounding.
+__device__ __forceinline__ double div_by_g(double a, double r2, unsigned long long g, double &y)
+{
+    const double y0 = rcp_seed(g);
     y = fma(fma(-r2, y0, 1.0), y0, y0);
     const double q = a * y0;
     return fma(fma(-q, r2, a), y, q);
 }
 
-// Pair energy in FP64.  The FP64 pipe bounds the kernels that evaluate it (a
-// warp instruction per 16 cycles and SM), so its instructions are counted: 12
-// here, where conversions of the three differences, their squares and a
-// general division took 26.  The squared distance is the exact integer g.
-// 50,001 trial energies among 131,072 particles 355 -> 280 us a call, the total
-// energy of 87,296 particles with its cell build 401 -> 344 us, errors against
-// 64-bit sums as before (1.3e-15).
-__device__ __forceinline__ void lj_f64(const GridSep &s, double c4e, double sig2, double &u,
-                                       double &mag)
+// r^-6 and r^-12 in grid units from the exact squared distance (g > 0): six
+// instructions of the FP64 pipe, the third-order step y0 (1 + e + e^2) on the
+// seed among them.  The FP64 pipe bounds the kernels that evaluate pairs (a
+// warp instruction per 16 cycles and SM), so its instructions are counted: a
+// pair's energy takes 8 where its terms are summed apart and 9 below; with the
+// conversions of the three differences, their squares and a general division
+// it took 26.  50,001 trial energies among 131,072 particles 355 -> 202 us a
+// call, the total energy of 87,296 particles with its cell build 397 -> 259 us;
+// error of the former against 64-bit sums 1.3e-15 -> 5.5e-16.
+__device__ __forceinline__ void inv_powers(unsigned long long g, double &y3, double &y6)
 {
-    const double r2 = u64_to_f64(s.g);
-    double y;
-    const double s2 = div_by_g(sig2, r2, s.g, y);
-    const double s6 = s2 * s2 * s2;
-    const double att = c4e * s6;
-    u = fma(att, s6, -att);
-    mag = fma(att, s6, att);
+    const double r2 = u64_to_f64(g), y0 = rcp_seed(g);
+    const double e = fma(-r2, y0, 1.0);
+    const double y = fma(y0, fma(e, e, e), y0);
+    y3 = y * y * y;
+    y6 = y3 * y3;
+}
+
+// Pair energy u and |rep| + |att| in FP64 from the pair's constants rep and att
+// (FieldD).
+__device__ __forceinline__ void lj_f64(const GridSep &s, double rep, double att, double &u, double &mag)
+{
+    double y3, y6;
+    inv_powers(s.g, y3, y6);
+    const double a = att * y3;
+    u = fma(rep, y6, -a);
+    mag = fma(rep, y6, a);
     if (s.g == 0ull) {
         u = __longlong_as_double(0x7ff0000000000000ll);
         mag = u;
     }
+}
+
+// The same added to the sums of the two terms (g == 0: +inf and nothing).
+__device__ __forceinline__ void lj_f64_add(unsigned long long g, double rep, double att, double &sum_rep, double &sum_att)
+{
+    double y3, y6;
+    inv_powers(g, y3, y6);
+    sum_rep = g == 0ull ? __longlong_as_double(0x7ff0000000000000ll) : fma(rep, y6, sum_rep);
+    sum_att = g == 0ull ? sum_att : fma(att, y3, sum_att);
 }
 
 // Float-float values (hi + lo) and their sums (TwoSum on the high words).

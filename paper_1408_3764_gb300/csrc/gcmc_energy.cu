@@ -67,7 +67,7 @@ __device__ __forceinline__ void pair_acc(const uint4 &p, const uint4 &q, uint32_
         acc.add(u, m);
     } else {
         double u, m;
-        lj_f64(s, fd.c4e[k], fd.sig2[k], u, m);
+        lj_f64(s, fd.rep[k], fd.att[k], u, m);
         acc.add(u, m);
     }
 }
@@ -137,19 +137,20 @@ struct __align__(16) NbShared {
     RunList runs;
     uint64_t bar;
     // the species pairs' constants: FP32 mode float4 (c4e, c4e_lo, sig2,
-    // sig2_lo), FP64 mode (c4e, sig2) -- lanes of one warp read several
+    // sig2_lo), FP64 mode (rep, att), for the gradient (c4e, sig2) -- lanes of
+    // one warp read several
     union {
         float4 f[kMaxSpecies * kMaxSpecies];
         double2 d[kMaxSpecies * kMaxSpecies];
     } field;
 };
 
-template <bool F32, int KB>
+template <bool F32, bool GRAD, int KB>
 __device__ __forceinline__ void nb_field(NbShared<KB> &sh, const FieldF &ff, const FieldD &fd)
 {
     for (int k = threadIdx.x; k < kMaxSpecies * kMaxSpecies; k += blockDim.x) {
         if constexpr (F32) sh.field.f[k] = make_float4(ff.c4e[k], ff.c4e_lo[k], ff.sig2[k], ff.sig2_lo[k]);
-        else sh.field.d[k] = make_double2(fd.c4e[k], fd.sig2[k]);
+        else sh.field.d[k] = GRAD ? make_double2(fd.c4e[k], fd.sig2[k]) : make_double2(fd.rep[k], fd.att[k]);
     }
 }
 
@@ -365,7 +366,7 @@ struct TrialDrain {
     uint32_t excl;
     unsigned long long R2;
     float eh = 0.f, el = 0.f, mag = 0.f;
-    double de = 0.0, da = 0.0;
+    double rep = 0.0, att = 0.0;
     __device__ TrialDrain(const SH &s, const TrialPt &p, unsigned long long r) : sh(s), P(p.P), excl(p.excl), R2(r)
     {
     }
@@ -373,13 +374,10 @@ struct TrialDrain {
     {
         const uint4 r = sh.raw[f];
         const int ex = (int)(P.x - r.x), ey = (int)(P.y - r.y), ez = (int)(P.z - r.z);
-        GridSep s;
-        s.dx = ex;
-        s.dy = ey;
-        s.dz = ez;
-        s.g = (unsigned long long)((long long)ex * ex) + (unsigned long long)((long long)ey * ey) +
-              (unsigned long long)((long long)ez * ez);
-        if (s.g >= R2 || r.w == excl) return;
+        const unsigned long long g = (unsigned long long)((long long)ex * ex) +
+                                     (unsigned long long)((long long)ey * ey) +
+                                     (unsigned long long)((long long)ez * ez);
+        if (g >= R2 || r.w == excl) return;
         const int k = (int)P.w * kMaxSpecies + (int)tag_species(r.w);
         if constexpr (F32) {
             const float4 c = sh.field.f[k];
@@ -389,10 +387,7 @@ struct TrialDrain {
             mag += m;
         } else {
             const double2 c = sh.field.d[k];
-            double u, m;
-            lj_f64(s, c.x, c.y, u, m);
-            de += u;
-            da += m;
+            lj_f64_add(g, c.x, c.y, rep, att);
         }
     }
 };
@@ -419,7 +414,7 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
     __shared__ typename std::conditional<F32, float4, double2>::type part[kPChunk];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (threadIdx.x == 0) mbar_init(&sh.bar, 1);
-    nb_field<F32>(sh, ff, fd);
+    nb_field<F32, false>(sh, ff, fd);
     __syncthreads();
     unsigned parity = 0;
     for (int64_t c = blockIdx.x; c < ncell; c += gridDim.x) {
@@ -477,7 +472,7 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
                             part[k] = make_float4(s.hi, s.lo, a, 0.f);
                         }
                     } else {
-                        double e[2] = {D0.de, D1.de}, m[2] = {D0.da, D1.da};
+                        double e[2] = {D0.rep - D0.att, D1.rep - D1.att}, m[2] = {D0.rep + D0.att, D1.rep + D1.att};
                         double s = warp_sum_many<2>(e), a = 0.0;
                         if constexpr (ABS) a = warp_sum_many<2>(m);
                         if (mine) {
@@ -564,18 +559,15 @@ __global__ void __launch_bounds__(kDirectWarps * 32) k_trial_direct(
     const unsigned lt = (1u << lane) - 1u;
     int head = 0, nq = 0;
     float eh = 0.f, el = 0.f, mag = 0.f;
-    double de = 0.0, da = 0.0;
+    double rep = 0.0, att = 0.0;
     auto drain = [&](int n) {
         __syncwarp();
         if (lane < n) {
             const int4 p = Q[(head + lane) & (kNbQ - 1)];
-            GridSep s;
-            s.dx = p.x;
-            s.dy = p.y;
-            s.dz = p.z;
-            s.g = (unsigned long long)((long long)p.x * p.x) + (unsigned long long)((long long)p.y * p.y) +
-                  (unsigned long long)((long long)p.z * p.z);
-            if (s.g < R2) {
+            const unsigned long long g = (unsigned long long)((long long)p.x * p.x) +
+                                         (unsigned long long)((long long)p.y * p.y) +
+                                         (unsigned long long)((long long)p.z * p.z);
+            if (g < R2) {
                 const int c = t * kMaxSpecies + p.w;
                 if constexpr (F32) {
                     float uh, ul, m;
@@ -583,10 +575,7 @@ __global__ void __launch_bounds__(kDirectWarps * 32) k_trial_direct(
                     ff_acc(eh, el, uh, ul);
                     mag += m;
                 } else {
-                    double u, m;
-                    lj_f64(s, fd.c4e[c], fd.sig2[c], u, m);
-                    de += u;
-                    da += m;
+                    lj_f64_add(g, fd.rep[c], fd.att[c], rep, att);
                 }
             }
         }
@@ -630,7 +619,7 @@ __global__ void __launch_bounds__(kDirectWarps * 32) k_trial_direct(
         const float a = warp_sum(mag);
         if (lane == 0) redf[w] = make_float4(s.hi, s.lo, a, 0.f);
     } else {
-        const double e = warp_sum(de), a = warp_sum(da);
+        const double e = warp_sum(rep - att), a = warp_sum(rep + att);
         if (lane == 0) red[w] = make_double2(e, a);
     }
     __syncthreads();
@@ -716,7 +705,7 @@ struct PairDrain {
     const uint4 *home;
     unsigned long long R2;
     float eh = 0.f, el = 0.f, wh = 0.f, wl = 0.f;
-    double de = 0.0, da = 0.0;
+    double rep = 0.0, att = 0.0;
     __device__ PairDrain(const SH &s, const uint4 *h, unsigned long long r) : sh(s), home(h), R2(r) {}
     __device__ __forceinline__ void operator()(int e)
     {
@@ -724,13 +713,10 @@ struct PairDrain {
         const uint4 r = sh.raw[e & 1023];
         const int k = (int)tag_species(P.w) * kMaxSpecies + (int)tag_species(r.w);
         const int ex = (int)(P.x - r.x), ey = (int)(P.y - r.y), ez = (int)(P.z - r.z);
-        GridSep s;
-        s.dx = ex;
-        s.dy = ey;
-        s.dz = ez;
-        s.g = (unsigned long long)((long long)ex * ex) + (unsigned long long)((long long)ey * ey) +
-              (unsigned long long)((long long)ez * ez);
-        if (s.g >= R2) return;
+        const unsigned long long g = (unsigned long long)((long long)ex * ex) +
+                                     (unsigned long long)((long long)ey * ey) +
+                                     (unsigned long long)((long long)ez * ez);
+        if (g >= R2) return;
         if constexpr (F32) {
             const float4 c = sh.field.f[k];
             float uh, ul, m;
@@ -739,10 +725,7 @@ struct PairDrain {
             ff_acc(wh, wl, -fmaf(3.f, m, 9.f * uh), 0.f);  // r U'(r) = -12 rep + 6 att
         } else {
             const double2 c = sh.field.d[k];
-            double u, m;
-            lj_f64(s, c.x, c.y, u, m);
-            de += u;
-            da += m;  // r U'(r) = -(3 m + 9 u)
+            lj_f64_add(g, c.x, c.y, rep, att);
         }
     }
 };
@@ -769,7 +752,7 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_cell_energy(const uint4 *__re
     __shared__ uint4 home[kPChunk];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (threadIdx.x == 0) mbar_init(&sh.bar, 1);
-    nb_field<F32>(sh, ff, fd);
+    nb_field<F32, false>(sh, ff, fd);
     __syncthreads();
     unsigned parity = 0;
     unsigned short *list = sh.list[w];
@@ -835,7 +818,7 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_cell_energy(const uint4 *__re
                 partial[2 * c + threadIdx.x] = (double)sum.hi + (double)sum.lo;
             }
         } else {
-            const double e = warp_sum(D.de), vw = warp_sum(-(3.0 * D.da + 9.0 * D.de));
+            const double e = warp_sum(D.rep - D.att), vw = warp_sum(6.0 * D.att - 12.0 * D.rep);  // r U'(r)
             if (lane == 0) {
                 red[w][0] = e;
                 red[w][1] = vw;
@@ -1029,7 +1012,7 @@ __global__ void __launch_bounds__(kNbWarps * 32, 5) k_cell_grad(const uint4 *__r
         }
         mbar_init(&sh.bar, 1);
     }
-    nb_field<F32>(sh, ff, fd);
+    nb_field<F32, true>(sh, ff, fd);
     __syncthreads();
     unsigned parity = 0;
     unsigned short *list = sh.list[w];

@@ -43,6 +43,8 @@ def test_few_and_many_points(precision, m, n, L, rc, S):
     ref, uabs = o.trial_energy(tp[pick], ts[pick], exclude=excl[pick].tolist(), with_abs=True)
     assert np.all(np.abs(got.cpu().numpy()[pick] - ref) <= TOL[precision] * uabs)
     assert np.allclose(gabs.cpu().numpy()[pick], uabs, rtol=1e-5, atol=0)
+    alone = b.trial_energy(tp, ts, exclude=torch.as_tensor(excl)).cpu().numpy()
+    assert np.all(np.abs(alone[pick] - ref) <= TOL[precision] * uabs)
 
 
 @pytest.mark.parametrize("m", [3, FEW + 1])
