@@ -37,6 +37,11 @@
 // 2,048 particles in FP64 23.0 -> 8.5 ms, 2*10^4 of 131,072 in FP32 29.9 ->
 // 15.9 ms, the 64-chain isotherm step 223 -> 130 ms.
 //
+// The microcell chain (Sec. 3.3.3) is the same kernel with the evaluation over
+// the cube of microcells and both lists kept: 4,000 moves of 87,296 particles in
+// FP32 19.1 -> 7.5 ms against a block of eight warps that evaluated and
+// committed one move after another.  Its counters stay in global memory.
+//
 // Movers hand the turn on through shared memory with block-scope fences;
 // every wait is bounded and sets a timeout status instead of hanging.  Cell
 // counters live in shared memory (uint16) for the whole launch; particle data
@@ -103,6 +108,12 @@ struct ChainArgs {
     uint4 *cell_pos;
     int32_t *cell_count;
     uint4 *pos_by_id;
+    // the microcell list (microcell launches): M per side, cubes of nax per
+    // side reaching D each way, mcap slots of ncm records
+    int M, nax, mD, mcap;
+    uint32_t ncm;
+    uint8_t *mc_count;
+    uint4 *mc_pos;
     int64_t *d_n;
     double *d_energy;
     gcmc_trace *trace;
@@ -114,12 +125,16 @@ constexpr int kMaxMovers = kChainWarps - 1;
 constexpr int kRS = 32;                      // log, book and outlook rings (at least 2 kMaxMovers)
 constexpr int kWords = 16;                   // moves a mover draws the words of at once
 constexpr int kQ = 128;                      // a mover's queue of pairs: at most 31 + 64 wait
-// a mover's dynamic shared memory: queue, work cells, words
-constexpr int kMoverBytes = kQ * 16 + 64 * 16 + kWords * 48;
+// a mover's dynamic shared memory: queue, words and the work cells, or -- in a
+// microcell launch -- the records of kMcGroup microcells
+constexpr int kMcGroup = 128;
+constexpr int kMoverBytes = kQ * 16 + kWords * 48 + 64 * 16;
+constexpr int kMicroMoverBytes = kQ * 16 + kWords * 48 + kMcGroup * kMicroMaxCap * 4;
 constexpr unsigned long long kWaitNs = 1000000000ull;  // a wait gives up after 1 s (default)
 static_assert(kRS >= 2 * kMaxMovers, "ring entries of moves that can still be read");
 
 constexpr uint32_t kOld = 1u, kNew = 2u;
+constexpr int kStatusMicroOverflow = 64;  // a move needs a full microcell
 
 // ---------------------------------------------------------------- trials
 struct Trial {
@@ -178,15 +193,15 @@ struct __align__(16) LogRec {
 struct __align__(16) BookRec {  // mover -> keeper
     double dU64, lnA;  // dU when decided in FP64 or evaluated in FP64 mode
     double dW;         // virial change of the trial (virial runs)
+    double uab;
     float hi, lo;      // dU = hi + lo otherwise
-    float uab;
     // bit 0 accepted, 1 possible, 2 dU64 holds dU, 3 near the threshold, 4
     // decided in FP64, 5 evaluated again; type << 8, species << 16
     int bits;
     int index;
     int n;             // N_s before the move
     int ready;         // move + 1
-    int pad[3];
+    int pad[2];
 };
 constexpr int kBkAcc = 1, kBkPossible = 2, kBkUse64 = 4, kBkNear = 8, kBkRefined = 16, kBkAgain = 32;
 
@@ -217,6 +232,27 @@ __device__ __forceinline__ int vload(const int &x) { return *(volatile const int
 __device__ __forceinline__ void vstore(int &x, int v) { *(volatile int *)&x = v; }
 __device__ __forceinline__ int cload(const uint16_t &x) { return *(volatile const uint16_t *)&x; }
 __device__ __forceinline__ void cstore(uint16_t &x, int v) { *(volatile uint16_t *)&x = (uint16_t)v; }
+// Counters in global memory, shared by the warps of one block.
+__device__ __forceinline__ int gload(const int32_t *p)
+{
+    int v;
+    asm volatile("ld.relaxed.cta.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void gstore(int32_t *p, int v)
+{
+    asm volatile("st.relaxed.cta.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ int gload(const uint8_t *p)
+{
+    uint32_t v;
+    asm volatile("ld.relaxed.cta.global.u8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return (int)v;
+}
+__device__ __forceinline__ void gstore(uint8_t *p, int v)
+{
+    asm volatile("st.relaxed.cta.global.u8 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 __device__ __forceinline__ void fence_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 
 __device__ __forceinline__ int4 turn_load(const Shared &sh)
@@ -308,17 +344,39 @@ struct Entry {
     uint4 Q;
     int cell, slot;
 };
+template <bool MICRO>
 __device__ __noinline__ Entry find_now(const ChainArgs &a, const uint16_t *cnt, int s, int i, int lane)
 {
     Entry r;
     r.Q = a.pos_by_id[(long long)s * a.maxN + i];
     r.cell = cell_of(r.Q.x, r.Q.y, r.Q.z, a.T);
-    const int n = cload(cnt[r.cell]);
+    const int n = MICRO ? gload(a.cell_count + r.cell) : cload(cnt[r.cell]);
     const uint4 *cell = a.cell_pos + (long long)r.cell * a.cap;
     uint4 v = make_uint4(0, 0, 0, 0);
     if (lane < n) v = cell[lane];
     r.slot = find_far(cell, r.Q.w, n, v, lane).at;
     return r;
+}
+
+// A microcell's entries as a warp sees them: its count, the lane's entry and
+// the slot of `tag` (-1: not there).
+struct MicroEntry {
+    int n, slot;
+    uint4 v;
+};
+__device__ __forceinline__ MicroEntry micro_find(const ChainArgs &a, uint32_t c, uint32_t tag, int lane)
+{
+    MicroEntry r;
+    r.n = __shfl_sync(0xffffffffu, gload(a.mc_count + c), 0);
+    fence_cta();
+    r.v = make_uint4(0, 0, 0, 0);
+    if (lane < r.n) r.v = a.mc_pos[(long long)lane * a.ncm + c];
+    r.slot = __ffs(__ballot_sync(0xffffffffu, lane < r.n && r.v.w == tag)) - 1;
+    return r;
+}
+__device__ __forceinline__ uint32_t micro_of(const uint4 &p, int M)
+{
+    return (uint32_t)((cell_coord(p.z, (uint32_t)M) * M + cell_coord(p.y, (uint32_t)M)) * M + cell_coord(p.x, (uint32_t)M));
 }
 
 // The decision in FP64: accepted, near the threshold, ln A.
@@ -376,13 +434,14 @@ __device__ __noinline__ bool wait_never(const ChainArgs &a, Shared &sh)
     }
 }
 
+template <bool MICRO>
 struct Mover {
     const ChainArgs &a;
     Shared &sh;
     uint16_t *cnt;
     int4 *q;         // kQ queued pairs: separation, pair index | 0x100 for a term that counts negatively
-    int4 *tab;       // 64 work cells: record offset (2 words), flags
     WordRec *words;  // kWords
+    int4 *tab;       // 64 work cells: record offset (2 words), flags; microcells: record offsets
     uint4 *cell_pos;
     unsigned long long R2;
     float r2hi;
@@ -412,6 +471,15 @@ struct Mover {
                 ++s;
             }
         }
+    }
+
+    // the counters: in shared memory, with microcells in global memory (the
+    // evaluation does not read them there)
+    __device__ __forceinline__ int count(int c) const { return MICRO ? gload(a.cell_count + c) : cload(cnt[c]); }
+    __device__ __forceinline__ void set_count(int c, int n) const
+    {
+        if (MICRO) gstore(a.cell_count + c, n);
+        else cstore(cnt[c], n);
     }
 
     __device__ __forceinline__ int cell_at(int x, int y, int z) const
@@ -468,6 +536,224 @@ struct Mover {
         o.e = o.el = o.ua = o.w = 0.f;
         o.de = o.da = o.dw = 0.0;
         if (!t.possible) return;
+        if constexpr (MICRO && P32) {
+            evaluate_micro32(t, o);
+            return;
+        }
+        if constexpr (MICRO) evaluate_micro<VIR>(t, o);
+        else evaluate_cells<P32, VIR>(t, o);
+        if constexpr (P32) {
+            const FF s = ff_warp_sum(FF{o.e, o.el});
+            o.e = s.hi;
+            o.el = s.lo;
+            o.ua = warp_sum(o.ua);
+            if (VIR) o.w = warp_sum(o.w);
+        } else {
+            o.de = warp_sum(o.de);
+            o.da = warp_sum(o.da);
+            if (VIR) o.dw = warp_sum(o.dw);
+        }
+    }
+
+    // Lowest cell of the cube around grid coordinate X (0 when the cube spans
+    // the axis).
+    __device__ __forceinline__ int cube_base(uint32_t X) const
+    {
+        return a.nax >= a.M ? 0 : cell_coord(X, (uint32_t)a.M) - a.mD;
+    }
+    // The change of a cube's base between two positions, as a wrapped difference.
+    __device__ __forceinline__ int cube_shift(int d) const { return 2 * d > a.M ? d - a.M : (2 * d < -a.M ? d + a.M : d); }
+
+    // The trial's energy change over the microcells (Sec. 3.3.3): the cube
+    // around its position; for a displacement that moves the cube by at most
+    // a cell per axis the union of both cubes, each record tested against
+    // both positions; for a longer one the old cube, then the new one.
+    // kMcGroup cells at a time: the lanes read their counts, number the
+    // records and list them, and the records are taken 32 at a time as in
+    // evaluate_cells.  FP64.
+    template <bool VIR>
+    __device__ __forceinline__ void evaluate_micro(const Trial &t, Sums &o) const
+    {
+        const unsigned lt = (1u << lane) - 1u;
+        uint32_t *list = (uint32_t *)tab;
+        const uint4 PA = t.type == 1 ? t.Pn : t.Po;
+        int bx = cube_base(PA.x), by = cube_base(PA.y), bz = cube_base(PA.z);
+        const int cx = cube_base(t.Pn.x), cy = cube_base(t.Pn.y), cz = cube_base(t.Pn.z);
+        int nx = a.nax, ny = a.nax, nz = a.nax, sets = 1;
+        if (t.type == 0) {
+            const int dx = cube_shift(cx - bx), dy = cube_shift(cy - by), dz = cube_shift(cz - bz);
+            if (max(max(abs(dx), abs(dy)), abs(dz)) > 1) {
+                sets = 2;
+            } else {
+                bx += min(dx, 0);
+                by += min(dy, 0);
+                bz += min(dz, 0);
+                nx += abs(dx);
+                ny += abs(dy);
+                nz += abs(dz);
+            }
+        }
+        const uint32_t self = t.Po.w;
+        const int wA = t.s * kMaxSpecies + (t.type == 1 ? 0 : 0x100), wB = t.s * kMaxSpecies;
+        const uint32_t ix = 0xFFFFFFFFu / (uint32_t)nx + 1u, iy = 0xFFFFFFFFu / (uint32_t)ny + 1u;  // i / nx = umulhi(i, ix)
+        const int n = nx * ny * nz;
+        int head = 0, nq = 0;
+        for (int set = 0; set < sets; ++set) {
+            const bool testA = set == 0, testB = t.type == 0 && (sets == 1 || set == 1);
+            if (set == 1) {
+                bx = cx;
+                by = cy;
+                bz = cz;
+            }
+#pragma unroll 1
+            for (int i0 = 0; i0 < n; i0 += kMcGroup) {
+                uint32_t c[kMcGroup / 32];
+                int k[kMcGroup / 32], mine = 0;
+#pragma unroll
+                for (int j = 0; j < kMcGroup / 32; ++j) {
+                    const int i = i0 + 32 * j + lane;
+                    c[j] = 0;
+                    k[j] = 0;
+                    if (i < n) {
+                        const int r = nx == 1 ? i : (int)__umulhi((uint32_t)i, ix), z = ny == 1 ? r : (int)__umulhi((uint32_t)r, iy);
+                        const int x = wrapc(bx + i - r * nx, a.M), y = wrapc(by + r - z * ny, a.M), w = wrapc(bz + z, a.M);
+                        c[j] = (uint32_t)((w * a.M + y) * a.M + x);
+                        k[j] = gload(a.mc_count + c[j]);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < kMcGroup / 32; ++j) mine += k[j];
+                fence_cta();  // the counts are read before the records they cover
+                const int inc = warp_inclusive_scan(mine), P = __shfl_sync(0xffffffffu, inc, 31);
+                int off = inc - mine;
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < kMcGroup / 32; ++j)
+#pragma unroll 1
+                    for (int q2 = 0; q2 < k[j]; ++q2) list[off++] = (uint32_t)q2 * a.ncm + c[j];
+                __syncwarp();
+                const bool final = set == sets - 1 && i0 + kMcGroup >= n;
+                uint4 r = make_uint4(0, 0, 0, 0);
+                bool have = lane < P;
+                if (have) r = a.mc_pos[list[lane]];
+#pragma unroll 1
+                for (int base = 0; base < P || (final && nq > 0); base += 32) {
+                    uint4 rn = r;
+                    const bool next = base + 32 + lane < P;
+                    if (next) rn = a.mc_pos[list[base + 32 + lane]];
+                    if (have && r.w == self) have = false;  // the particle itself (no tag for an insertion)
+                    if (testA) {
+                        const int ex = (int)(PA.x - r.x), ey = (int)(PA.y - r.y), ez = (int)(PA.z - r.z);
+                        const float gx = (float)ex, gy = (float)ey, gz = (float)ez;
+                        const bool in = have && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < r2hi;
+                        const unsigned b = __ballot_sync(0xffffffffu, in);
+                        if (in) q[(head + nq + __popc(b & lt)) & (kQ - 1)] = make_int4(ex, ey, ez, wA + (int)tag_species(r.w));
+                        nq += __popc(b);
+                    }
+                    if (testB) {
+                        const int ex = (int)(t.Pn.x - r.x), ey = (int)(t.Pn.y - r.y), ez = (int)(t.Pn.z - r.z);
+                        const float gx = (float)ex, gy = (float)ey, gz = (float)ez;
+                        const bool in = have && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < r2hi;
+                        const unsigned b = __ballot_sync(0xffffffffu, in);
+                        if (in) q[(head + nq + __popc(b & lt)) & (kQ - 1)] = make_int4(ex, ey, ez, wB + (int)tag_species(r.w));
+                        nq += __popc(b);
+                    }
+                    const bool last = final && base + 32 >= P;
+#pragma unroll 1
+                    while (nq >= 32 || (last && nq > 0)) {
+                        const int cq = min(nq, 32);
+                        __syncwarp();
+                        if (lane < cq) pair_term<false, VIR>(q[(head + lane) & (kQ - 1)], o);
+                        head += cq;
+                        nq -= cq;
+                        __syncwarp();
+                    }
+                    r = rn;
+                    have = next;
+                }
+            }
+        }
+    }
+
+    // The same in FP32: plain FP32 terms, whose order of addition is part of
+    // the result to its last digits -- eight groups of 32 lanes stride over the
+    // cells of the old cube and then the new one, four strides at a time, slot
+    // by slot; a group's sums cross its lanes and are added in group order.
+    // The warp takes the groups one after another; a step's counts are read
+    // while the records of the step before it are evaluated.
+    __device__ __forceinline__ void evaluate_micro32(const Trial &t, Sums &o) const
+    {
+        constexpr int kB = 4, kGroups = 8, kStride = 32 * kGroups;
+        const int nax = a.nax, n3 = nax * nax * nax, total = (t.type == 0 ? 2 : 1) * n3;
+        const uint4 P0 = t.type == 1 ? t.Pn : t.Po;
+        const int bx = cube_base(P0.x), by = cube_base(P0.y), bz = cube_base(P0.z);
+        const int cx = cube_base(t.Pn.x), cy = cube_base(t.Pn.y), cz = cube_base(t.Pn.z);
+        const uint32_t ix = 0xFFFFFFFFu / (uint32_t)nax + 1u;  // i / nax = umulhi(i, ix), nax > 1
+        uint32_t c[kB], cn[kB];
+        int k[kB], kn[kB];
+        auto counts = [&](int f0) {
+#pragma unroll
+            for (int j = 0; j < kB; ++j) {
+                const int f = f0 + j * kStride;
+                cn[j] = 0;
+                kn[j] = 0;
+                if (f < total) {
+                    const bool side = f >= n3;
+                    const int i = side ? f - n3 : f;
+                    const int r = nax == 1 ? i : (int)__umulhi((uint32_t)i, ix), z = nax == 1 ? r : (int)__umulhi((uint32_t)r, ix);
+                    const int x = wrapc((side ? cx : bx) + i - r * nax, a.M), y = wrapc((side ? cy : by) + r - z * nax, a.M),
+                              w = wrapc((side ? cz : bz) + z, a.M);
+                    cn[j] = (uint32_t)((w * a.M + y) * a.M + x);
+                    kn[j] = gload(a.mc_count + cn[j]);
+                }
+            }
+        };
+        counts(lane);
+#pragma unroll 1
+        for (int g = 0; g < kGroups; ++g) {
+            float e = 0.f, u = 0.f;
+#pragma unroll 1
+            for (int b0 = 0; b0 < total; b0 += kB * kStride) {
+                const int f0 = b0 + 32 * g + lane;
+                int kmax = 0;
+#pragma unroll
+                for (int j = 0; j < kB; ++j) {
+                    c[j] = cn[j];
+                    k[j] = kn[j];
+                    kmax = max(kmax, k[j]);
+                }
+                fence_cta();  // the counts are read before the records they cover
+                const bool more = b0 + kB * kStride < total;
+                if (more || g + 1 < kGroups) counts(more ? f0 + kB * kStride : 32 * (g + 1) + lane);
+#pragma unroll 1
+                for (int q2 = 0; q2 < kmax; ++q2) {
+                    uint4 r[kB];
+#pragma unroll
+                    for (int j = 0; j < kB; ++j)
+                        if (q2 < k[j]) r[j] = a.mc_pos[(long long)q2 * a.ncm + c[j]];
+#pragma unroll
+                    for (int j = 0; j < kB; ++j) {
+                        if (q2 >= k[j]) continue;
+                        if (t.type != 1 && r[j].w == t.Po.w) continue;
+                        const bool old_side = t.type == 2 || (t.type == 0 && f0 + j * kStride < n3);
+                        const GridSep sep = grid_sep(old_side ? t.Po : t.Pn, r[j]);
+                        if (sep.g >= R2) continue;
+                        const int kk = t.s * kMaxSpecies + (int)tag_species(r[j].w);
+                        float x, m;
+                        lj_f32(sep, a.ff.c4e[kk], a.ff.sig2[kk], x, m);
+                        e += old_side ? -x : x;
+                        u += m;
+                    }
+                }
+            }
+            o.e += warp_sum(e);
+            o.ua += warp_sum(u);
+        }
+    }
+
+    template <bool P32, bool VIR>
+    __device__ __forceinline__ void evaluate_cells(const Trial &t, Sums &o) const
+    {
         const unsigned lt = (1u << lane) - 1u;
         // lane l owns work cells l and l + 32.  The counts are read before the
         // records: a count covers records that are already in place.
@@ -574,17 +860,6 @@ struct Mover {
             if (last) break;
             r = rn;
             f = fn;
-        }
-        if constexpr (P32) {
-            const FF s = ff_warp_sum(FF{o.e, o.el});
-            o.e = s.hi;
-            o.el = s.lo;
-            o.ua = warp_sum(o.ua);
-            if (VIR) o.w = warp_sum(o.w);
-        } else {
-            o.de = warp_sum(o.de);
-            o.da = warp_sum(o.da);
-            if (VIR) o.dw = warp_sum(o.dw);
         }
     }
 
@@ -723,20 +998,20 @@ struct Mover {
 };
 
 // FP64 evaluation of a trial inside the FP32 error band.
-template <bool VIR>
-__device__ __noinline__ Sums evaluate64(Mover M, Trial t)
+template <bool VIR, bool MICRO>
+__device__ __noinline__ Sums evaluate64(Mover<MICRO> M, Trial t)
 {
     Sums d;
     M.template evaluate<false, VIR>(t, d);
     return d;
 }
 
-template <bool F32, bool VIR, bool PROF>
+template <bool F32, bool VIR, bool PROF, bool MICRO>
 __device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint16_t *cnt, unsigned char *mine, int warp)
 {
     const int lane = threadIdx.x & 31, n = a.n_moves, W = a.movers;
-    Mover M{a, sh, cnt, (int4 *)mine, (int4 *)(mine + kQ * 16), (WordRec *)(mine + kQ * 16 + 64 * 16), a.cell_pos, a.R2,
-            a.r2hi, lane, a.T, a.S, a.cap, lane % 3 | (lane / 3 % 3) << 8 | (lane / 9) << 16};
+    Mover<MICRO> M{a, sh, cnt, (int4 *)mine, (WordRec *)(mine + kQ * 16), (int4 *)(mine + kQ * 16 + kWords * 48),
+                   a.cell_pos, a.R2, a.r2hi, lane, a.T, a.S, a.cap, lane % 3 | (lane / 3 % 3) << 8 | (lane / 9) << 16};
     const int S = M.S;
     unsigned long long c_eval = 0, c_room = 0, c_wait = 0, c_logs = 0, c_pick = 0, c_dec = 0, c_app = 0, c_book = 0,
                        c_all = 0;
@@ -809,8 +1084,8 @@ __device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint1
                     t.py = cell_coord(t.Po.y, (uint32_t)M.T);
                     t.pz = cell_coord(t.Po.z, (uint32_t)M.T);
                     t.co = (t.pz * M.T + t.py) * M.T + t.px;
-                    nco = __shfl_sync(0xffffffffu, cload(cnt[t.co]), 0);
-                    if (qcell >= 0) qn = __shfl_sync(0xffffffffu, cload(cnt[qcell]), 0);
+                    nco = __shfl_sync(0xffffffffu, M.count(t.co), 0);
+                    if (qcell >= 0) qn = __shfl_sync(0xffffffffu, M.count(qcell), 0);
                     fence_cta();
                     if (lane < nco) lastv = M.cell_pos[(long long)t.co * M.cap + lane];
                     if (lane < qn) qtag = M.cell_pos[(long long)qcell * M.cap + lane].w;
@@ -835,6 +1110,19 @@ __device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint1
                         t.cross = t.co != t.cn;
                         t.far = t.cross && !(near1(t.px - t.qx, M.T) && near1(t.py - t.qy, M.T) && near1(t.pz - t.qz, M.T));
                     }
+                }
+            }
+            // the microcells, and the entry that a removal moves (for the log)
+            uint32_t mo = 0, mn = 0;
+            uint4 mlast = make_uint4(0, 0, 0, 0);
+            int m_last = -1;  // its slot (-1: none)
+            if constexpr (MICRO) {
+                mn = micro_of(t.Pn, a.M);
+                mo = type == 1 ? mn : micro_of(t.Po, a.M);
+                if (t.possible && type != 1 && (type == 2 || mo != mn)) {
+                    const MicroEntry x = micro_find(a, mo, t.Po.w, lane);
+                    if (x.slot != x.n - 1) m_last = x.n - 1;
+                    mlast = x.v;
                 }
             }
             Sums E;
@@ -876,7 +1164,7 @@ __device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint1
             bool have64 = !F32;
             if constexpr (F32) {
                 if (need64 || ((band_mask >> 16) & 1u)) {
-                    const Sums d = evaluate64<VIR>(M, t);
+                    const Sums d = evaluate64<VIR, MICRO>(M, t);
                     E.de = d.de;
                     E.da = d.da;
                     E.dw = d.dw;
@@ -891,13 +1179,13 @@ __device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint1
                     fence_cta();
                     __syncwarp();
                 }
-                if (last_mine) L.moved = lastv;
+                if (MICRO ? lane == m_last : last_mine) L.moved = MICRO ? mlast : lastv;
                 if (lane == 0) {
                     L.ids = make_int4(type == 1 ? t.cn : t.co, t.cross ? t.cn : qcell, type == 1 ? -1 : (s << 24) | idx,
                                       last_id);
                     const uint4 p = type == 1 ? t.Pn : t.Po;
                     L.pos0 = make_uint4(p.x, p.y, p.z,
-                                        (type == 0 ? 1u : 0u) | (has_last ? 2u : 0u) | (type == 1 ? 4u : 0u) | ((uint32_t)s << 8));
+                                        (type == 0 ? 1u : 0u) | ((MICRO ? m_last >= 0 : has_last) ? 2u : 0u) | (type == 1 ? 4u : 0u) | ((uint32_t)s << 8));
                     L.pos1 = t.Pn;
                     if (type) vstore(sh.outlook[slot], mtag | (((acc_mask >> 16) & 1u) ? (s << 2) | type : 0));
                 }
@@ -964,7 +1252,7 @@ __device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint1
             const unsigned long long t3 = prof_clock<PROF>();
             c_wait += t3 - t2;
             const int ns = vload(sh.n[s]);
-            const int c_n = t.cn >= 0 ? cload(cnt[t.cn]) : 0;
+            const int c_n = t.cn >= 0 ? M.count(t.cn) : 0;
             const uint32_t hist = (uint32_t)v.y & ((1u << (m - c0)) - 1u);  // m - c0 < kRS
             if (t.possible) {
                 const uint32_t fresh = __ballot_sync(0xffffffffu, lane < m - c0 && vload(sh.ver[(m - 1 - lane) & (kRS - 1)]) != ver);
@@ -1002,14 +1290,47 @@ __device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint1
             if (in_band) {
                 const Decision d = decide_f64(a, w[6], w[7], type, s, ns, E.de, E.da);
                 lnA = d.lnA;
-                bits = (bits & ~kBkAcc) | kBkUse64 | kBkRefined | d.bits;
+                bits = (bits & ~kBkAcc) | kBkUse64 | (MICRO && !F32 ? 0 : kBkRefined) | d.bits;
             }
             const bool fin = bits & kBkAcc;
+            MicroEntry mx = {0, -1, make_uint4(0, 0, 0, 0)};
+            int n_mn = 0;
             if (fin) {
                 int stop_bits = 0;
                 if (type != 2 && (type == 1 || t.cross) && c_n >= M.cap) stop_bits = kStatusCellOverflow;
                 if (type == 1 && ns >= a.maxN) stop_bits = kStatusCapacity;
                 if (type != 1 && self_slot < 0) stop_bits = kStatusBadInput;  // a record missing from its cell
+                if constexpr (MICRO) {
+                    // the microcells as they are now
+                    if (type == 1 || (type == 0 && mn != mo)) {
+                        n_mn = __shfl_sync(0xffffffffu, gload(a.mc_count + mn), 0);
+                        if (!stop_bits && n_mn >= a.mcap) stop_bits = kStatusMicroOverflow;
+                    }
+                    if (type != 1) {
+                        mx = micro_find(a, mo, t.Po.w, lane);
+                        if (mx.slot < 0) stop_bits = kStatusBadInput;
+                        // a removal moves another entry than the log says: later moves test it again
+                        const int moves = (type == 2 || mn != mo) && mx.slot != mx.n - 1 ? mx.n - 1 : -1;
+                        const bool same = moves == m_last &&
+                                          (lane != moves || (mx.v.x == mlast.x && mx.v.y == mlast.y && mx.v.z == mlast.z));
+                        if (!stop_bits && !__all_sync(0xffffffffu, same)) {
+                            LogRec &L = sh.logs[slot];
+                            if (lane == 0) {
+                                vstore(sh.ver[slot], 0);
+                                fence_cta();
+                                L.pos0.w = (L.pos0.w & ~2u) | (moves >= 0 ? 2u : 0u);
+                            }
+                            __syncwarp();
+                            if (lane == moves) L.moved = mx.v;
+                            __syncwarp();
+                            if (lane == 0) {
+                                fence_cta();
+                                vstore(sh.ver[slot], mtag | 0x7E);
+                            }
+                            __syncwarp();
+                        }
+                    }
+                }
                 if (stop_bits) {
                     if (lane == 0) chain_stop(sh, stop_bits, 16);
                     goto done;
@@ -1031,7 +1352,7 @@ __device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint1
                     if (idx != last) {
                         // known from the evaluation unless a later move touched it
                         if (last_id != ((s << 24) | last) || (stale & hist) || qslot < 0) {
-                            const Entry x = find_now(a, cnt, s, last, lane);
+                            const Entry x = find_now<MICRO>(a, cnt, s, last, lane);
                             Q = x.Q;
                             qcell = x.cell;
                             qslot = x.slot;
@@ -1048,6 +1369,20 @@ __device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint1
                         }
                         // the last particle may be the entry that moves into the freed slot
                         both = qcell == t.co && qslot == nco - 1;
+                        if constexpr (MICRO) {
+                            // the same in the microcells
+                            const uint32_t mq = micro_of(Q, a.M);
+                            const MicroEntry x = micro_find(a, mq, Q.w, lane);
+                            if (x.slot < 0) {
+                                if (lane == 0) chain_stop(sh, kStatusBadInput, 32);
+                                goto done;
+                            }
+                            if (mq == mo && x.slot == mx.n - 1) {
+                                if (lane == mx.n - 1) mx.v.w = ntag;
+                            } else if (lane == 0) {
+                                a.mc_pos[(long long)x.slot * a.ncm + mq].w = ntag;
+                            }
+                        }
                         if (lane == 0) {
                             if (!both) M.cell_pos[(long long)qcell * M.cap + qslot].w = ntag;
                             by_id[idx] = make_uint4(Q.x, Q.y, Q.z, ntag);
@@ -1064,11 +1399,24 @@ __device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint1
                     if (both) lastv.w = ntag;
                     old_cell[self_slot] = lastv;
                 }
+                if constexpr (MICRO) {
+                    const bool leaves = type == 2 || (type == 0 && mn != mo);
+                    if (leaves && lane == mx.n - 1 && mx.slot != mx.n - 1) a.mc_pos[(long long)mx.slot * a.ncm + mo] = mx.v;
+                    if (type != 2 && lane == 0)
+                        a.mc_pos[(long long)(type == 0 && !leaves ? mx.slot : n_mn) * a.ncm + mn] =
+                            make_uint4(t.Pn.x, t.Pn.y, t.Pn.z, ntag);
+                    __syncwarp();
+                    if (lane == 0 && (leaves || type == 1)) {
+                        fence_cta();
+                        if (leaves) gstore(a.mc_count + mo, mx.n - 1);
+                        if (type != 2) gstore(a.mc_count + mn, n_mn + 1);
+                    }
+                }
                 __syncwarp();
                 if (lane == 0 && (type != 0 || t.cross)) {
                     fence_cta();  // the records before the counts that cover them
-                    if (type != 1) cstore(cnt[t.co], nco - 1);
-                    if (type != 2) cstore(cnt[t.cn], c_n + 1);
+                    if (type != 1) M.set_count(t.co, nco - 1);
+                    if (type != 2) M.set_count(t.cn, c_n + 1);
                     if (type != 0) vstore(sh.n[s], type == 1 ? ns + 1 : ns - 1);
                 }
             }
@@ -1084,7 +1432,7 @@ __device__ __forceinline__ void mover_loop(const ChainArgs &a, Shared &sh, uint1
                 B.dW = VIR ? (F32 && !in_band ? (double)E.w : E.dw) : 0.0;
                 B.hi = E.e;
                 B.lo = E.el;
-                B.uab = F32 && !in_band ? E.ua : (float)E.da;
+                B.uab = F32 && !in_band ? (double)E.ua : E.da;
                 B.bits = bits | (t.possible ? kBkPossible : 0) | (type << 8) | (s << 16);
                 B.index = type == 1 ? ns : idx;
                 B.n = ns;
@@ -1170,7 +1518,7 @@ __device__ void keeper_loop(const ChainArgs &a, Shared &sh)
                     }
                     tr.dU = possible ? dU : 0.0;
                     tr.lnA = lnA;
-                    tr.uabs = possible ? (double)B.uab : 0.0;
+                    tr.uabs = possible ? B.uab : 0.0;
                     tr.index = B.index;
                     tr.type = (uint8_t)type;
                     tr.species = (uint8_t)sp;
@@ -1223,7 +1571,7 @@ __device__ void keeper_loop(const ChainArgs &a, Shared &sh)
     }
 }
 
-template <bool F32, bool VIR, bool PROF>
+template <bool F32, bool VIR, bool PROF, bool MICRO>
 __global__ void __launch_bounds__(kChainWarps * 32, 1) k_chain(const ChainArgs *__restrict__ args)
 {
     constexpr int NTH = kChainWarps * 32;
@@ -1251,8 +1599,10 @@ __global__ void __launch_bounds__(kChainWarps * 32, 1) k_chain(const ChainArgs *
         }
         return;
     }
-    uint16_t *cnt = (uint16_t *)(dyn + (size_t)a.movers * kMoverBytes);
-    for (int c = tid; c < a.ncell; c += NTH) cnt[c] = (uint16_t)a.cell_count[c];
+    constexpr int kBytes = MICRO ? kMicroMoverBytes : kMoverBytes;
+    uint16_t *cnt = (uint16_t *)(dyn + (size_t)a.movers * kBytes);
+    if constexpr (!MICRO)
+        for (int c = tid; c < a.ncell; c += NTH) cnt[c] = (uint16_t)a.cell_count[c];
     if (tid < kMaxSpecies) sh.n[tid] = tid < a.S ? (int)a.d_n[tid] : 0;
     if (tid < kRS) {
         sh.book[tid].ready = 0;
@@ -1271,10 +1621,11 @@ __global__ void __launch_bounds__(kChainWarps * 32, 1) k_chain(const ChainArgs *
         sh.evaluations = 0;
     }
     __syncthreads();
-    if (warp < a.movers) mover_loop<F32, VIR, PROF>(a, sh, cnt, dyn + (size_t)warp * kMoverBytes, warp);
+    if (warp < a.movers) mover_loop<F32, VIR, PROF, MICRO>(a, sh, cnt, dyn + (size_t)warp * kBytes, warp);
     else if (warp == kChainWarps - 1) keeper_loop<VIR>(a, sh);
     __syncthreads();
-    for (int c = tid; c < a.ncell; c += NTH) a.cell_count[c] = cnt[c];
+    if constexpr (!MICRO)
+        for (int c = tid; c < a.ncell; c += NTH) a.cell_count[c] = cnt[c];
     if (tid < a.S) a.d_n[tid] = sh.n[tid];
     if (tid == 0) {
         ChainOut &o = *a.out;
@@ -1301,8 +1652,11 @@ constexpr int kMoverChoices[kChainConfigs] = {8, 5, 11, 15};
 template <bool F32, bool VIR>
 static void *chain_kernel(bool prof)
 {
-    return prof ? (void *)k_chain<F32, VIR, true> : (void *)k_chain<F32, VIR, false>;
+    return prof ? (void *)k_chain<F32, VIR, true, false> : (void *)k_chain<F32, VIR, false, false>;
 }
+// Moves in flight of a microcell launch: all there is room for (eleven: 8.4
+// instead of 7.5 ms for the 4,000 moves named at the top).
+constexpr int kMicroMovers = kMaxMovers;
 
 int chain_threads(int) { return kChainWarps * 32; }
 
@@ -1360,6 +1714,13 @@ static void fill_args(ChainArgs &a, const ChainJob &j, int movers, ChainOut *out
     a.cell_pos = ctx->cell_pos;
     a.cell_count = ctx->cell_count;
     a.pos_by_id = ctx->pos_by_id;
+    a.M = ctx->mc_M;
+    a.mD = ctx->mc_D;
+    a.nax = std::min(2 * ctx->mc_D + 1, ctx->mc_M);
+    a.mcap = ctx->mc_cap;
+    a.ncm = (uint32_t)ctx->mc_ncell;
+    a.mc_count = ctx->mc_count;
+    a.mc_pos = ctx->mc_pos;
     a.d_n = ctx->d_n;
     a.d_energy = ctx->d_energy;
     a.trace = j.trace ? j.trace + j.done : nullptr;
@@ -1426,7 +1787,8 @@ struct LaunchBufs {
 // with CUDA events on st around each launch (argument upload and result
 // download of a few hundred bytes included).
 static gcmc_status run_jobs(std::vector<ChainJob> &jobs, cudaStream_t st, bool f32, int config, LaunchBufs &B,
-                            int64_t *launches, std::string *err, bool use_graph = false, double *dev_ms = nullptr)
+                            int64_t *launches, std::string *err, bool use_graph = false, double *dev_ms = nullptr,
+                            bool micro = false)
 {
     const int K = (int)jobs.size();
     if (K == 0) return GCMC_OK;
@@ -1444,8 +1806,8 @@ static gcmc_status run_jobs(std::vector<ChainJob> &jobs, cudaStream_t st, bool f
     // a box of very many cells leaves room for fewer movers
     const size_t state = sizeof(Shared) + sizeof(ChainArgs) + 1024;
     const size_t room = (jobs[0].ctx->smem_optin - state - counters) / kMoverBytes;
-    const int movers = (int)std::min<size_t>(kMoverChoices[config], room);
-    const size_t smem = (size_t)movers * kMoverBytes + counters;
+    const int movers = micro ? kMicroMovers : (int)std::min<size_t>(kMoverChoices[config], room);
+    const size_t smem = micro ? (size_t)movers * kMicroMoverBytes : (size_t)movers * kMoverBytes + counters;
     // the virial sums are compiled in only when a chain of the launch keeps
     // it, the cycle counters only when a chain's context asked for them
     bool vir = false, prof = false;
@@ -1455,6 +1817,7 @@ static gcmc_status run_jobs(std::vector<ChainJob> &jobs, cudaStream_t st, bool f
     }
     void *kern = f32 ? (vir ? chain_kernel<true, true>(prof) : chain_kernel<true, false>(prof))
                      : (vir ? chain_kernel<false, true>(prof) : chain_kernel<false, false>(prof));
+    if (micro) kern = f32 ? (void *)k_chain<true, false, false, true> : (void *)k_chain<false, false, false, true>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) {
         if (err) *err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e);
@@ -1464,6 +1827,10 @@ static gcmc_status run_jobs(std::vector<ChainJob> &jobs, cudaStream_t st, bool f
         bool any = false;
         for (int k = 0; k < K; ++k) {
             fill_args(B.h_args[k], jobs[k], movers, B.d_out + k);
+            if (micro) {  // no diagnostic stall, the default limit of the waits
+                B.h_args[k].stall_at = -1;
+                B.h_args[k].wait_ns = kWaitNs;
+            }
             any = any || B.h_args[k].n_moves > 0;
         }
         if (!any) break;
@@ -1555,6 +1922,15 @@ static gcmc_status run_jobs(std::vector<ChainJob> &jobs, cudaStream_t st, bool f
                 j.result = fail(ctx, GCMC_ERR_TIMEOUT,
                                 "gcmc_run_moves: a bounded wait inside the chain kernel gave up (sites " +
                                     std::to_string(o.pad) + ")");
+                continue;
+            }
+            if (o.status & kStatusMicroOverflow) {
+                if (ctx->mc_cap_req != 0 || ctx->mc_cap >= kMicroMaxCap) {
+                    j.result = fail(ctx, GCMC_ERR_CELL_OVERFLOW, "gcmc_run_moves_micro: a microcell is full");
+                } else {
+                    const gcmc_status rs = micro_grow(ctx, std::min(kMicroMaxCap, ctx->mc_cap + 2));
+                    if (rs != GCMC_OK) j.result = rs;
+                }
                 continue;
             }
             if (o.status & (kStatusCellOverflow | kStatusCapacity)) {
@@ -1697,6 +2073,44 @@ gcmc_status run_moves(gcmc_ctx *ctx, uint64_t seed, uint64_t first, int64_t n_mo
     st = run_jobs_tuned(jobs, ctx->stream, ctx->precision == GCMC_FP32, ctx->chain_config, bufs, &ctx->launches,
                         &err, false, nullptr);
     if (st != GCMC_OK) return fail(ctx, st, err);
+    if (stats) *stats = j.agg;
+    return j.result;
+}
+
+gcmc_status run_moves_micro(gcmc_ctx *ctx, uint64_t seed, uint64_t first, int64_t n_moves, const gcmc_move_mix *mix,
+                            gcmc_move_stats *stats, gcmc_trace *trace)
+{
+    gcmc_status st;
+    if (!ctx->mc_valid) {
+        st = micro_build(ctx, ctx->mc_edge, ctx->mc_cap_req);
+        if (st != GCMC_OK) return st;
+    }
+    if (!ctx->energy_valid) {
+        st = total_energy(ctx, nullptr);
+        if (st != GCMC_OK) return st;
+    }
+    static thread_local LaunchBufs bufs;
+    std::vector<ChainJob> jobs(1);
+    ChainJob &j = jobs[0];
+    memset(&j, 0, sizeof(j));
+    j.ctx = ctx;
+    j.seed = seed;
+    j.first = first;
+    j.n_moves = n_moves;
+    j.mix = *mix;
+    j.trace = trace;
+    j.result = GCMC_OK;
+    j.agg.energy = ctx->energy;
+    for (int q = 0; q < kMaxSpecies; ++q) j.agg.n[q] = ctx->n_host[q];
+    j.agg.virial = j.agg.sum_virial = NAN;
+    ctx->last_refetch = 0;
+    ctx->last_refines = 0;
+    std::string err;
+    st = run_jobs(jobs, ctx->stream, ctx->precision == GCMC_FP32, 0, bufs, &ctx->launches, &err, false, nullptr, true);
+    if (st != GCMC_OK) return fail(ctx, st, err);
+    if (j.result == GCMC_ERR_NONFINITE) fail(ctx, j.result, "gcmc_run_moves_micro: the running energy is not finite");
+    j.agg.chain_ms = 0.0;
+    for (double &v : ctx->last_prof) v = 0.0;
     if (stats) *stats = j.agg;
     return j.result;
 }

@@ -146,7 +146,9 @@ gcmc_status export_positions(gcmc_ctx *ctx, double *pos, int32_t *species);
 gcmc_status run_moves(gcmc_ctx *ctx, uint64_t seed, uint64_t first, int64_t n_moves,
                       const gcmc_move_mix *mix, gcmc_move_stats *stats, gcmc_trace *trace);
 // micro.cu
+constexpr int kMicroMaxCap = 15;  // slots per microcell, at most
 gcmc_status micro_build(gcmc_ctx *ctx, double edge, int cap_req);
+gcmc_status micro_grow(gcmc_ctx *ctx, int ncap);
 gcmc_status run_moves_micro(gcmc_ctx *ctx, uint64_t seed, uint64_t first, int64_t n_moves,
                             const gcmc_move_mix *mix, gcmc_move_stats *stats, gcmc_trace *trace);
 void micro_free(gcmc_ctx *ctx);
