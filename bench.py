@@ -71,7 +71,7 @@ CHAIN_TRAFFIC = {"sha256_prefix": "fb1ab48a525325ae", "bytes": 19.05e6, "moves":
 # valid for the sources whose joint sha256 has this prefix (the kernels of
 # these calls are those of the captured revision)
 KERNEL_TRAFFIC = {
-    "cells": {"sources": ("gcmc_cells.cu", "gcmc_device.cuh"), "sha256_prefix": "f1eee5859ed09753",
+    "cells": {"sources": ("gcmc_cells.cu", "gcmc_device.cuh"), "sha256_prefix": "0943f0587b70112e",
               "bytes": {"cell_build_mixture_1m": 115.4e6}},
     "energy": {"sources": ("gcmc_energy.cu", "gcmc_stage.cuh", "gcmc_device.cuh"),
                "sha256_prefix": "477fe33da7cfd2a6",
