@@ -512,12 +512,14 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
 // is one launch and one wait: binning the points takes two fills, five
 // launches and a copy before and after the energies, and a pass over every
 // cell, which is what bounds small calls: 64 points against 2,048 particles
-// take 16 us instead of 52 (FP64), against 2^20 particles 18 instead of 78.
+// take 16 us instead of 52 (FP64), against 2^20 particles 16 instead of 78.
 // Many points share their cell's staged records, so the binned path wins where
-// the points are many: at 4,096 points 55 against 67 us (FP64) and 25 against
-// 54 (FP32) for 2,048 particles, at 8,192 94 against 89 and 34 against 64.
+// the points are many, the later the more cells it has to pass over.  Direct
+// and binned, against 2,048 / 20,000 / 2^20 particles: FP64 at 4,096 points
+// 44 / 44 / 45 us and (8,192 points) 61 / 62 / 126, where direct takes twice
+// the 44; FP32 at 16,384 points 53 / 54 / 62 and 71 / 61 / 153.
 constexpr int kDirectWarps = 4;
-constexpr int64_t kDirectPoints = 4096;
+constexpr int64_t kDirectPoints64 = 4096, kDirectPoints32 = 16384;
 
 template <bool F32>
 __global__ void __launch_bounds__(kDirectWarps * 32) k_trial_direct(
@@ -1187,7 +1189,8 @@ gcmc_status trial_energy(gcmc_ctx *ctx, const double *pos, const int32_t *specie
     float r2hi;
     bool wrap;
     screen_bound(ctx, r2hi, wrap);
-    if (m <= kDirectPoints && !(out_abs && ctx->precision == GCMC_FP32)) {
+    // FP32 sums of magnitudes keep the order of the binned path
+    if (m <= (ctx->precision == GCMC_FP64 ? kDirectPoints64 : out_abs ? 0 : kDirectPoints32)) {
         st = ensure_pinned(ctx, kPinnedBytes);
         if (st != GCMC_OK) return st;
         // the status word lies in pinned host memory, written by the kernel

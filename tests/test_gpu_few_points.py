@@ -24,7 +24,7 @@ FEW = 4096
 
 
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
-@pytest.mark.parametrize("m", [1, 2, FEW, FEW + 1])
+@pytest.mark.parametrize("m", [1, 2, FEW, FEW + 1, 4 * FEW, 4 * FEW + 1])
 @pytest.mark.parametrize("n,L,rc,S", [(0, 8.0, 2.5, 1), (90, 5.6, 2.5, 2), (1500, 7.6, 2.5, 3), (1000, 13.0, 2.5, 2)])
 def test_few_and_many_points(precision, m, n, L, rc, S):
     pos, types, eps, sigma = W.tiny_system(n=max(n, 1), L=L, rc=rc, n_species=S, seed=n + 3)
