@@ -74,9 +74,9 @@ KERNEL_TRAFFIC = {
     "cells": {"sources": ("gcmc_cells.cu", "gcmc_device.cuh"), "sha256_prefix": "0943f0587b70112e",
               "bytes": {"cell_build_mixture_1m": 115.4e6}},
     "energy": {"sources": ("gcmc_energy.cu", "gcmc_stage.cuh", "gcmc_device.cuh"),
-               "sha256_prefix": "0df15e1747f6541b",
-               "bytes": {"trial_energy_mixture_1m": 151.6e6, "total_energy_mixture_1m": 17.97e6,
-                         "energy_grad_262k": 6.39e6}},
+               "sha256_prefix": "0ea83cb5757db123",
+               "bytes": {"trial_energy_mixture_1m": 152.1e6, "total_energy_mixture_1m": 17.93e6,
+                         "energy_grad_262k": 5.47e6}},
 }
 DEFAULT_MOVES = {"isotherm": 100_000, "c2": 1_000_000, "c1": 10_000}
 DEFAULT_CPU_MOVES = {"isotherm": 20_000, "c2": 1_000_000, "c1": 10_000}
