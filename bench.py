@@ -74,7 +74,7 @@ KERNEL_TRAFFIC = {
     "cells": {"sources": ("gcmc_cells.cu", "gcmc_device.cuh"), "sha256_prefix": "0943f0587b70112e",
               "bytes": {"cell_build_mixture_1m": 115.4e6}},
     "energy": {"sources": ("gcmc_energy.cu", "gcmc_stage.cuh", "gcmc_device.cuh"),
-               "sha256_prefix": "0ea83cb5757db123",
+               "sha256_prefix": "770bd8275192054c",
                "bytes": {"trial_energy_mixture_1m": 152.1e6, "total_energy_mixture_1m": 17.93e6,
                          "energy_grad_262k": 5.47e6}},
 }

@@ -107,12 +107,13 @@ __device__ __forceinline__ void pair_acc(const uint4 &p, const uint4 &q, uint32_
 // holds many CTAs (nine of four warps).  With 768 for both (six CTAs) the
 // trial energies took 1.09 ms and the total energy 0.95 ms.
 constexpr int kBufFull = 544, kBufHalf = 384;
-// ... and where plain FP32 sums of a point's terms are results: their order,
-// the pairs of a pass by staged index, is part of the result to its last digits
+// ... and where plain FP32 sums of a point's terms are results (forces, table
+// gradients, magnitudes): their order, the pairs of a pass by staged index, is
+// part of the result to its last digits
 constexpr int kBufOrdered = 896;
 constexpr int kPChunk = 64;   // points per chunk (per-point sums in shared memory)
 constexpr int kNbWarps = 4;   // warps of a neighbourhood CTA (two: trial energies 14 % slower; eight: total energy 18 %)
-constexpr int kNbQ = 128;     // queue entries per warp of k_trial_direct (a ring: up to 31 + 2 x 32 pending)
+constexpr int kNbQ = 128;     // queue entries per warp of the other trial kernels (a ring: up to 31 + 2 x 32 pending)
 static_assert(kBufFull % 32 == 0 && kBufHalf % 32 == 0 && kBufOrdered % 32 == 0 && kBufFull <= 1024 &&
                   kBufHalf <= 1024 && kBufOrdered <= 1024 && kPChunk <= 64,
               "list entries and masks");
@@ -130,7 +131,7 @@ template <int KB>
 struct __align__(16) NbShared {
     static constexpr int kBuf = KB;
     uint4 raw[KB];       // staged records (X, Y, Z, tag)
-    float4 fl[KB];       // the same relative to the home cell centre
+    float4 fl[KB];       // the same relative to the home cell centre, tag bits in .w
     // pairs inside the cutoff: staged index | point << 10; up to 31 left over
     // and a point's pairs
     unsigned short list[kNbWarps][KB + 32];
@@ -145,8 +146,8 @@ struct __align__(16) NbShared {
     } field;
 };
 
-template <bool F32, bool GRAD, int KB>
-__device__ __forceinline__ void nb_field(NbShared<KB> &sh, const FieldF &ff, const FieldD &fd)
+template <bool F32, bool GRAD, class SH>
+__device__ __forceinline__ void nb_field(SH &sh, const FieldF &ff, const FieldD &fd)
 {
     for (int k = threadIdx.x; k < kMaxSpecies * kMaxSpecies; k += blockDim.x) {
         if constexpr (F32) sh.field.f[k] = make_float4(ff.c4e[k], ff.c4e_lo[k], ff.sig2[k], ff.sig2_lo[k]);
@@ -228,18 +229,16 @@ __device__ __forceinline__ void nb_screen_exact(const float4 *fl, const uint4 *r
     }
 }
 
-// Writes the records of a mask to the list by ascending index, without that of
-// tag `excl` (~0: none); returns their number.
-__device__ __forceinline__ int nb_list_ordered(unsigned short *list, uint32_t mask, int rows, const uint4 *raw,
-                                               uint32_t excl)
+// Writes the records of a mask to the list by ascending index; returns their
+// number.
+__device__ __forceinline__ int nb_list_ordered(unsigned short *list, uint32_t mask, int rows)
 {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     int n = 0;
 #pragma unroll 2
     for (int r = 0; r < rows; ++r) {
-        bool in = (mask >> (rows - 1 - r)) & 1u;
-        if (excl != 0xFFFFFFFFu && in) in = raw[32 * r + lane].w != excl;
+        const bool in = (mask >> (rows - 1 - r)) & 1u;
         const unsigned b = __ballot_sync(0xffffffffu, in);
         if (in) list[n + __popc(b & lt)] = (unsigned short)(32 * r + lane);
         n += __popc(b);
@@ -325,8 +324,8 @@ __device__ __forceinline__ T warp_sum_many(T *v)
 // (bulk copies, then the float conversion).  Returns false -- in every
 // thread -- when the copy did not land within the wait limit; the timeout
 // bit is then set and the block must return.
-template <int KB>
-__device__ __forceinline__ bool nb_stage(NbShared<KB> &sh, const uint4 *__restrict__ cpos, int w0, int w1,
+template <class SH>
+__device__ __forceinline__ bool nb_stage(SH &sh, const uint4 *__restrict__ cpos, int w0, int w1,
                                          uint32_t cx0, uint32_t cy0, uint32_t cz0, unsigned &parity,
                                          int *__restrict__ status)
 {
@@ -345,7 +344,7 @@ __device__ __forceinline__ bool nb_stage(NbShared<KB> &sh, const uint4 *__restri
     parity ^= 1u;
     for (int f = threadIdx.x; f < w1 - w0; f += blockDim.x) {
         const uint4 r = sh.raw[f];
-        sh.fl[f] = make_float4(rel_f(r.x, cx0), rel_f(r.y, cy0), rel_f(r.z, cz0), 0.f);
+        sh.fl[f] = make_float4(rel_f(r.x, cx0), rel_f(r.y, cy0), rel_f(r.z, cz0), __uint_as_float(r.w));
     }
     __syncthreads();
     return true;
@@ -395,8 +394,7 @@ struct TrialDrain {
 // Trial points binned by cell: cell c holds the points pts[ps[c] .. ps[c+1]).
 // Each warp screens two points together (they share the loads of the staged
 // records), evaluates the pairs of each and sums both across its lanes at once.
-// ABS: with the sums of |rep| + |att|, which FP32 mode adds in plain FP32, by
-// ascending staged index.
+// ABS (FP64 mode): with the sums of |rep| + |att|.
 template <bool F32, bool ABS>
 __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
     const TrialPt *__restrict__ pts, const int32_t *__restrict__ ps, const uint4 *__restrict__ cpos,
@@ -405,13 +403,13 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
     double *__restrict__ out_abs, int *__restrict__ status)
 {
     extern __shared__ __align__(128) unsigned char dyn[];
-    constexpr bool kOrdered = F32 && ABS;
-    using SH = NbShared<kOrdered ? kBufOrdered : kBufFull>;
+    static_assert(!(F32 && ABS), "k_trial_scaled");
+    using SH = NbShared<kBufFull>;
     constexpr int kBuf = SH::kBuf;
     SH &sh = *reinterpret_cast<SH *>(dyn);
-    // per-point sums over the passes: FP32 mode float-float (hi, lo) and
-    // uabs in .z; FP64 mode energy and uabs in .x, .y
-    __shared__ typename std::conditional<F32, float4, double2>::type part[kPChunk];
+    // per-point sums over the passes: FP32 mode float-float; FP64 mode energy
+    // and uabs
+    __shared__ typename std::conditional<F32, float2, double2>::type part[kPChunk];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (threadIdx.x == 0) mbar_init(&sh.bar, 1);
     nb_field<F32, false>(sh, ff, fd);
@@ -441,35 +439,18 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
                     uint32_t mask[2];
                     TrialDrain<F32, SH> D0(sh, t0, R2), D1(sh, t1, R2);
                     unsigned short *list = sh.list[w];
-                    if constexpr (kOrdered) {
-                        const uint4 P[2] = {t0.P, t1.P};
-                        nb_screen_exact<2>(sh.fl, sh.raw, nst, P, pf, R2, r2hi, wrap, mask);
-                        nb_flush(list, nb_list_ordered(list, mask[0], rows, sh.raw, t0.excl), D0);
-                        if (i + 1 < pn) nb_flush(list, nb_list_ordered(list, mask[1], rows, sh.raw, t1.excl), D1);
-                    } else {
-                        nb_screen<2>(sh.fl, nst, pf, r2hi, wrap, mask);
-                        nb_flush(list, nb_append(list, 0, mask[0], rows, 0), D0);
-                        if (i + 1 < pn) nb_flush(list, nb_append(list, 0, mask[1], rows, 0), D1);
-                    }
+                    nb_screen<2>(sh.fl, nst, pf, r2hi, wrap, mask);
+                    nb_flush(list, nb_append(list, 0, mask[0], rows, 0), D0);
+                    if (i + 1 < pn) nb_flush(list, nb_append(list, 0, mask[1], rows, 0), D1);
                     // lane 0 gets point i, lane 16 point i + 1
                     const int k = i + (lane >> 4);
                     const bool mine = (lane & 15) == 0 && k < pn;
                     if constexpr (F32) {
                         FF e[2] = {FF{D0.eh, D0.el}, FF{D1.eh, D1.el}};
                         FF s = warp_sum_many<2>(e);
-                        float a = 0.f;
-                        if constexpr (ABS) {
-                            float keep = lane & 16 ? D1.mag : D0.mag;
-                            a = keep + __shfl_xor_sync(0xffffffffu, lane & 16 ? D0.mag : D1.mag, 16);
-#pragma unroll
-                            for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-                        }
                         if (mine) {
-                            if (base > 0) {
-                                s = ff_add(FF{part[k].x, part[k].y}, s);
-                                a += part[k].z;
-                            }
-                            part[k] = make_float4(s.hi, s.lo, a, 0.f);
+                            if (base > 0) s = ff_add(FF{part[k].x, part[k].y}, s);
+                            part[k] = make_float2(s.hi, s.lo);
                         }
                     } else {
                         double e[2] = {D0.rep - D0.att, D1.rep - D1.att}, m[2] = {D0.rep + D0.att, D1.rep + D1.att};
@@ -488,16 +469,133 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
             __syncthreads();
             for (int i = threadIdx.x; i < pn; i += blockDim.x) {
                 const int k = pts[pb + i].idx;
-                double e, a;
-                if constexpr (F32) {
-                    e = (double)part[i].x + (double)part[i].y;
-                    a = (double)part[i].z;
-                } else {
-                    e = part[i].x;
-                    a = part[i].y;
+                out[k] = F32 ? (double)part[i].x + (double)part[i].y : (double)part[i].x;
+                if constexpr (ABS) out_abs[k] = part[i].y;
+            }
+            __syncthreads();  // the sums are read before the next chunk's
+        }
+    }
+}
+
+// FP32 mode with the sums of |rep| + |att|, which are plain FP32: their order --
+// the pairs of a pass of kBufOrdered records by ascending index, 32 at a time --
+// is part of the result to its last digits.  One point per warp, two rows a
+// step, a vote and a population count each, which lists the pairs in that order
+// as it screens them.  Masks and lists as above, put in order afterwards, took
+// 1.40 instead of 1.25 ms for 800,000 points against 2^20 particles.
+constexpr int kScaledWarps = 8;
+struct __align__(16) ScaledShared {
+    uint4 raw[kBufOrdered];
+    float4 fl[kBufOrdered];
+    int q[kScaledWarps][kNbQ];
+    RunList runs;
+    uint64_t bar;
+    union {
+        float4 f[kMaxSpecies * kMaxSpecies];
+        double2 d[kMaxSpecies * kMaxSpecies];
+    } field;
+};
+
+__global__ void __launch_bounds__(kScaledWarps * 32) k_trial_scaled(
+    const TrialPt *__restrict__ pts, const int32_t *__restrict__ ps, const uint4 *__restrict__ cpos,
+    const int32_t *__restrict__ cs, int T, int64_t ncell, uint64_t R2, float r2hi, bool wrap,
+    const __grid_constant__ FieldF ff, const __grid_constant__ FieldD fd, double *__restrict__ out,
+    double *__restrict__ out_abs, int *__restrict__ status)
+{
+    extern __shared__ __align__(128) unsigned char dyn[];
+    using SH = ScaledShared;
+    SH &sh = *reinterpret_cast<SH *>(dyn);
+    __shared__ float4 part[kPChunk];  // per-point sums over the passes: hi, lo, uabs
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    const float r2lo = r2hi - 2e-5f * r2hi;
+    if (threadIdx.x == 0) mbar_init(&sh.bar, 1);
+    nb_field<true, false>(sh, ff, fd);
+    __syncthreads();
+    unsigned parity = 0;
+    int *Q = sh.q[w];
+    for (int64_t c = blockIdx.x; c < ncell; c += gridDim.x) {
+        const int p0 = ps[c], p1 = ps[c + 1];
+        if (p1 == p0) continue;  // uniform across the block
+        const int cx = (int)(c % T), cy = (int)((c / T) % T), cz = (int)(c / ((int64_t)T * T));
+        __syncthreads();
+        if (w == 0) runs27(cs, T, cx, cy, cz, sh.runs);
+        __syncthreads();
+        const int total = sh.runs.end[17];
+        const uint32_t cx0 = cell_centre(cx, T), cy0 = cell_centre(cy, T), cz0 = cell_centre(cz, T);
+        for (int pb = p0; pb < p1; pb += kPChunk) {
+            const int pn = min(kPChunk, p1 - pb);
+            for (int base = 0; base < max(total, 1); base += kBufOrdered) {
+                const int nst = max(min(kBufOrdered, total - base), 0);
+                if ((base > 0 || pb == p0 || total > kBufOrdered) &&
+                    !nb_stage(sh, cpos, base, base + nst, cx0, cy0, cz0, parity, status))
+                    return;
+                for (int i = w; i < pn; i += kScaledWarps) {
+                    const TrialPt tp = pts[pb + i];
+                    const float3 pf = make_float3(rel_f(tp.P.x, cx0), rel_f(tp.P.y, cy0), rel_f(tp.P.z, cz0));
+                    TrialDrain<true, SH> D(sh, tp, R2);
+                    int head = 0, n = 0;
+                    for (int b = 0; b < nst; b += 64) {
+                        bool in[2], band[2];
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const int f = b + 32 * u + lane;
+                            in[u] = band[u] = false;
+                            if (f < nst) {
+                                const float4 q = sh.fl[f];
+                                float dx = pf.x - q.x, dy = pf.y - q.y, dz = pf.z - q.z;
+                                if (wrap) {
+                                    dx = wrap_grid(dx);
+                                    dy = wrap_grid(dy);
+                                    dz = wrap_grid(dz);
+                                }
+                                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                                const bool other = __float_as_uint(q.w) != tp.excl;
+                                in[u] = other && r2 < r2lo;
+                                band[u] = other && r2 >= r2lo && r2 <= r2hi;
+                            }
+                        }
+                        // inside the thin band around rc^2 the exact integer test decides
+                        if (__any_sync(0xffffffffu, band[0] || band[1])) {
+#pragma unroll
+                            for (int u = 0; u < 2; ++u)
+                                if (band[u]) in[u] = grid_sep(tp.P, sh.raw[b + 32 * u + lane]).g < R2;
+                        }
+                        const unsigned b0 = __ballot_sync(0xffffffffu, in[0]), b1 = __ballot_sync(0xffffffffu, in[1]);
+                        if ((b0 | b1) == 0u) continue;
+                        const int end = head + n, n0 = __popc(b0);
+                        if (in[0]) Q[(end + __popc(b0 & lt)) & (kNbQ - 1)] = b + lane;
+                        if (in[1]) Q[(end + n0 + __popc(b1 & lt)) & (kNbQ - 1)] = b + 32 + lane;
+                        n += n0 + __popc(b1);
+                        if (n >= 32) {
+                            __syncwarp();
+                            do {
+                                D(Q[(head + lane) & (kNbQ - 1)]);
+                                head = (head + 32) & (kNbQ - 1);
+                                n -= 32;
+                            } while (n >= 32);
+                            __syncwarp();
+                        }
+                    }
+                    __syncwarp();
+                    if (lane < n) D(Q[(head + lane) & (kNbQ - 1)]);
+                    __syncwarp();
+                    FF s = ff_warp_sum(FF{D.eh, D.el});
+                    float a = warp_sum(D.mag);
+                    if (lane == 0) {
+                        if (base > 0) {
+                            s = ff_add(FF{part[i].x, part[i].y}, s);
+                            a += part[i].z;
+                        }
+                        part[i] = make_float4(s.hi, s.lo, a, 0.f);
+                    }
                 }
-                out[k] = e;
-                if constexpr (ABS) out_abs[k] = a;
+            }
+            __syncthreads();
+            for (int i = threadIdx.x; i < pn; i += blockDim.x) {
+                const int k = pts[pb + i].idx;
+                out[k] = (double)part[i].x + (double)part[i].y;
+                out_abs[k] = (double)part[i].z;
             }
             __syncthreads();  // the sums are read before the next chunk's
         }
@@ -514,25 +612,36 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
 // cell, which is what bounds small calls: 64 points against 2,048 particles
 // take 16 us instead of 52 (FP64), against 2^20 particles 16 instead of 78.
 // Many points share their cell's staged records, so the binned path wins where
-// the points are many, the later the more cells it has to pass over.  Direct
-// and binned, against 2,048 / 20,000 / 2^20 particles: FP64 at 4,096 points
-// 44 / 44 / 45 us and (8,192 points) 61 / 62 / 126, where direct takes twice
-// the 44; FP32 at 16,384 points 53 / 54 / 62 and 71 / 61 / 153.
+// the points are many, the later the more cells they are spread over (about
+// 12 ns a cell that holds some).  Direct and binned, against 2,048 / 20,000 /
+// 2^20 particles: FP64 at 4,096 points 44 / 44 / 45 us and (8,192 points) 61 /
+// 62 / 126, where direct takes twice the 44; FP32 at 16,384 points 53 / 54 / 62
+// and 71 / 61 / 153; with |rep| + |att| 41 / 35 / 60 and 85 / 74 / 224.  The
+// lines below follow these, with a share of the cells for large boxes.
 constexpr int kDirectWarps = 4;
-constexpr int64_t kDirectPoints64 = 4096, kDirectPoints32 = 16384;
+static int64_t direct_points(const gcmc_ctx *ctx, bool abs)
+{
+    if (ctx->precision == GCMC_FP64) return std::max<int64_t>(4096, ctx->ncell / 6);
+    return abs ? std::max<int64_t>(32768, 2 * ctx->ncell) : std::max<int64_t>(16384, ctx->ncell);
+}
 
-template <bool F32>
-__global__ void __launch_bounds__(kDirectWarps * 32) k_trial_direct(
+// ORDERED (FP32 mode with |rep| + |att|): one warp per point, the pairs listed
+// by ascending index in passes of kBufOrdered records as the binned path lists
+// them, so that the plain FP32 sums are the same bits.
+template <bool F32, bool ORDERED>
+__global__ void __launch_bounds__((ORDERED ? 1 : kDirectWarps) * 32) k_trial_direct(
     const double *__restrict__ pos, const int32_t *__restrict__ species, const int64_t *__restrict__ exclude, double q,
     int T, int S, const uint4 *__restrict__ cpos, const int32_t *__restrict__ cs, uint64_t R2, float r2hi,
     const __grid_constant__ FieldF ff, const __grid_constant__ FieldD fd, double *__restrict__ out,
     double *__restrict__ out_abs, volatile int *__restrict__ host_status)
 {
-    constexpr int NT = kDirectWarps * 32;
+    constexpr int NW = ORDERED ? 1 : kDirectWarps, NT = NW * 32;
+    constexpr int kPass = ORDERED ? kBufOrdered : 1 << 30;
+    static_assert(kBufOrdered % (2 * 32) == 0, "a pass is whole steps");
     __shared__ RunList runs;
-    __shared__ int4 queue[kDirectWarps][kNbQ];
-    __shared__ double2 red[kDirectWarps];
-    __shared__ float4 redf[kDirectWarps];
+    __shared__ int4 queue[NW][kNbQ];
+    __shared__ double2 red[NW];
+    __shared__ float4 redf[NW];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t k = blockIdx.x;
     const int t = species[k];
@@ -562,6 +671,8 @@ __global__ void __launch_bounds__(kDirectWarps * 32) k_trial_direct(
     int head = 0, nq = 0;
     float eh = 0.f, el = 0.f, mag = 0.f;
     double rep = 0.0, att = 0.0;
+    FF sum = {0.f, 0.f};  // ORDERED: of the passes
+    float sum_mag = 0.f;
     auto drain = [&](int n) {
         __syncwarp();
         if (lane < n) {
@@ -608,17 +719,24 @@ __global__ void __launch_bounds__(kDirectWarps * 32) k_trial_direct(
         for (int u = 0; u < 2; ++u) {
             const int ex = (int)(X[0] - r[u].x), ey = (int)(X[1] - r[u].y), ez = (int)(X[2] - r[u].z);
             const float gx = (float)ex, gy = (float)ey, gz = (float)ez;
-            const bool in = have[u] && r[u].w != excl && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) <= r2hi;
+            bool in = have[u] && r[u].w != excl && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) <= r2hi;
+            if (ORDERED && in) in = grid_sep(make_uint4(X[0], X[1], X[2], 0u), r[u]).g < R2;
             const unsigned b = __ballot_sync(0xffffffffu, in);
             if (in) Q[(head + nq + __popc(b & lt)) & (kNbQ - 1)] = make_int4(ex, ey, ez, (int)tag_species(r[u].w));
             nq += __popc(b);
         }
         while (nq >= 32) drain(32);
+        if (ORDERED && ((base + 2 * NT) % kPass == 0 || base + 2 * NT >= total)) {
+            if (nq > 0) drain(nq);
+            sum = ff_add(sum, ff_warp_sum(FF{eh, el}));
+            sum_mag += warp_sum(mag);
+            eh = el = mag = 0.f;
+        }
     }
     if (nq > 0) drain(nq);
     if constexpr (F32) {
-        const FF s = ff_warp_sum(FF{eh, el});
-        const float a = warp_sum(mag);
+        const FF s = ORDERED ? sum : ff_warp_sum(FF{eh, el});
+        const float a = ORDERED ? sum_mag : warp_sum(mag);
         if (lane == 0) redf[w] = make_float4(s.hi, s.lo, a, 0.f);
     } else {
         const double e = warp_sum(rep - att), a = warp_sum(rep + att);
@@ -630,7 +748,7 @@ __global__ void __launch_bounds__(kDirectWarps * 32) k_trial_direct(
         if constexpr (F32) {
             FF s = {redf[0].x, redf[0].y};
             float ua = redf[0].z;
-            for (int i = 1; i < kDirectWarps; ++i) {
+            for (int i = 1; i < NW; ++i) {
                 s = ff_add(s, FF{redf[i].x, redf[i].y});
                 ua += redf[i].z;
             }
@@ -639,7 +757,7 @@ __global__ void __launch_bounds__(kDirectWarps * 32) k_trial_direct(
         } else {
             e = red[0].x;
             a = red[0].y;
-            for (int i = 1; i < kDirectWarps; ++i) {
+            for (int i = 1; i < NW; ++i) {
                 e += red[i].x;
                 a += red[i].y;
             }
@@ -1069,7 +1187,7 @@ __global__ void __launch_bounds__(kNbWarps * 32, 5) k_cell_grad(const uint4 *__r
                             uint32_t x = i == i0 ? mask[0] : mask[1];
                             const int self = own + pb + i - base;  // the particle's own record
                             if (self >= 0 && self < nst && (self & 31) == lane) x &= ~(1u << (rows - 1 - (self >> 5)));
-                            nb_flush(list, nb_list_ordered(list, x, rows, sh.raw, 0xFFFFFFFFu), D);
+                            nb_flush(list, nb_list_ordered(list, x, rows), D);
                             // lanes 0, 8, 16 get the force's x, y, z
                             Sum f[4] = {to_sum(D.fx), to_sum(D.fy), to_sum(D.fz), Sum{}};
                             const Sum force = warp_sum_many<4>(f);
@@ -1199,21 +1317,20 @@ gcmc_status trial_energy(gcmc_ctx *ctx, const double *pos, const int32_t *specie
     float r2hi;
     bool wrap;
     screen_bound(ctx, r2hi, wrap);
-    // FP32 sums of magnitudes keep the order of the binned path
-    if (m <= (ctx->precision == GCMC_FP64 ? kDirectPoints64 : out_abs ? 0 : kDirectPoints32)) {
+    if (m <= direct_points(ctx, out_abs != nullptr)) {
         st = ensure_pinned(ctx, kPinnedBytes);
         if (st != GCMC_OK) return st;
         // the status word lies in pinned host memory, written by the kernel
         volatile int *status = (volatile int *)((double *)ctx->h_pinned + 13);
         *status = 0;
-        if (ctx->precision == GCMC_FP32)
-            k_trial_direct<true><<<(unsigned)m, kDirectWarps * 32, 0, s>>>(pos, species, exclude, ctx->q, ctx->T, ctx->S,
-                                                                          ctx->cpos, ctx->cell_start, ctx->R2, r2hi,
-                                                                          ctx->ff, ctx->fd, out, out_abs, status);
-        else
-            k_trial_direct<false><<<(unsigned)m, kDirectWarps * 32, 0, s>>>(pos, species, exclude, ctx->q, ctx->T, ctx->S,
-                                                                           ctx->cpos, ctx->cell_start, ctx->R2, r2hi,
-                                                                           ctx->ff, ctx->fd, out, out_abs, status);
+        auto launch = [&](auto kern, int warps) {
+            kern<<<(unsigned)m, warps * 32, 0, s>>>(pos, species, exclude, ctx->q, ctx->T, ctx->S, ctx->cpos,
+                                                    ctx->cell_start, ctx->R2, r2hi, ctx->ff, ctx->fd, out, out_abs,
+                                                    status);
+        };
+        if (ctx->precision == GCMC_FP64) launch(k_trial_direct<false, false>, kDirectWarps);
+        else if (out_abs) launch(k_trial_direct<true, true>, 1);
+        else launch(k_trial_direct<true, false>, kDirectWarps);
         ctx->launches += 1;
         GCMC_CUDA(ctx, cudaGetLastError());
         GCMC_CUDA(ctx, cudaStreamSynchronize(s));
@@ -1249,19 +1366,19 @@ gcmc_status trial_energy(gcmc_ctx *ctx, const double *pos, const int32_t *specie
     if (st != GCMC_OK) return st;
     k_trial_place<<<gb, 256, 0, s>>>(tmp, cid, m, ps, fill, pts);
     const unsigned nb = nb_blocks(ctx, ncell);
-    auto launch = [&](auto kern, size_t smem) {
+    auto launch = [&](auto kern, int warps, size_t smem) {
         gcmc_status r = nb_smem(ctx, kern, smem);
         if (r == GCMC_OK)
-            kern<<<nb, kNbWarps * 32, smem, s>>>(pts, ps, ctx->cpos, ctx->cell_start, ctx->T, ncell, ctx->R2, r2hi, wrap,
-                                                 ctx->ff, ctx->fd, out, out_abs, ctx->d_status);
+            kern<<<nb, warps * 32, smem, s>>>(pts, ps, ctx->cpos, ctx->cell_start, ctx->T, ncell, ctx->R2, r2hi, wrap,
+                                              ctx->ff, ctx->fd, out, out_abs, ctx->d_status);
         return r;
     };
     if (ctx->precision == GCMC_FP32)
-        st = out_abs ? launch(k_trial_energy<true, true>, sizeof(NbShared<kBufOrdered>))
-                     : launch(k_trial_energy<true, false>, sizeof(NbShared<kBufFull>));
+        st = out_abs ? launch(k_trial_scaled, kScaledWarps, sizeof(ScaledShared))
+                     : launch(k_trial_energy<true, false>, kNbWarps, sizeof(NbShared<kBufFull>));
     else
-        st = out_abs ? launch(k_trial_energy<false, true>, sizeof(NbShared<kBufFull>))
-                     : launch(k_trial_energy<false, false>, sizeof(NbShared<kBufFull>));
+        st = out_abs ? launch(k_trial_energy<false, true>, kNbWarps, sizeof(NbShared<kBufFull>))
+                     : launch(k_trial_energy<false, false>, kNbWarps, sizeof(NbShared<kBufFull>));
     if (st != GCMC_OK) return st;
     ctx->launches += 3;
     GCMC_CUDA(ctx, cudaGetLastError());

@@ -24,7 +24,7 @@ FEW = 4096
 
 
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
-@pytest.mark.parametrize("m", [1, 2, FEW, FEW + 1, 4 * FEW, 4 * FEW + 1])
+@pytest.mark.parametrize("m", [1, 2, FEW, FEW + 1, 4 * FEW, 4 * FEW + 1, 8 * FEW + 1])
 @pytest.mark.parametrize("n,L,rc,S", [(0, 8.0, 2.5, 1), (90, 5.6, 2.5, 2), (1500, 7.6, 2.5, 3), (1000, 13.0, 2.5, 2)])
 def test_few_and_many_points(precision, m, n, L, rc, S):
     pos, types, eps, sigma = W.tiny_system(n=max(n, 1), L=L, rc=rc, n_species=S, seed=n + 3)
@@ -45,6 +45,21 @@ def test_few_and_many_points(precision, m, n, L, rc, S):
     assert np.allclose(gabs.cpu().numpy()[pick], uabs, rtol=1e-5, atol=0)
     alone = b.trial_energy(tp, ts, exclude=torch.as_tensor(excl)).cpu().numpy()
     assert np.all(np.abs(alone[pick] - ref) <= TOL[precision] * uabs)
+
+
+@pytest.mark.parametrize("n,L", [(90, 5.6), (1500, 7.6), (2000, 16.0)])
+def test_fp32_magnitudes_do_not_depend_on_the_path(n, L):
+    """The plain FP32 sums of |rep| + |att| of the same points, one block per point
+    and binned (one point more), bit for bit, also over several passes."""
+    m = 8 * FEW
+    pos, types, eps, sigma = W.tiny_system(n=n, L=L, rc=2.5, n_species=2, seed=n)
+    b = Box(L, 2.5, eps, sigma, precision="fp32")
+    b.build_cells(torch.as_tensor(pos), torch.as_tensor(types))
+    tp, ts = W.insertion_points(m + 1, L, 2, 6)
+    excl = torch.arange(m + 1) % 11 - 1
+    few = b.trial_energy(tp[:m], ts[:m], exclude=excl[:m], with_abs=True)[1]
+    many = b.trial_energy(tp, ts, exclude=excl, with_abs=True)[1]
+    assert torch.equal(few, many[:m])
 
 
 @pytest.mark.parametrize("m", [3, FEW + 1])
