@@ -1734,6 +1734,7 @@ struct LaunchBufs {
     ChainArgs *h_args = nullptr;  // pinned
     ChainOut *h_out = nullptr;    // pinned
     int cap = 0;
+    int device = -1;  // where they are: a thread may use contexts of several devices
     // a captured round (upload, kernel, download) and what it was captured for
     cudaGraphExec_t exec = nullptr;
     void *g_kern = nullptr;
@@ -1748,7 +1749,7 @@ struct LaunchBufs {
         g_K = 0;
         g_smem = 0;
     }
-    ~LaunchBufs()
+    void free_all()
     {
         drop_graph();
         if (ev0) cudaEventDestroy(ev0);
@@ -1757,21 +1758,21 @@ struct LaunchBufs {
         if (d_out) cudaFree(d_out);
         if (h_args) cudaFreeHost(h_args);
         if (h_out) cudaFreeHost(h_out);
+        ev0 = ev1 = nullptr;
+        d_args = h_args = nullptr;
+        d_out = h_out = nullptr;
+        cap = 0;
     }
+    ~LaunchBufs() { free_all(); }
     cudaError_t ensure(int k)
     {
-        if (k <= cap) return cudaSuccess;
-        drop_graph();
-        if (d_args) cudaFree(d_args);
-        if (d_out) cudaFree(d_out);
-        if (h_args) cudaFreeHost(h_args);
-        if (h_out) cudaFreeHost(h_out);
-        d_args = nullptr;
-        d_out = nullptr;
-        h_args = nullptr;
-        h_out = nullptr;
-        cap = 0;
-        cudaError_t e = cudaMalloc(&d_args, k * sizeof(ChainArgs));
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (k <= cap && dev == device) return cudaSuccess;
+        free_all();
+        device = dev;
+        e = cudaMalloc(&d_args, k * sizeof(ChainArgs));
         if (e == cudaSuccess) e = cudaMalloc(&d_out, k * sizeof(ChainOut));
         if (e == cudaSuccess) e = cudaMallocHost(&h_args, k * sizeof(ChainArgs));
         if (e == cudaSuccess) e = cudaMallocHost(&h_out, k * sizeof(ChainOut));
