@@ -267,7 +267,7 @@ class Box:
 
     def set_wait_limit(self, ns: int, stall_move: int = -1) -> None:
         """Diagnostic hook: the chain kernel's wait limit in ns (0: the default)
-        and a move at which the committer waits on a flag nothing sets (-1: none)."""
+        and a move at which its warp waits on a flag nothing sets (-1: none)."""
         check(self._lib.gcmc_set_wait_limit(self._h, int(ns), int(stall_move)), self._h)
 
     def build_microcells(self, edge: float = 1.0, capacity: int = 0) -> None:
@@ -524,8 +524,9 @@ class _CellListEnergy(torch.autograd.Function):
             dpos = g["dpos"]
             gp = go.to(dpos.dtype) * dpos
             gp = gp.to(ctx.pos_dtype)
-        ge = go.detach().cpu().to(ctx.e_dtype) * torch.as_tensor(g["deps"], dtype=ctx.e_dtype)
-        gs = go.detach().cpu().to(ctx.s_dtype) * torch.as_tensor(g["dsigma"], dtype=ctx.s_dtype)
+        go_host = go.detach().cpu()  # one copy (and wait) for both tables
+        ge = go_host.to(ctx.e_dtype) * torch.as_tensor(g["deps"], dtype=ctx.e_dtype)
+        gs = go_host.to(ctx.s_dtype) * torch.as_tensor(g["dsigma"], dtype=ctx.s_dtype)
         ctx.box = None
         return gp, ge, gs, None, None, None, None
 
