@@ -211,7 +211,7 @@ gcmc_status gcmc_check_state(gcmc_ctx *ctx);
 
 /* Diagnostic hook for the failure path: ns = the limit, in ns of the GPU's
  * global timer, of every wait inside the chain kernel (0: the default,
- * 1 s); stall_move >= 0: in later gcmc_run_moves calls the committer, about
+ * 1 s); stall_move >= 0: in later gcmc_run_moves calls a mover, about
  * to commit move stall_move of the call, waits on a flag that nothing sets
  * (-1: no stall).  A wait that runs out stops the chain before its next
  * move: every committed move is applied and booked, the kernel returns and
@@ -393,9 +393,10 @@ gcmc_status gcmc_batch_destroy(gcmc_batch *batch);
 /* Moves first_move .. first_move + n_moves - 1 of every chain, as
  * gcmc_run_moves would run them one context at a time.  seeds, mixes:
  * host, n_chains each; stats: host, n_chains, or NULL.  On the first call
- * with the automatic team shape, the first quarter of the moves runs under
- * shape 0, then every shape is timed on two short chunks (in ascending, then
- * descending shape order) and the shape with the smallest total is kept.  Errors: as gcmc_run_moves, the first
+ * with the automatic choice of moves in flight, the first quarter of the
+ * moves runs under choice 0, then every choice is timed on two short chunks
+ * (in ascending, then descending order) and the one with the smallest total
+ * is kept.  Errors: as gcmc_run_moves, the first
  * failing chain's status (its context has the message); INVALID_ARG. */
 gcmc_status gcmc_batch_run_moves(gcmc_batch *batch, const uint64_t *seeds, uint64_t first_move, int64_t n_moves,
                                  const gcmc_move_mix *mixes, gcmc_move_stats *stats);
@@ -432,7 +433,7 @@ gcmc_status gcmc_batch_export_positions(gcmc_batch *batch, double *const *pos, i
  * The batch keeps the pointers, not the memory.  Errors: INVALID_ARG. */
 gcmc_status gcmc_batch_set_traces(gcmc_batch *batch, gcmc_trace *const *traces);
 
-/* Sets the team shape (-1 automatic, -2 leave unchanged) and reports the
+/* Sets the choice of moves in flight (-1 automatic, -2 leave unchanged) and reports the
  * current one and the per-shape probe times in ms of the last tuning (the
  * sum of the shape's two chunks; host,
  * GCMC_CHAIN_CONFIGS doubles, or NULL).  Errors: INVALID_ARG. */

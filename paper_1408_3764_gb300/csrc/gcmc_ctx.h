@@ -71,7 +71,7 @@ struct gcmc_ctx {
     int chain_config = -1;  // choice of moves in flight of the chain kernel (-1: tuned on the first call)
     bool chain_prof = false;  // chain launches count cycles per role (gcmc_chain_profile)
     uint64_t wait_ns = 0;   // limit of the chain kernel's waits (0: the default, 1 s)
-    int64_t stall_at = -1;  // diagnostic stall of the committer at this move of a call (-1 none)
+    int64_t stall_at = -1;  // diagnostic stall at this move of a call (-1 none)
 
     // ---- microcells (Sec. 3.3), valid while mc_valid
     bool mc_valid = false;
