@@ -34,8 +34,9 @@
 // move leaves the set-up (trial, cells, sums) unreplicated, and W evaluations
 // in flight hide its latency.  Measured against two teams of six warps that
 // evaluated a move together and a separate committing warp: 10^4 moves of
-// 2,048 particles in FP64 23.0 -> 8.5 ms, 2*10^4 of 131,072 in FP32 29.9 ->
-// 15.9 ms, the 64-chain isotherm step 223 -> 130 ms.
+// 2,048 particles in FP64 23.0 -> 8.0 ms (8.5 before the shorter FP64 pair
+// term), 2*10^4 of 131,072 in FP32 29.9 -> 15.6 ms, the 64-chain isotherm step
+// 223 -> 126 ms.
 //
 // The microcell chain (Sec. 3.3.3) is the same kernel with the evaluation over
 // the cube of microcells and both lists kept: 4,000 moves of 87,296 particles in
