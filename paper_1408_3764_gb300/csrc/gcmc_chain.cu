@@ -905,18 +905,19 @@ struct Mover {
     // explicit error band, for N_s = ns: 1 accept, 0 reject, -1 inside the
     // band or not finite (decided in FP64).  The band holds the rounding of
     // every term at its own size: ln K is the difference of z = ln z + ln V
-    // (rounded, 6e-8 |z|) and l = ln N (logf, 1.2e-7 |l|), which cancel.
+    // (rounded, 6e-8 |z|, and |z| <= |ln K| + l) and l = ln N (logf, 1.2e-7 l),
+    // which cancel.
     __device__ __forceinline__ int decide_f32(int type, int sp, int ns, float lnu, float dUf, float uab) const
     {
-        float z = 0.f, l = 0.f;
+        float lnK = 0.f, l = 0.f;
         if (type != 0) {
-            z = a.lnzv_f[sp];
+            const float z = a.lnzv_f[sp];
             l = logf((float)(type == 1 ? ns + 1 : ns));
+            lnK = type == 1 ? z - l : l - z;
         }
-        const float lnK = type == 1 ? z - l : l - z;
         const float bd = a.beta_f * dUf;
         const float band =
-            a.beta_f * a.tol_f * uab + 1e-6f * (1.f + fabsf(z) + fabsf(l) + fabsf(bd) + fabsf(lnu));
+            a.beta_f * a.tol_f * uab + 1e-6f * (1.f + fabsf(lnK) + 2.f * l + fabsf(bd) + fabsf(lnu));
         const float diff = lnu - (lnK - bd);
         if (fabsf(diff) > band) return (diff < 0.f) ? 1 : 0;
         return -1;

@@ -171,9 +171,8 @@ gcmc_status gcmc_create(const gcmc_params *p, void *stream, gcmc_ctx **out)
             ctx->fd.sig2[a * kMaxSpecies + b] = sg * sg;
             pair_constants(e, s, p->L, ctx->fd.rep[a * kMaxSpecies + b], ctx->fd.att[a * kMaxSpecies + b]);
             ctx->ff.c4e[a * kMaxSpecies + b] = (float)(4.0 * e);
-            ctx->ff.sig2[a * kMaxSpecies + b] = (float)(sg * sg);
             ctx->ff.c4e_lo[a * kMaxSpecies + b] = (float)(4.0 * e - (double)(float)(4.0 * e));
-            ctx->ff.sig2_lo[a * kMaxSpecies + b] = (float)(sg * sg - (double)(float)(sg * sg));
+            set_sig2(ctx->ff, a * kMaxSpecies + b, (float)(4.0 * e) > 0.f ? sg * sg : 0.0);
         }
     ctx->max_particles_req = p->max_particles;
     ctx->cap_req = p->cell_capacity;

@@ -104,6 +104,13 @@ gcmc_status cuda_fail(gcmc_ctx *ctx, cudaError_t e, const char *where);
 // gradient's scalars, then its status.
 constexpr size_t kPinnedBytes = 8 * (16 + 2 + 2 * kMaxSpecies * kMaxSpecies + 8);
 
+// sig2 of a species pair as the float-float of FieldF.
+inline void set_sig2(FieldF &f, int k, double sig2)
+{
+    f.sig2[k] = (float)sig2;
+    f.sig2_lo[k] = (float)(sig2 - (double)(float)sig2);
+}
+
 gcmc_status ensure_scratch(gcmc_ctx *ctx, size_t bytes);
 gcmc_status ensure_red(gcmc_ctx *ctx, size_t n);
 gcmc_status ensure_pinned(gcmc_ctx *ctx, size_t bytes);

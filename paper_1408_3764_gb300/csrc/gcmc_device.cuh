@@ -185,6 +185,8 @@ __device__ __forceinline__ GridSep grid_sep(uint4 a, uint4 b)
 //   c4e = 4 eps,  sig2 = (sigma / h)^2,
 //   U = c4e (s^6 s^6 - s^6) with s^2 = sig2 / r_grid^2.
 // ---------------------------------------------------------------------------
+// In FieldF a pair without interaction (c4e = 0 as a float) has sig2 = 0: its s^12
+// would overflow for close pairs, and 0 times that is not 0.
 struct FieldF {
     float c4e[kMaxSpecies * kMaxSpecies];
     float sig2[kMaxSpecies * kMaxSpecies];
@@ -212,7 +214,7 @@ __device__ __forceinline__ void lj_f32(const GridSep &s, float c4e, float sig2, 
     const float att = c4e * s6;
     u = rep - att;
     mag = rep + att;
-    if (s.g == 0ull) {
+    if (s.g == 0ull || att > 3.402823466e38f) {  // coincident, or both terms beyond the floats
         u = __int_as_float(0x7f800000);
         mag = u;
     }
@@ -230,7 +232,9 @@ __device__ __forceinline__ void lj_f32(const GridSep &s, float c4e, float sig2, 
 // Every operation is FP32 (the FP32 pipe); the result uh + ul carries a
 // relative error near 1e-13 of rep + att, where a plain FP32 evaluation
 // carries about 1e-6.  m = rep + att in plain FP32 (an error scale only).
-// g == 0 (both particles on one grid point) gives U = +inf.
+// g == 0 (both particles on one grid point) gives U = +inf, and so does uh where
+// s^12 is beyond the floats (ul is not a number then; sums by ff_acc keep the
+// infinity in their high word).
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float r;
@@ -378,28 +382,37 @@ __device__ __forceinline__ void lj_f64_add(unsigned long long g, double rep, dou
     sum_att = g == 0ull ? sum_att : fma(att, y3, sum_att);
 }
 
-// Float-float values (hi + lo) and their sums (TwoSum on the high words).
+// Float-float values (hi + lo) and their sums (TwoSum on the high words).  INF:
+// an infinite sum (pairs closer than about 6e-4 sigma) keeps its high word: the
+// error term, not a number then, is replaced (fmaxf returns its other argument),
+// one instruction; ff_value leaves the low word out.
 struct FF {
     float hi, lo;
 };
+template <bool INF>
+__device__ __forceinline__ FF ff_norm(float s, float t)
+{
+    if (INF) t = fmaxf(t, -3.402823466e38f);
+    const float h = s + t;
+    return FF{h, t - (h - s)};
+}
+template <bool INF = true>
 __device__ __forceinline__ FF ff_add(FF a, FF b)
 {
     const float s = a.hi + b.hi;
     const float bb = s - a.hi;
     const float e = (a.hi - (s - bb)) + (b.hi - bb);
-    const float t = e + (a.lo + b.lo);  // the same for (a, b) and (b, a): a butterfly leaves every lane one value
-    const float h = s + t;
-    return FF{h, t - (h - s)};
+    return ff_norm<INF>(s, e + (a.lo + b.lo));  // the same for (a, b) and (b, a): a butterfly leaves every lane one value
 }
+template <bool INF = true>
 __device__ __forceinline__ FF ff_add_f(FF a, float x)
 {
     const float s = a.hi + x;
     const float bb = s - a.hi;
     const float e = (a.hi - (s - bb)) + (x - bb);
-    const float t = e + a.lo;
-    const float h = s + t;
-    return FF{h, t - (h - s)};
+    return ff_norm<INF>(s, e + a.lo);
 }
+template <bool INF = true>
 __device__ __forceinline__ FF ff_warp_sum(FF v)
 {
 #pragma unroll
@@ -407,9 +420,13 @@ __device__ __forceinline__ FF ff_warp_sum(FF v)
         FF w;
         w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
         w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-        v = ff_add(v, w);
+        v = ff_add<INF>(v, w);
     }
     return v;
+}
+__device__ __forceinline__ double ff_value(float hi, float lo)
+{
+    return isinf(hi) ? (double)hi : (double)hi + (double)lo;
 }
 
 // ---------------------------------------------------------------------------

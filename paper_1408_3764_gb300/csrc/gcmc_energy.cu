@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_trial_energy(
             __syncthreads();
             for (int i = threadIdx.x; i < pn; i += blockDim.x) {
                 const int k = pts[pb + i].idx;
-                out[k] = F32 ? (double)part[i].x + (double)part[i].y : (double)part[i].x;
+                out[k] = F32 ? ff_value((float)part[i].x, (float)part[i].y) : (double)part[i].x;
                 if constexpr (ABS) out_abs[k] = part[i].y;
             }
             __syncthreads();  // the sums are read before the next chunk's
@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(kScaledWarps * 32) k_trial_scaled(
             __syncthreads();
             for (int i = threadIdx.x; i < pn; i += blockDim.x) {
                 const int k = pts[pb + i].idx;
-                out[k] = (double)part[i].x + (double)part[i].y;
+                out[k] = ff_value(part[i].x, part[i].y);
                 out_abs[k] = (double)part[i].z;
             }
             __syncthreads();  // the sums are read before the next chunk's
@@ -752,7 +752,7 @@ __global__ void __launch_bounds__((ORDERED ? 1 : kDirectWarps) * 32) k_trial_dir
                 s = ff_add(s, FF{redf[i].x, redf[i].y});
                 ua += redf[i].z;
             }
-            e = (double)s.hi + (double)s.lo;
+            e = ff_value(s.hi, s.lo);
             a = (double)ua;
         } else {
             e = red[0].x;
@@ -935,7 +935,7 @@ __global__ void __launch_bounds__(kNbWarps * 32) k_cell_energy(const uint4 *__re
             if (threadIdx.x < 2) {
                 FF sum = {0.f, 0.f};
                 for (int k = 0; k < kNbWarps; ++k) sum = ff_add(sum, FF{redf[k][threadIdx.x].x, redf[k][threadIdx.x].y});
-                partial[2 * c + threadIdx.x] = (double)sum.hi + (double)sum.lo;
+                partial[2 * c + threadIdx.x] = ff_value(sum.hi, sum.lo);
             }
         } else {
             const double e = warp_sum(D.rep - D.att), vw = warp_sum(6.0 * D.att - 12.0 * D.rep);  // r U'(r)
@@ -1104,7 +1104,7 @@ __device__ __forceinline__ void sum_add(FF &a, float x) { a = ff_add_f(a, x); }
 __device__ __forceinline__ void sum_add(double &a, double x) { a += x; }
 __device__ __forceinline__ FF to_sum(float x) { return FF{x, 0.f}; }
 __device__ __forceinline__ double to_sum(double x) { return x; }
-__device__ __forceinline__ double sum_value(FF a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double sum_value(FF a) { return ff_value(a.hi, a.lo); }
 __device__ __forceinline__ double sum_value(double a) { return a; }
 
 template <bool F32, int NS>
@@ -1477,13 +1477,15 @@ gcmc_status energy_grad_begin(gcmc_ctx *ctx, float *dpos, bool input_order)
     const unsigned nb = nb_blocks(ctx, ctx->ncell);
     double *part = ctx->d_red;
     double *res = ctx->d_red + (size_t)ctx->ncell * width;
+    FieldF ff = ctx->ff;  // dE/deps of a pair with eps = 0 needs its sigma
+    for (int k = 0; k < kMaxSpecies * kMaxSpecies; ++k) set_sig2(ff, k, ctx->fd.sig2[k]);
     GCMC_CUDA(ctx, cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->stream));
 #define GCMC_GRAD(F, NSP)                                                                                     \
     do {                                                                                                      \
         st = nb_smem(ctx, k_cell_grad<F, NSP>, sizeof(NbShared<kBufOrdered>));                                \
         if (st != GCMC_OK) return st;                                                                         \
         k_cell_grad<F, NSP><<<nb, kNbWarps * 32, sizeof(NbShared<kBufOrdered>), ctx->stream>>>(               \
-            ctx->cpos, ctx->cell_start, ctx->T, ctx->ncell, ctx->R2, r2hi, wrap, S, ctx->ff, ctx->fd,          \
+            ctx->cpos, ctx->cell_start, ctx->T, ctx->ncell, ctx->R2, r2hi, wrap, S, ff, ctx->fd,               \
             1.0 / ctx->h, ctx->d_n, input_order ? ctx->order : nullptr, dpos, part, ctx->d_status);           \
     } while (0)
     if (ctx->precision == GCMC_FP32) {
