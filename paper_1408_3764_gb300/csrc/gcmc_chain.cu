@@ -544,7 +544,7 @@ struct Mover {
         if constexpr (MICRO) evaluate_micro<VIR>(t, o);
         else evaluate_cells<P32, VIR>(t, o);
         if constexpr (P32) {
-            const FF s = ff_warp_sum(FF{o.e, o.el});
+            const FF s = ff_warp_sum<false>(FF{o.e, o.el});  // (not finite: decided in FP64)
             o.e = s.hi;
             o.el = s.lo;
             o.ua = warp_sum(o.ua);
