@@ -1055,27 +1055,32 @@ struct GradDrain {
         const unsigned long long g = (unsigned long long)((long long)ex * ex) +
                                      (unsigned long long)((long long)ey * ey) +
                                      (unsigned long long)((long long)ez * ez);
-        R c4e, s2, coef;  // coef: 1 / r^2, then r U'(r) / r^2
+        // coef: 1 / r^2, then r U'(r) / r^2.  s^2 is bounded where s^12 is far
+        // beyond the floats (coincident pairs: beyond the doubles, whatever
+        // their eps), so that s^6 is finite and rep - att is +inf, not a
+        // difference of infinities.
+        R c4e, s2, coef;
         if constexpr (F32) {
             const float4 c = sh.field.f[k];
             const float r2 = fmaf(__uint2float_rn((uint32_t)(g >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)g));
             const float y = rcp_approx(r2);
-            c4e = c.x;
-            s2 = c.z / r2;
+            c4e = r2 == 0.f ? 1.f : c.x;
+            s2 = fminf(c.z / r2, 1e11f);
             coef = fmaf(fmaf(-r2, y, 1.f), y, y);
         } else {
             const double2 c = sh.field.d[k];
             const double r2 = u64_to_f64(g);
             double y;
-            c4e = c.x;
+            c4e = g == 0ull ? 1.0 : c.x;
             s2 = div_by_g(c.y, r2, g, y);
-            if (g == 0ull) s2 = __longlong_as_double(0x7ff0000000000000ll);
+            if (g == 0ull) s2 = 1e80;
             coef = fma(fma(-r2, y, 1.0), y, y);
         }
         const R s6 = s2 * s2 * s2;
         const R rep = c4e * s6 * s6, att = c4e * s6;
         const R rdu = (R)(-12) * rep + (R)6 * att;  // r U'(r)
         coef *= rdu;
+        if constexpr (F32) coef = fmaxf(coef, -3.402823466e38f);  // no force along an axis without distance
         fx += coef * (R)ex;
         fy += coef * (R)ey;
         fz += coef * (R)ez;
@@ -1226,7 +1231,10 @@ __global__ void __launch_bounds__(kNbWarps * 32, 5) k_cell_grad(const uint4 *__r
                         const int64_t row = order ? order[h0 + pb + i] : base_s[tag_species(tg)] + tag_index(tg);
 #pragma unroll
                         for (int a = 0; a < 3; ++a) {
-                            if constexpr (F32) dpos[3 * row + a] = (fpart[i][a].hi + fpart[i][a].lo) * (float)inv_h;
+                            if constexpr (F32) {
+                                const FF f = fpart[i][a];
+                                dpos[3 * row + a] = (isinf(f.hi) ? f.hi : f.hi + f.lo) * (float)inv_h;
+                            }
                             else dpos[3 * row + a] = (float)(fpart[i][a] * inv_h);
                         }
                     }

@@ -104,3 +104,52 @@ def test_total_energy_and_gradient_of_an_overlap(precision, S, apart):
         assert abs(energy - o.total_energy()) <= 1e-12 * abs(energy)
         for k in ("energy", "virial"):
             assert abs(g[k] - ref[k]) <= 1e-11 * abs(ref[k])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("S", [1, 3])
+@pytest.mark.parametrize("steps", [0, 1, 40, 200, 2000, 50_000])
+def test_gradient_of_a_pair_on_an_axis(precision, S, steps):
+    """A pair `steps` grid points (2.1e-9 each) apart along x: the infinities of
+    the energy, the virial and the force along x, no NaN in any result.  (A
+    coincident pair's force has no direction and is not looked at.)"""
+    L, n = 9.0, 300
+    pos, types, eps, sigma = W.tiny_system(n=n, L=L, rc=2.5, n_species=S, seed=4)
+    h = L / 2.0 ** 32
+    pos[0] = (np.floor(pos[0] / h) + 0.5) * h
+    pos[1] = pos[0] + np.array([steps * h, 0.0, 0.0])
+    b = Box(L, 2.5, eps, sigma, precision=precision)
+    b.build_cells(torch.as_tensor(pos), torch.as_tensor(types))
+    energy, g = b.total_energy(), b.energy_grad(input_order=True)
+    force = g["dpos"].cpu().numpy()
+    assert not np.isnan(g["deps"]).any() and not np.isnan(g["dsigma"]).any()
+    if precision == "fp32" or steps == 0:
+        assert energy == math.inf and g["energy"] == math.inf and g["virial"] == -math.inf
+        assert g["deps"].max() == math.inf and g["dsigma"].max() == math.inf
+    else:
+        o = O.System(L, 2.5, eps, sigma)
+        o.build(pos, types)
+        ref = o.energy_grad()
+        for k in ("energy", "virial"):
+            assert abs(g[k] - ref[k]) <= 1e-11 * abs(ref[k])
+    assert not np.isnan(force[2:]).any() and np.isfinite(force[2:]).all()
+    if steps:
+        # U falls steeply with the distance: dE/dx of the left one is +inf
+        assert force[0, 0] == np.inf and force[1, 0] == -np.inf
+        assert np.isfinite(force[:2, 1:]).all()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_gradient_without_interaction(precision):
+    """eps = 0: no energy of a close pair, +inf of a coincident one (as the total energy)."""
+    L = 9.0
+    h = L / 2.0 ** 32
+    pos = W.uniform_positions(300, L, 3)
+    pos[0] = (np.floor(pos[0] / h) + 0.5) * h
+    for steps, ref in ((40, 0.0), (0, math.inf)):
+        pos[1] = pos[0] + np.array([steps * h, 0.0, 0.0])
+        b = Box(L, 2.5, [[0.0]], [[1.0]], precision=precision)
+        b.build_cells(torch.as_tensor(pos), torch.zeros(300, dtype=torch.int32))
+        g = b.energy_grad()
+        assert b.total_energy() == ref and g["energy"] == ref
+        assert not np.isnan(g["deps"]).any() and g["deps"][0, 0] > 0.0
