@@ -1055,31 +1055,30 @@ struct GradDrain {
         const unsigned long long g = (unsigned long long)((long long)ex * ex) +
                                      (unsigned long long)((long long)ey * ey) +
                                      (unsigned long long)((long long)ez * ez);
-        // coef: 1 / r^2, then r U'(r) / r^2.  s^2 is bounded where s^12 is far
-        // beyond the floats (coincident pairs: beyond the doubles, whatever
-        // their eps), so that s^6 is finite and rep - att is +inf, not a
-        // difference of infinities.
-        R c4e, s2, coef;
+        // s^2 is bounded where s^12 is far beyond the floats (coincident pairs:
+        // beyond the doubles, whatever their eps), so that s^6 is finite and
+        // rep - att is +inf, not a difference of infinities.  y: about 1 / r^2.
+        R c4e, s2, r2, y;
         if constexpr (F32) {
             const float4 c = sh.field.f[k];
-            const float r2 = fmaf(__uint2float_rn((uint32_t)(g >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)g));
-            const float y = rcp_approx(r2);
+            r2 = fmaf(__uint2float_rn((uint32_t)(g >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)g));
+            y = rcp_approx(r2);
             c4e = r2 == 0.f ? 1.f : c.x;
             s2 = fminf(c.z / r2, 1e11f);
-            coef = fmaf(fmaf(-r2, y, 1.f), y, y);
         } else {
             const double2 c = sh.field.d[k];
-            const double r2 = u64_to_f64(g);
-            double y;
+            r2 = u64_to_f64(g);
             c4e = g == 0ull ? 1.0 : c.x;
             s2 = div_by_g(c.y, r2, g, y);
             if (g == 0ull) s2 = 1e80;
-            coef = fma(fma(-r2, y, 1.0), y, y);
         }
         const R s6 = s2 * s2 * s2;
         const R rep = c4e * s6 * s6, att = c4e * s6;
         const R rdu = (R)(-12) * rep + (R)6 * att;  // r U'(r)
-        coef *= rdu;
+        // rdu / r^2 with one rounding: the quotient corrected by its residual, in as
+        // many instructions as a reciprocal and a product take
+        R coef = rdu * y;
+        coef = fma(fma(-coef, r2, rdu), y, coef);
         if constexpr (F32) coef = fmaxf(coef, -3.402823466e38f);  // no force along an axis without distance
         fx += coef * (R)ex;
         fy += coef * (R)ey;
