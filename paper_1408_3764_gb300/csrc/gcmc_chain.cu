@@ -91,7 +91,6 @@ struct ChainArgs {
     long long maxN;
     int S;
     unsigned long long R2;
-    int rcg;  // smallest integer with rcg^2 >= R2 (per-axis pre-filter)
     float r2hi;  // FP32 squared distances above it are outside the cutoff
     unsigned long long thr_disp, thr_ins;
     uint32_t span;  // 2 D + 1 grid steps
@@ -213,7 +212,7 @@ struct __align__(16) Shared {
     int4 turn;
     LogRec logs[kRS];
     BookRec book[kRS];
-    double2 field[kMaxSpecies * kMaxSpecies];  // FP32 mode: float4 (c4e, sig2, c4e_lo, sig2_lo); FP64: (c4e, sig2)
+    float4 field[kMaxSpecies * kMaxSpecies];  // FP32 mode: (c4e, sig2, c4e_lo, sig2_lo); FP64 pairs read ChainArgs::fd
     int ver[kRS];      // of the log entries: (move << 8) | evaluation, 0 while one is written
     int outlook[kRS];  // of pending moves: (move << 8) | species << 2 | 1 (adds a particle) or 2 (removes one)
     int n[kMaxSpecies];
@@ -875,7 +874,7 @@ struct Mover {
         const int k = p.w & 0xFF;
         const bool neg = (p.w & 0x100) != 0;
         if constexpr (P32) {
-            const float4 c = ((const float4 *)sh.field)[k];
+            const float4 c = sh.field[k];
             float uh, ul, m;
             lj_ff(p.x, p.y, p.z, c.x, c.z, c.y, c.w, uh, ul, m);
             ff_acc(o.e, o.el, neg ? -uh : uh, neg ? -ul : ul);
@@ -1615,10 +1614,9 @@ __global__ void __launch_bounds__(kChainWarps * 32, 1) k_chain(const ChainArgs *
         sh.outlook[tid] = -1;
         sh.ver[tid] = 0;
     }
-    for (int k = tid; k < kMaxSpecies * kMaxSpecies; k += NTH) {
-        if constexpr (F32) ((float4 *)sh.field)[k] = make_float4(a.ff.c4e[k], a.ff.sig2[k], a.ff.c4e_lo[k], a.ff.sig2_lo[k]);
-        else sh.field[k] = make_double2(a.fd.c4e[k], a.fd.sig2[k]);
-    }
+    if constexpr (F32)
+        for (int k = tid; k < kMaxSpecies * kMaxSpecies; k += NTH)
+            sh.field[k] = make_float4(a.ff.c4e[k], a.ff.sig2[k], a.ff.c4e_lo[k], a.ff.sig2_lo[k]);
     if (tid < 12) sh.prof[tid] = 0ull;
     if (tid == 0) {
         sh.turn = make_int4(0, 0, 0, 0);
@@ -1664,8 +1662,6 @@ static void *chain_kernel(bool prof)
 // instead of 7.5 ms for the 4,000 moves named at the top).
 constexpr int kMicroMovers = kMaxMovers;
 
-int chain_threads(int) { return kChainWarps * 32; }
-
 // One chain of a launch: its context, random stream, moves and outputs.
 struct ChainJob {
     gcmc_ctx *ctx;
@@ -1696,7 +1692,6 @@ static void fill_args(ChainArgs &a, const ChainJob &j, int movers, ChainOut *out
     a.maxN = ctx->maxN;
     a.S = ctx->S;
     a.R2 = ctx->R2;
-    a.rcg = ctx->rcg;
     // FP32 r^2 from exact integer separations carries a relative error below
     // 1e-6: every pair inside the cutoff passes the screen
     a.r2hi = (float)((double)ctx->R2 * (1.0 + 1e-5));
@@ -1846,7 +1841,7 @@ static gcmc_status run_jobs(std::vector<ChainJob> &jobs, cudaStream_t st, bool f
             if (r == cudaSuccess) r = cudaMemsetAsync(B.d_out, 0, K * sizeof(ChainOut), st);
             if (r == cudaSuccess) {
                 void *kargs[] = {(void *)&B.d_args};
-                r = cudaLaunchKernel(kern, dim3(K), dim3(chain_threads(config)), kargs, smem, st);
+                r = cudaLaunchKernel(kern, dim3(K), dim3(kChainWarps * 32), kargs, smem, st);
             }
             if (r == cudaSuccess)
                 r = cudaMemcpyAsync(B.h_out, B.d_out, K * sizeof(ChainOut), cudaMemcpyDeviceToHost, st);

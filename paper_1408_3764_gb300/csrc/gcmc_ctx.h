@@ -163,7 +163,6 @@ gcmc_status run_batch(gcmc_ctx *const *ctxs, int K, const uint64_t *seeds, uint6
                       const gcmc_move_mix *mixes, gcmc_move_stats *stats, int &config, int64_t *launches,
                       std::string *err, cudaStream_t stream, bool use_graph, double *probe_ms,
                       double *dev_ms, gcmc_trace *const *traces = nullptr);
-int chain_threads(int config);
 constexpr int kChainConfigs = 4;
 
 }  // namespace gcmc

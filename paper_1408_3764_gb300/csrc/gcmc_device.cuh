@@ -9,17 +9,12 @@
 namespace gcmc {
 
 constexpr int kMaxSpecies = 8;
-constexpr int kWarp = 32;
 
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon et al., SC'11): ten rounds, each two 32x32->64-bit
 // multiplies whose halves are mixed with the other counter words and the
 // key; the key advances by the two Weyl constants between rounds.
 // ---------------------------------------------------------------------------
-struct Words8 {
-    uint32_t w[8];
-};
-
 __device__ __forceinline__ uint4 philox_block(uint4 c, uint2 k)
 {
 #pragma unroll
@@ -33,18 +28,6 @@ __device__ __forceinline__ uint4 philox_block(uint4 c, uint2 k)
         k.y += 0xBB67AE85u;
     }
     return c;
-}
-
-// The eight words of move m of chain `chain`.
-__device__ __forceinline__ Words8 move_words(uint64_t seed, uint64_t m, uint32_t chain)
-{
-    const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
-    const uint4 a = philox_block(make_uint4((uint32_t)m, (uint32_t)(m >> 32), chain, 0u), key);
-    const uint4 b = philox_block(make_uint4((uint32_t)m, (uint32_t)(m >> 32), chain, 1u), key);
-    Words8 r;
-    r.w[0] = a.x; r.w[1] = a.y; r.w[2] = a.z; r.w[3] = a.w;
-    r.w[4] = b.x; r.w[5] = b.y; r.w[6] = b.z; r.w[7] = b.w;
-    return r;
 }
 
 // 53-bit uniform in [0, 1) from words 6 and 7.
@@ -85,36 +68,6 @@ __device__ __forceinline__ int pick_index(uint32_t n, const uint32_t *w, int typ
     return (int)__umulhi(w[5], n);
 }
 
-// Whether pick_index gives the same index for every count in [lo, hi]
-// (1 <= lo <= hi): the counts share k, and a try below lo comes before any
-// try in [lo, hi).
-__device__ __forceinline__ bool pick_is_stable(uint32_t lo, uint32_t hi, const uint32_t *w, int type)
-{
-    const int k = 32 - __clz((int)(hi - 1u));
-    if (32 - __clz((int)(lo - 1u)) != k) return false;
-    if (k == 0) return true;
-    const int sh = 32 - k;
-    uint32_t tries[3];
-    int nt = 1;
-    tries[0] = w[1] >> sh;
-    if (type == 2) {
-        tries[1] = w[2] >> sh;
-        tries[2] = w[3] >> sh;
-        nt = 3;
-    } else if (k <= 16) {
-        tries[1] = (w[1] << 16) >> sh;
-        nt = 2;
-    }
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        if (j < nt) {
-            if (tries[j] < lo) return true;
-            if (tries[j] < hi) return false;
-        }
-    }
-    return false;  // every try fails for some count: the fallback depends on it
-}
-
 // ---------------------------------------------------------------------------
 // Grid and cells
 // ---------------------------------------------------------------------------
@@ -141,20 +94,6 @@ __device__ __forceinline__ int cell_of(uint32_t X, uint32_t Y, uint32_t Z, int T
 {
     return (cell_coord(Z, (uint32_t)T) * T + cell_coord(Y, (uint32_t)T)) * T +
            cell_coord(X, (uint32_t)T);
-}
-
-// Cell id of the neighbour at offset (ox, oy, oz) in {-1,0,1}^3.
-__device__ __forceinline__ int neighbour_cell(int cx, int cy, int cz, int k, int T)
-{
-    int ox = k % 3 - 1, oy = (k / 3) % 3 - 1, oz = k / 9 - 1;
-    int nx = cx + ox, ny = cy + oy, nz = cz + oz;
-    nx += (nx < 0) ? T : 0;
-    nx -= (nx >= T) ? T : 0;
-    ny += (ny < 0) ? T : 0;
-    ny -= (ny >= T) ? T : 0;
-    nz += (nz < 0) ? T : 0;
-    nz -= (nz >= T) ? T : 0;
-    return (nz * T + ny) * T + nx;
 }
 
 // Particle tag stored in the 4th word of a position: (index << 8) | species.
