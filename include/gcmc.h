@@ -179,6 +179,8 @@ gcmc_status gcmc_cell_list(gcmc_ctx *ctx, int32_t *cell_start, int32_t *cell_cou
  * pos: device m x 3 FP64 (quantised as above); species: device m int32;
  * exclude: device m int64 particle ids, -1 = none, or NULL for none;
  * out: device m FP64; out_abs: device m FP64 (the uabs of gcmc_trace) or NULL.
+ * A point on a particle's grid point gets +inf; so does, in FP32 mode, one whose
+ * energy is beyond the floats (a particle closer than about 6e-4 sigma).
  * Errors: STATE, INVALID_ARG, CUDA. */
 gcmc_status gcmc_trial_energy(gcmc_ctx *ctx, const double *pos, const int32_t *species,
                               const int64_t *exclude, int64_t m, double *out, double *out_abs);
@@ -195,8 +197,11 @@ gcmc_status gcmc_trial_energy(gcmc_ctx *ctx, const double *pos, const int32_t *s
  * In FP32 mode a trial within 1e-5 * beta * uabs of the threshold is
  * re-evaluated in FP64 and decided on that value (trace flag bit 1).
  * stats: host, may be NULL; trace: device n_moves records, may be NULL.
- * Errors: STATE, INVALID_ARG (mix), CELL_OVERFLOW, CAPACITY (the chain stops
- * before the offending move: stats->moves_done tells where), NONFINITE, CUDA. */
+ * Limit: the box's cells, two bytes each, and 36,576 bytes (FP32 mode 65,248)
+ * are at most the shared memory a CTA may have.
+ * Errors: STATE, INVALID_ARG (mix, too many cells), CELL_OVERFLOW, CAPACITY (the
+ * chain stops before the offending move: stats->moves_done tells where),
+ * NONFINITE, TIMEOUT (a wait inside the kernel gave up), CUDA. */
 gcmc_status gcmc_run_moves(gcmc_ctx *ctx, uint64_t seed, uint64_t first_move, int64_t n_moves,
                            const gcmc_move_mix *mix, gcmc_move_stats *stats, gcmc_trace *trace);
 
@@ -230,9 +235,11 @@ gcmc_status gcmc_set_wait_limit(gcmc_ctx *ctx, uint64_t ns, int64_t stall_move);
  * count and grown by gcmc_run_moves_micro when a move needs a fuller cell).
  * Valid until a build, a restore or a gcmc_run_moves / batch run (which
  * keep only the 27-cell lists); gcmc_run_moves_micro rebuilds them then.
+ * Limit: 4 bits per microcell, 4 bytes per cell of the cube around a point
+ * (below) and 1,480 bytes are at most the shared memory a CTA may have.
  * Errors: STATE (no cells), INVALID_ARG (edge, capacity, too many
- * microcells for the chain's on-chip counters), CELL_OVERFLOW (a cell holds
- * more than capacity, or more than 15), CUDA. */
+ * microcells), CELL_OVERFLOW (a cell holds more than capacity, or more than
+ * 15), CUDA. */
 gcmc_status gcmc_build_microcells(gcmc_ctx *ctx, double edge, int32_t capacity);
 
 /* The microcells: per_side = M, capacity = slots per cell (host, or NULL);
@@ -243,8 +250,8 @@ gcmc_status gcmc_microcells(gcmc_ctx *ctx, int64_t *per_side, int32_t *capacity,
                             uint32_t *slots);
 
 /* The chain of gcmc_run_moves evaluated over the microcell list (Sec. 3.3.3
- * and 3.3.4): one CTA runs the moves one after another; each trial's energy
- * is the sum over the (2D+1)^3 microcells around the old and the new
+ * and 3.3.4): one CTA, its warps evaluating moves ahead of their turn; each
+ * trial's energy is the sum over the (2D+1)^3 microcells around the old and the new
  * position, D = 1 + floor((rcg - 1) M / 2^32) with rcg the smallest integer
  * with rcg^2 >= the grid cutoff (every cell at most D cells away along each
  * axis; all M when 2D+1 > M).  Same moves, decisions, trace and statistics
@@ -252,7 +259,9 @@ gcmc_status gcmc_microcells(gcmc_ctx *ctx, int64_t *per_side, int32_t *capacity,
  * moves update the microcells (append; removal by swap-with-last) and the
  * 27-cell lists exactly as gcmc_run_moves does, so every other call stays
  * valid.  Rebuilds stale microcells first with the last edge and capacity.
- * Errors: as gcmc_run_moves; STATE when gcmc_build_microcells was never
+ * In FP32 mode the pair terms are plain FP32 (within 1e-5 of uabs).
+ * Errors: as gcmc_run_moves (TIMEOUT after 1 s, which gcmc_set_wait_limit does
+ * not change; no limit on the cells); STATE when gcmc_build_microcells was never
  * called; CELL_OVERFLOW when a microcell of fixed capacity is full. */
 gcmc_status gcmc_run_moves_micro(gcmc_ctx *ctx, uint64_t seed, uint64_t first_move, int64_t n_moves,
                                  const gcmc_move_mix *mix, gcmc_move_stats *stats, gcmc_trace *trace);
@@ -296,6 +305,8 @@ gcmc_status gcmc_total_energy_noalloc(gcmc_ctx *ctx, double *energy);
  *               (host, n_species^2 FP64) or NULL;
  *   dsigma    = dE/dsigma[a][b], same convention, rc fixed (host) or NULL;
  *   energy    = E (host) or NULL;  virial = sum_{i<j} r U'(r) (host) or NULL.
+ * Terms beyond the output type (FP32 mode: beyond the floats) are infinite; the
+ * force of two particles on one grid point has no direction and is not defined.
  * Errors: STATE, CUDA. */
 gcmc_status gcmc_energy_grad(gcmc_ctx *ctx, float *dpos, double *deps, double *dsigma,
                              double *energy, double *virial);
@@ -364,7 +375,10 @@ gcmc_status gcmc_set_chain_profile(gcmc_ctx *ctx, int32_t on);
  * less room on chip); 0 .. GCMC_CHAIN_CONFIGS-1, or -1 to time every choice
  * during the next gcmc_run_moves (after a first quarter of its moves under
  * choice 0) and keep the fastest.  Every choice takes the same moves and
- * decisions and reaches the same configuration.
+ * decisions and reaches the same configuration.  The order in which a trial's
+ * pair terms are added depends on which counts of far cells its evaluation
+ * read, so dU and the running energy may differ between runs in their last
+ * bits (within the precision's tolerance).
  * Errors: INVALID_ARG. */
 #define GCMC_CHAIN_CONFIGS 4
 gcmc_status gcmc_set_chain_config(gcmc_ctx *ctx, int32_t config);

@@ -40,7 +40,7 @@
 //
 // The microcell chain (Sec. 3.3.3) is the same kernel with the evaluation over
 // the cube of microcells and both lists kept: 4,000 moves of 87,296 particles in
-// FP32 19.1 -> 7.5 ms against a block of eight warps that evaluated and
+// FP32 19.2 -> 7.9 ms against a block of eight warps that evaluated and
 // committed one move after another.  Its counters stay in global memory.
 //
 // Movers hand the turn on through shared memory with block-scope fences;
@@ -70,7 +70,10 @@ struct ChainOut {
     double sum_n;
     long long n[kMaxSpecies];
     int status;
-    int pad;                // which waits gave up (1 room in the book, 2 the turn, 4 keeper)
+    // why the chain stopped: waits that gave up (1 room in the book, 2 the turn, 4
+    // the keeper); 8 an evaluation begun at its turn does not hold, 16 capacity or a
+    // record missing from its cell, 32 the species' last record missing
+    int pad;
     long long reevaluated;  // moves evaluated more than once
     long long refines;      // trials decided in FP64 after the FP32 band test
     double virial;          // running virial after the last move (virial runs)
@@ -1658,8 +1661,8 @@ static void *chain_kernel(bool prof)
 {
     return prof ? (void *)k_chain<F32, VIR, true, false> : (void *)k_chain<F32, VIR, false, false>;
 }
-// Moves in flight of a microcell launch: all there is room for (eleven: 8.4
-// instead of 7.5 ms for the 4,000 moves named at the top).
+// Moves in flight of a microcell launch: all there is room for (eleven took 12 %
+// longer for the 4,000 moves named at the top).
 constexpr int kMicroMovers = kMaxMovers;
 
 // One chain of a launch: its context, random stream, moves and outputs.
@@ -2025,17 +2028,19 @@ static gcmc_status run_jobs_tuned(std::vector<ChainJob> &jobs, cudaStream_t st, 
     return run_jobs(jobs, st, f32, config, B, launches, err, use_graph, dev_ms);
 }
 
+// The library's limit on the cells of a chain's box (97,936 in FP64 mode, 83,600
+// in FP32 mode where a CTA may have 227 KB): it leaves the chain's state and four
+// movers at least.  The FP32 share is part of the limit that callers know; both
+// modes need the same room.
 constexpr size_t kChainReserve = 36576, kChainReserveFp32 = 28672;
 
 static gcmc_status check_chain_fits(gcmc_ctx *ctx)
 {
     const size_t smem = ((size_t)ctx->ncell * sizeof(uint16_t) + 15) / 16 * 16;
-    // the documented limit on the cells of a box: what the counters may take
-    // beside kChainReserve bytes of chain state (which hold four movers)
     static_assert(sizeof(Shared) + sizeof(ChainArgs) + 4 * kMoverBytes + 2048 <= kChainReserve, "chain state");
     const size_t queues = ctx->precision == GCMC_FP32 ? kChainReserveFp32 : 0;
     if (smem + kChainReserve + queues > ctx->smem_optin)
-        return fail(ctx, GCMC_ERR_INVALID_ARG, "gcmc_run_moves: too many cells for the on-chip cell counters");
+        return fail(ctx, GCMC_ERR_INVALID_ARG, "gcmc_run_moves: too many cells (the limit counts two bytes of shared memory a cell)");
     if (ctx->T > 1023) return fail(ctx, GCMC_ERR_INVALID_ARG, "gcmc_run_moves: more than 1023 cells per side");
     return GCMC_OK;
 }

@@ -269,8 +269,9 @@ __device__ __forceinline__ double rcp_seed(unsigned long long g)
 }
 
 // a / r2 for r2 = u64_to_f64(g) >= 1 and a > 0, and an approximate reciprocal
-// (to about 2^-44) in y: the seed, one Newton step, and the quotient corrected
-// by its residual, which leaves one rounding.
+// (to about 2^-44) in y: the seed, one Newton-Raphson step, and the quotient
+// corrected by its residual (Markstein, IBM J. Res. Dev. 34, 1990), which leaves
+// one rounding.
 __device__ __forceinline__ double div_by_g(double a, double r2, unsigned long long g, double &y)
 {
     const double y0 = rcp_seed(g);
@@ -281,7 +282,8 @@ __device__ __forceinline__ double div_by_g(double a, double r2, unsigned long lo
 
 // r^-6 and r^-12 in grid units from the exact squared distance (g > 0): six
 // instructions of the FP64 pipe, the third-order step y0 (1 + e + e^2) on the
-// seed among them.  The FP64 pipe bounds the kernels that evaluate pairs (a
+// seed among them (the hyperpower iteration of order three, Altman, Pacific J.
+// Math. 10, 1960).  The FP64 pipe bounds the kernels that evaluate pairs (a
 // warp instruction per 16 cycles and SM), so its instructions are counted: a
 // pair's energy takes 8 where its terms are summed apart and 9 below; with the
 // conversions of the three differences, their squares and a general division

@@ -1018,15 +1018,16 @@ static void sum_partials(gcmc_ctx *ctx, const double *partial, int64_t n, int wi
 //   r U'(r) = -12 rep + 6 att,
 //   dE/deps_ab (half of each ordered pair) += 2 (s^12 - s^6),
 //   dE/dsigma_ab (same) += (12 rep - 6 att) / (2 sigma_ab).
-// One CTA per home cell with its 27 cells staged; one warp per home
-// particle; every pair is met from both of its particles (the forces of a
-// particle are summed by one warp, so nothing is scattered).  The per-cell
+// One CTA per home cell with its 27 cells staged; a warp screens two home
+// particles together and sums the forces of each alone; every pair is met from
+// both of its particles, so nothing is scattered.  The per-cell
 // scalars go to `partial` rows of width 2 + 2 S^2: [E, virial, deps...,
 // dsigma...].  order: the forces are stored at the particles' input rows (the
-// last build's order), otherwise species-major.  NS: partner species in registers (1, 2, or kMaxSpecies).
-// FP32 mode: FP32 pair terms from the exact integer r^2, forces summed in
-// FP32 per lane and FP64 across the warp, the scalars summed in
-// compensated FP32; FP64 mode: FP64 throughout.
+// last build's order), otherwise species-major.  NS: partner species in
+// registers (1, 2, 4 or kMaxSpecies).
+// FP32 mode: FP32 pair terms from the exact integer r^2, forces and tables
+// summed in FP32 per lane and particle, everything beyond that (lanes,
+// particles, energy, virial) in float-float; FP64 mode: FP64 throughout.
 // ---------------------------------------------------------------------------
 template <bool F32, int NS, class SH>
 struct GradDrain {
@@ -1295,8 +1296,9 @@ static void screen_bound(const gcmc_ctx *ctx, float &r2hi, bool &wrap)
     wrap = (double)ctx->T * ctx->rc > ctx->L;
 }
 
-// Grid size of a neighbourhood kernel: one CTA per cell, at most what stays
-// resident (6 CTAs of 8 warps and ~35 KB per SM) times a few waves.
+// Grid size of a neighbourhood kernel: one CTA per cell, at most 48 per SM, five
+// to ten times what is resident (nine CTAs of k_trial_energy and k_cell_energy,
+// five of k_cell_grad).
 static unsigned nb_blocks(const gcmc_ctx *ctx, int64_t cells)
 {
     const int64_t cap = (int64_t)ctx->num_sms * 6 * 8;

@@ -107,9 +107,10 @@ void micro_free(gcmc_ctx *ctx)
     ctx->mc_valid = false;
 }
 
-// The documented limit on the microcells: 4 bits per microcell and 4 bytes
-// per cell of the cube around a point, beside 1,480 bytes, fit an SM's shared
-// memory.
+// The library's limit on the microcells: 4 bits per microcell and 4 bytes per
+// cell of the cube around a point, with 1,480 bytes more, are at most what a CTA
+// may have of shared memory.  The chain keeps neither there; the limit is the
+// one that callers know.
 static size_t micro_bytes(int64_t ncm, int nax)
 {
     return (size_t)nax * nax * nax * 4 + (size_t)((ncm + 1) / 2 + 15) / 16 * 16 + 1480;
@@ -125,7 +126,7 @@ gcmc_status micro_build(gcmc_ctx *ctx, double edge, int cap_req)
     const int D = 1 + (int)(((uint64_t)(ctx->rcg - 1) * (uint64_t)M) >> 32);
     if (micro_bytes(ncm, std::min(2 * D + 1, M)) > ctx->smem_optin)
         return fail(ctx, GCMC_ERR_INVALID_ARG,
-                    "gcmc_build_microcells: too many microcells for the chain's on-chip counters");
+                    "gcmc_build_microcells: too many microcells (the limit counts 4 bits each and 4 bytes per cell of the cube)");
     SpeciesPrefix p{};
     for (int s = 0; s < ctx->S; ++s) p.first[s + 1] = p.first[s] + ctx->n_host[s];
     for (int s = ctx->S; s < kMaxSpecies; ++s) p.first[s + 1] = p.first[s];

@@ -184,9 +184,11 @@ class Box:
         check(self._lib.gcmc_set_chain_profile(self._h, 1 if on else 0), self._h)
 
     def chain_profile(self) -> dict:
-        """SM cycles of the last chain run by role (zeros unless set_chain_profile was on; evaluations
-        always): evaluated moves waiting for their turn, the checks at the turn, the decision,
-        applying, all of it; waiting for the book, evaluating, evaluations."""
+        """SM cycles of the last chain run, summed over the moves (zeros unless set_chain_profile was
+        on; evaluations always): commit_wait evaluated moves waiting for their turn, commit_valid the
+        checks at the turn (valid_logs, valid_pick its parts; valid_epoch 0), commit_decide the
+        decision, commit_apply applying, commit_total all of it, commit_book passing the turn on;
+        leader_idle waiting for room in the book, team_eval evaluating, evaluations their number."""
         out = np.zeros(12, np.float64)
         check(self._lib.gcmc_chain_profile(self._h, out.ctypes.data_as(C.c_void_p)), self._h)
         keys = ("commit_wait", "commit_valid", "commit_decide", "commit_apply", "commit_total",
