@@ -63,20 +63,18 @@ UNIT = "moves/s"
 FLUSH_BYTES = 256 << 20
 # DRAM bytes (read + write) of one full-size chain launch (64 chains x 10^5
 # moves) from an ncu capture (profiles/k_chain_isotherm_fp32.md), valid for
-# the chain kernel source with this sha256 prefix only (captured with the
-# source 19137a71284994a4, which differs from this one in comments only)
-CHAIN_TRAFFIC = {"sha256_prefix": "fb1ab48a525325ae", "bytes": 19.05e6, "moves": 6.4e6}
+# the chain kernel source with this sha256 prefix only
+CHAIN_TRAFFIC = {"sha256_prefix": "3e167f04a9ddd60c", "bytes": 19.72e6, "moves": 6.4e6}
 # DRAM bytes (read + write, summed over the call's launches) of the timed calls
 # of --kernels-only from one ncu capture (profiles/cell_build_mixture_1m.md),
-# valid for the sources whose joint sha256 has this prefix (the kernels of
-# these calls are those of the captured revision)
+# valid for the sources whose joint sha256 has this prefix
 KERNEL_TRAFFIC = {
-    "cells": {"sources": ("gcmc_cells.cu", "gcmc_device.cuh"), "sha256_prefix": "0943f0587b70112e",
+    "cells": {"sources": ("gcmc_cells.cu", "gcmc_device.cuh"), "sha256_prefix": "1149d08b42cda602",
               "bytes": {"cell_build_mixture_1m": 115.4e6}},
     "energy": {"sources": ("gcmc_energy.cu", "gcmc_stage.cuh", "gcmc_device.cuh"),
-               "sha256_prefix": "770bd8275192054c",
-               "bytes": {"trial_energy_mixture_1m": 152.1e6, "total_energy_mixture_1m": 17.93e6,
-                         "energy_grad_262k": 5.47e6}},
+               "sha256_prefix": "bbbc2de3a29c6a8e",
+               "bytes": {"trial_energy_mixture_1m": 151.7e6, "total_energy_mixture_1m": 17.94e6,
+                         "energy_grad_262k": 5.48e6}},
 }
 DEFAULT_MOVES = {"isotherm": 100_000, "c2": 1_000_000, "c1": 10_000}
 DEFAULT_CPU_MOVES = {"isotherm": 20_000, "c2": 1_000_000, "c1": 10_000}
